@@ -1057,6 +1057,9 @@ size_t api_bwd_workspace(const Geo& g, int N) {
 cudaError_t api_run_boundary(int dt, int N, FwdParams& p, float* states, int emit_all, cudaStream_t s) {
   const Geo& g = p.g;
   cudaError_t e = cudaSuccess;
+  // with the final state alone, only the state after the last full chunk is
+  // used below: the carry leaves the chunk start states unwritten
+  p.carry_last_only = !emit_all && p.yc == nullptr;
   if (g.nc_full > 0) e = launched(launch_chunk_local(dt, N, p, s), s);
   if (e == cudaSuccess) e = launched(launch_chunk_carry(N, p, s), s);
   if (e != cudaSuccess) return e;

@@ -36,6 +36,11 @@ constexpr int kLocalSpan = 32;  // tokens staged per step of the chunk-local sca
 constexpr int kScanSeg = 16;
 
 // REV: the scan runs right to left in time (logical token t is row L-1-t).
+// Bound by the exponentials (one ex2 per token, channel and state) together
+// with the packed FP32 operations around them: 262,144 x 2048 x 16 takes
+// 1245 us, of which the ex2 alone need 853. The staged spans have a
+// compile-time stride, so a token's addresses are immediates (1273 us with a
+// run-time stride and half the unroll).
 template <typename T, int N, bool REV>
 __global__ void __launch_bounds__(kCta) k_chunk_local(const FwdParams p) {
   extern __shared__ __align__(16) unsigned char smem[];
@@ -51,7 +56,7 @@ __global__ void __launch_bounds__(kCta) k_chunk_local(const FwdParams p) {
           dguard(kSiteChunkLocal, ((b * (g.nc + 1) + c) * g.D + dl) * N + N - 1, g.Bt * (g.nc + 1) * g.D * N)))
       return;
   }
-  Stage<T, N, 2, 1, 2, 0, REV> st;
+  Stage<T, N, 2, 1, 2, kLocalSpan, REV> st;
   st.carve(smem, kLocalSpan);
   auto prow = [&](int64_t t) { return b * g.L + (REV ? g.L - 1 - t : t); };  // row of logical token t
   st.td_src[0] = (const T*)p.xc;
@@ -80,7 +85,7 @@ __global__ void __launch_bounds__(kCta) k_chunk_local(const FwdParams p) {
       st.issue((sp + 1) & 1, prow(tbeg + tn), (int)((tc - tn) < kLocalSpan ? (tc - tn) : kLocalSpan), g.D, d0);
     }
     st.complete(sp & 1, ns, sp + 1 < nspan ? 1 : 0);
-#pragma unroll 4
+#pragma unroll 8
     for (int i = 0; i < ns; ++i) {
       const float dt = st.at(1, i);
       scan_state<N>(h, A2, dt, st.at(0, i), st.row(0, i));
@@ -93,42 +98,66 @@ __global__ void __launch_bounds__(kCta) k_chunk_local(const FwdParams p) {
   }
 }
 
+// The carry over chunks is one fused multiply-add per chunk and state, so the
+// kernel is bound by how many bytes it keeps in flight. A CTA of 64 threads
+// owns 64 consecutive (channel, state) elements of one batch row, one per
+// thread, and streams the chunk rows (256 bytes of local end states plus the
+// sums of dt) through a ring of kCarryStages cp.async groups of kCarryRows
+// rows: 12 KB ahead of the chain per CTA. With one load per thread and chunk,
+// eight in flight, 2048 chunks x 32768 elements took 291 us (1.8 TB/s).
+constexpr int kCarryW = 64, kCarryRows = 16, kCarryStages = 4;
 template <int N>
-__global__ void __launch_bounds__(256) k_chunk_carry(const FwdParams p) {
+__global__ void __launch_bounds__(kCarryW) k_chunk_carry(const FwdParams p) {
+  constexpr int CH = kCarryW / N;        // channels of the CTA's elements
+  constexpr int HQ = kCarryW / 4, SQ = CH / 4;  // 16-byte pieces of one row of states, of dt sums
+  __shared__ __align__(16) float hbuf[kCarryStages][kCarryRows][kCarryW];
+  __shared__ __align__(16) float sbuf[kCarryStages][kCarryRows][CH];
   const Geo& g = p.g;
-  const int64_t idx = (int64_t)blockIdx.x * 256 + threadIdx.x;
-  if (idx >= g.Bt * g.D * N) return;
-  const int n = (int)(idx % N);
-  const int64_t d = (idx / N) % g.D, b = idx / ((int64_t)N * g.D);
-  // debug build: the last state slot this thread writes (no barrier follows)
-  if (!dguard(kSiteChunkCarry, ((b * (g.nc + 1) + g.nc_full) * g.D + d) * N + n, g.Bt * (g.nc + 1) * g.D * N)) return;
-  const float A2 = __fmul_rn(p.Af[d * N + n], kLog2e);
-  float H = p.init ? p.init[(b * g.D + d) * N + n] : 0.f;
-  const int64_t hstride = g.D * N;
-  float* hs = p.hst + b * (g.nc + 1) * hstride + d * N + n;
-  const float* sd = p.sdt + b * g.nc * g.D + d;
-  constexpr int U = 8;
-  int c = 0;
-  for (; c + U <= g.nc_full; c += U) {
-    float hl[U], s[U];
-#pragma unroll
-    for (int j = 0; j < U; ++j) {
-      hl[j] = hs[(int64_t)(c + j) * hstride];
-      s[j] = sd[(int64_t)(c + j) * g.D];
+  const int64_t DN = g.D * N, b = blockIdx.y, e0 = (int64_t)blockIdx.x * kCarryW, e = e0 + threadIdx.x;
+  const bool act = e < DN;
+  // debug build: the last state slot the CTA writes
+  if (!dguard(kSiteChunkCarry, (b * (g.nc + 1) + g.nc_full) * DN + (e0 + kCarryW < DN ? e0 + kCarryW : DN) - 1,
+              g.Bt * (g.nc + 1) * DN))
+    return;
+  const float A2 = act ? __fmul_rn(p.Af[e], kLog2e) : 0.f;
+  float H = act && p.init ? p.init[b * DN + e] : 0.f;
+  float* hrow = p.hst + b * (g.nc + 1) * DN + e0;
+  const float* srow = p.sdt + b * g.nc * g.D + e0 / N;
+  const int nst = (g.nc_full + kCarryRows - 1) / kCarryRows;
+  auto issue = [&](int st) {  // rows of stage st; pieces past the row's end or the last chunk are left out
+    if (st < nst) {
+      const int c0 = st * kCarryRows, slot = st % kCarryStages;
+      for (int q = threadIdx.x; q < kCarryRows * HQ; q += kCarryW) {
+        const int r = q / HQ, j = (q - r * HQ) * 4;
+        if (c0 + r < g.nc_full && e0 + j < DN) cp_async16(&hbuf[slot][r][j], hrow + (int64_t)(c0 + r) * DN + j, 16);
+      }
+      for (int q = threadIdx.x; q < kCarryRows * SQ; q += kCarryW) {
+        const int r = q / SQ, j = (q - r * SQ) * 4;
+        if (c0 + r < g.nc_full && e0 / N + j < g.D)
+          cp_async16(&sbuf[slot][r][j], srow + (int64_t)(c0 + r) * g.D + j, 16);
+      }
     }
+    cp_async_commit();
+  };
+  for (int st = 0; st < kCarryStages - 1; ++st) issue(st);
+  for (int st = 0; st < nst; ++st) {
+    asm volatile("cp.async.wait_group %0;\n" ::"n"(kCarryStages - 2) : "memory");
+    __syncthreads();  // stage st is complete, and stage st - 1 is no longer read
+    issue(st + kCarryStages - 1);
+    const int c0 = st * kCarryRows, slot = st % kCarryStages;
+    const int nr = g.nc_full - c0 < kCarryRows ? g.nc_full - c0 : kCarryRows;
 #pragma unroll
-    for (int j = 0; j < U; ++j) {
-      hs[(int64_t)(c + j) * hstride] = H;
-      H = __fmaf_rn(ex2(__fmul_rn(A2, s[j])), H, hl[j]);
+    for (int r = 0; r < kCarryRows; ++r) {
+      if (r >= nr) break;
+      const float hl = hbuf[slot][r][threadIdx.x], sd = sbuf[slot][r][threadIdx.x / N];
+      if (act && !p.carry_last_only) hrow[(int64_t)(c0 + r) * DN + threadIdx.x] = H;
+      H = __fmaf_rn(ex2(__fmul_rn(A2, sd)), H, hl);
     }
   }
-  for (; c < g.nc_full; ++c) {
-    const float hl = hs[(int64_t)c * hstride], s = sd[(int64_t)c * g.D];
-    hs[(int64_t)c * hstride] = H;
-    H = __fmaf_rn(ex2(__fmul_rn(A2, s)), H, hl);
+  if (act) {
+    hrow[(int64_t)g.nc_full * DN + threadIdx.x] = H;
+    dfinite(kSiteChunkCarry, H, b * DN + e);  // debug build: a non-finite cached state
   }
-  hs[(int64_t)g.nc_full * hstride] = H;
-  dfinite(kSiteChunkCarry, H, idx);  // debug build: a non-finite cached state
 }
 
 // MODE 0: all-block forward (clean + noisy). MODE 1: clean scan only (cache
@@ -151,8 +180,12 @@ struct ScanLayout {
 };
 
 // TILED (blocks shorter than kScanSeg): several blocks per staged tile.
+// The stride of the staged tiles is fixed at kScanSeg tokens, so a token's
+// addresses are immediates (16 tokens, 8 x 2048 x 1536 x 16, mode 0: 336 ->
+// 321 us). The clean scans alone fit six CTAs per SM (65,536 x 2048 x 16,
+// mode 1: 545 us with four, 528 with five, 520 with six, 610 with seven).
 template <typename T, typename TO, int N, int MODE, bool TILED>
-__global__ void __launch_bounds__(kCta, 4) k_block_scan(const FwdParams p) {
+__global__ void __launch_bounds__(kCta, MODE == 0 ? 4 : 6) k_block_scan(const FwdParams p) {
   using Ly = ScanLayout<MODE>;
   extern __shared__ __align__(16) unsigned char smem[];
   const Geo& g = p.g;
@@ -170,8 +203,8 @@ __global__ void __launch_bounds__(kCta, 4) k_block_scan(const FwdParams p) {
   // kScanSeg tokens), so the staging and its barriers are paid per tile
   const int TB = TILED ? kScanSeg / Bs : 1;
   constexpr bool kRev = MODE == 2;
-  Stage<T, N, Ly::NTD, Ly::NROW, 2, 0, kRev> st;
-  st.carve(smem, NSEG == 1 ? TB * Bs : SEG);
+  Stage<T, N, Ly::NTD, Ly::NROW, 2, kScanSeg, kRev> st;
+  st.carve(smem, kScanSeg);
   // the row holding logical row x = b L + t (t reversed in time for MODE 2)
   auto prow = [&](int64_t x) { return kRev ? 2 * b * g.L + g.L - 1 - x : x; };
   const bool dbuf = p.stage_bufs == 2 && NSEG == 1;
@@ -504,16 +537,14 @@ template <typename T, typename TO, int N, int MODE>
 int block_scan_bufs_t(int64_t Bs) {
   using Ly = ScanLayout<MODE>;
   if (Bs > kScanSeg) return 1;  // segments are staged when needed
-  const int tile = (int)(kScanSeg / Bs * Bs);
   const size_t extra = Ly::kNoisy ? (size_t)Bs * kCta * sizeof(float) : 0;
-  return 2 * Stage<T, N, Ly::NTD, Ly::NROW, 2>::buf_bytes(tile) + extra <= kDoubleBufferLimit ? 2 : 1;
+  return 2 * Stage<T, N, Ly::NTD, Ly::NROW, 2>::buf_bytes(kScanSeg) + extra <= kDoubleBufferLimit ? 2 : 1;
 }
 
 template <typename T, typename TO, int N, int MODE>
 size_t block_scan_smem_t(int64_t Bs) {
   using Ly = ScanLayout<MODE>;
-  const int seg = Bs < kScanSeg ? (int)(kScanSeg / Bs * Bs) : kScanSeg;  // staged tokens
-  size_t b = Stage<T, N, Ly::NTD, Ly::NROW, 2>::buf_bytes(seg) * block_scan_bufs_t<T, TO, N, MODE>(Bs);
+  size_t b = Stage<T, N, Ly::NTD, Ly::NROW, 2>::buf_bytes(kScanSeg) * block_scan_bufs_t<T, TO, N, MODE>(Bs);
   if (Ly::kNoisy) b += (size_t)Bs * kCta * sizeof(float);
   return b;
 }
@@ -579,10 +610,9 @@ cudaError_t launch_chunk_local(int dt, int N, const FwdParams& p, cudaStream_t s
 }
 
 cudaError_t launch_chunk_carry(int N, const FwdParams& p, cudaStream_t s) {
-  const int64_t total = p.g.Bt * p.g.D * N;
-  if (total == 0) return cudaSuccess;
-  const unsigned blocks = (unsigned)((total + 255) / 256);
-  BDS_DISPATCH_N(N, k_chunk_carry<NN><<<blocks, 256, 0, s>>>(p); return cudaGetLastError();)
+  if (p.g.Bt * p.g.D * N == 0) return cudaSuccess;
+  const dim3 grid((unsigned)((p.g.D * N + kCarryW - 1) / kCarryW), (unsigned)p.g.Bt);
+  BDS_DISPATCH_N(N, k_chunk_carry<NN><<<grid, kCarryW, 0, s>>>(p); return cudaGetLastError();)
 }
 
 cudaError_t launch_block_scan(int dt, int N, int mode, int nchunks, const FwdParams& p, cudaStream_t s) {

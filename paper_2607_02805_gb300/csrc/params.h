@@ -37,6 +37,7 @@ struct FwdParams {
   const float* seed;   // active block: [Bt][D][N]
   int c_begin;         // first chunk handled by a block-scan launch
   int stage_bufs;      // block scan: 2 = copy the next block while computing, 1 = synchronous
+  int carry_last_only; // chunk carry: only the state after the last full chunk is read afterwards
   int rev;             // chunk-local scan: right to left in time (with block-scan mode 2)
   // active block with adaptive layer norm: per batch row shift, scale, gate
   // [Bt][D] and per token (mean, 1/sqrt(var + eps)) of the block's input
