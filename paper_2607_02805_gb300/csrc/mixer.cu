@@ -22,7 +22,7 @@ namespace bds {
 namespace {
 
 constexpr int kW = 4;           // convolution width
-constexpr int kParSplit = 256;  // token slices of the parameter-gradient reduction
+constexpr int kParSplit = 256;  // most token slices of the parameter-gradient reduction
 
 // The logistic function and softplus on the fast hardware paths (__expf,
 // __logf, __fdividef): relative errors of order 1e-6, far inside the
@@ -55,28 +55,6 @@ __device__ __forceinline__ float raw_c(const MixIn<T>& a, int64_t b, int64_t u, 
   if (u >= 0) return cvt(a.xr_c[(b * a.L + u) * a.D + d]);
   return a.conv_init != nullptr ? a.conv_init[(b * (kW - 1) + (kW - 1) + u) * a.D + d] : 0.f;
 }
-// Raw input seen by a noisy token of the block starting at k0, at position u:
-// the noisy stream inside the block, the clean stream before it.
-template <typename T>
-__device__ __forceinline__ float raw_n(const MixIn<T>& a, int64_t b, int64_t u, int64_t k0, int64_t d) {
-  return u >= k0 ? cvt(a.xr_n[(b * a.L + u) * a.D + d]) : raw_c(a, b, u, d);
-}
-template <typename T>
-__device__ __forceinline__ float pre_c(const MixIn<T>& a, int64_t b, int64_t t, int64_t d) {
-  float pre = a.cb[d];
-#pragma unroll
-  for (int j = 0; j < kW; ++j) pre = __fmaf_rn(a.w[d * kW + j], raw_c(a, b, t - (kW - 1) + j, d), pre);
-  return pre;
-}
-template <typename T>
-__device__ __forceinline__ float pre_n(const MixIn<T>& a, int64_t b, int64_t t, int64_t d) {
-  const int64_t k0 = t - t % a.Bs;
-  float pre = a.cb[d];
-#pragma unroll
-  for (int j = 0; j < kW; ++j) pre = __fmaf_rn(a.w[d * kW + j], raw_n(a, b, t - (kW - 1) + j, k0, d), pre);
-  return pre;
-}
-
 // Vector access: V = 16 / sizeof(T) consecutive channels per thread (8 for
 // bf16, 4 for fp32; d_inner is a multiple of V), so every token-by-channel
 // load is 16 bytes per thread.
@@ -129,172 +107,386 @@ __device__ __forceinline__ void stv(bf16* p, const float (&v)[V]) {
   }
 }
 
-// Raw inputs of window tap j (position u) for V channels from d: the clean
-// stream, or the initial convolution state before token 0. u is the same for
-// the whole CTA (one token row per CTA), so the branches are uniform.
-template <typename T, int V>
-__device__ __forceinline__ void raw_cv(const MixIn<T>& a, int64_t b, int64_t u, int64_t d, float (&r)[V]) {
-  if (u >= 0) {
-    ld16(a.xr_c + (b * a.L + u) * a.D + d, r);
-  } else if (a.conv_init != nullptr) {
-    ldf<V>(a.conv_init + (b * (kW - 1) + (kW - 1) + u) * a.D + d, r);
+// Q = 2 or 4 consecutive channels of one row; d_inner is a multiple of 4, so
+// the rows of Q channels are aligned to the access.
+template <int Q>
+__device__ __forceinline__ void ldq(const float* p, float (&v)[Q]) {
+  if (Q == 4) {
+    const float4 u = *reinterpret_cast<const float4*>(p);
+    v[0] = u.x, v[1] = u.y, v[Q - 2] = u.z, v[Q - 1] = u.w;
   } else {
-#pragma unroll
-    for (int v = 0; v < V; ++v) r[v] = 0.f;
+    const float2 u = *reinterpret_cast<const float2*>(p);
+    v[0] = u.x, v[1] = u.y;
   }
 }
-// The same for a noisy token of the block starting at k0: the noisy stream
-// inside the block, the clean one (or the initial state) before it.
-template <typename T, int V>
-__device__ __forceinline__ void raw_nv(const MixIn<T>& a, int64_t b, int64_t u, int64_t k0, int64_t d, float (&r)[V]) {
-  if (u >= k0)
-    ld16(a.xr_n + (b * a.L + u) * a.D + d, r);
+template <int Q>
+__device__ __forceinline__ void ldq(const bf16* p, float (&v)[Q]) {
+  uint32_t u[Q / 2];
+  if (Q == 4)
+    *reinterpret_cast<uint2*>(u) = *reinterpret_cast<const uint2*>(p);
   else
-    raw_cv<T, V>(a, b, u, d, r);
+    u[0] = *reinterpret_cast<const uint32_t*>(p);
+#pragma unroll
+  for (int e = 0; e < Q / 2; ++e) {
+    v[2 * e] = __uint_as_float(u[e] << 16);
+    v[2 * e + 1] = __uint_as_float(u[e] & 0xffff0000u);
+  }
 }
-// Scan inputs in fp32: x = SiLU(conv), dt = softplus(dt_raw + bias), for the
-// clean stream (if x_c) and the noisy stream (if x_n).
-// Grid of the token-by-channel kernels: one CTA row per token (blockIdx.x,
-// batch row b = token / L), 256 channels per CTA (blockIdx.y); no per-element
-// division.
+template <int Q>
+__device__ __forceinline__ void stq(float* p, const float (&v)[Q]) {
+  if (Q == 4)
+    *reinterpret_cast<float4*>(p) = make_float4(v[0], v[1], v[Q - 2], v[Q - 1]);
+  else
+    *reinterpret_cast<float2*>(p) = make_float2(v[0], v[1]);
+}
+template <int Q>
+__device__ __forceinline__ void stq(bf16* p, const float (&v)[Q]) {
+#pragma unroll
+  for (int e = 0; e < Q / 2; ++e)
+    reinterpret_cast<__nv_bfloat162*>(p)[e] = __floats2bfloat162_rn(v[2 * e], v[2 * e + 1]);
+}
+template <int Q>
+__device__ __forceinline__ void zeroq(float (&v)[Q]) {
+#pragma unroll
+  for (int e = 0; e < Q; ++e) v[e] = 0.f;
+}
+
+// Raw clean inputs at position u of batch row b for Q channels from d: the
+// clean stream, the initial convolution state before token 0, zero past the
+// end (or without a clean stream, where no window reads them).
+template <typename T, int Q>
+__device__ __forceinline__ void raw_cq(const MixIn<T>& a, int64_t b, int u, int64_t d, float (&r)[Q]) {
+  if (u >= 0 && u < a.L && a.xr_c != nullptr)
+    ldq<Q>(a.xr_c + (b * a.L + u) * a.D + d, r);
+  else if (u < 0 && a.conv_init != nullptr)
+    ldq<Q>(a.conv_init + (b * (kW - 1) + (kW - 1) + u) * a.D + d, r);
+  else
+    zeroq<Q>(r);
+}
+// The noisy stream's raw inputs at u, zero outside the stream.
+template <typename T, int Q>
+__device__ __forceinline__ void raw_nq(const MixIn<T>& a, int64_t b, int u, int64_t d, float (&r)[Q]) {
+  if (u >= 0 && u < a.L)
+    ldq<Q>(a.xr_n + (b * a.L + u) * a.D + d, r);
+  else
+    zeroq<Q>(r);
+}
+// Positions fit 32 bits (the checks on dims bound len by 65535 chunks of at
+// most 256 tokens), so block offsets are 32-bit remainders.
 template <typename T>
-__global__ void __launch_bounds__(256) k_mix_prep(const MixIn<T> a, float* x_c, float* dt_c, float* x_n, float* dt_f,
-                                                  float* dt_r) {
-  const int64_t d = (int64_t)blockIdx.y * 256 + threadIdx.x;
-  if (d >= a.D) return;
-  const int64_t bt = blockIdx.x, b = bt / a.L, t = bt - b * a.L, i = bt * a.D + d;
-  if (x_c != nullptr) {
-    x_c[i] = silu(pre_c(a, b, t, d));
-    dt_c[i] = softplus(__fadd_rn(cvt(a.dtr_c[i]), a.bias_f[d]));
-  }
-  if (x_n != nullptr) {
-    x_n[i] = silu(pre_n(a, b, t, d));
-    dt_f[i] = softplus(__fadd_rn(cvt(a.dtr_f[i]), a.bias_f[d]));
-    dt_r[i] = softplus(__fadd_rn(cvt(a.dtr_r[i]), a.bias_r[d]));
-  }
+__device__ __forceinline__ int block_off(const MixIn<T>& a, int t) {
+  return (int)((uint32_t)t % (uint32_t)a.Bs);
 }
 
-// Backward through SiLU and softplus, in place on the scan's fp32 gradients:
-// gx <- gx * SiLU'(pre), gdt <- gdt * sigmoid(dt_raw + bias); the step-size
-// gradients also go out in the output type.
-template <typename T, typename TO>
-__global__ void __launch_bounds__(256) k_mix_dpre(const MixIn<T> a, float* gx_c, float* gdt_c, float* gx_n,
-                                                  float* gdt_f, float* gdt_r, TO* ddtr_c, TO* ddtr_f, TO* ddtr_r) {
-  const int64_t d = (int64_t)blockIdx.y * 256 + threadIdx.x;
-  if (d >= a.D) return;
-  const int64_t bt = blockIdx.x, b = bt / a.L, t = bt - b * a.L, i = bt * a.D + d;
-  gx_c[i] = __fmul_rn(gx_c[i], dsilu(pre_c(a, b, t, d)));
-  gx_n[i] = __fmul_rn(gx_n[i], dsilu(pre_n(a, b, t, d)));
-  const float vc = __fmul_rn(gdt_c[i], sigm(__fadd_rn(cvt(a.dtr_c[i]), a.bias_f[d])));
-  const float vf = __fmul_rn(gdt_f[i], sigm(__fadd_rn(cvt(a.dtr_f[i]), a.bias_f[d])));
-  const float vr = __fmul_rn(gdt_r[i], sigm(__fadd_rn(cvt(a.dtr_r[i]), a.bias_r[d])));
-  gdt_c[i] = vc;
-  gdt_f[i] = vf;
-  gdt_r[i] = vr;
-  ddtr_c[i] = to_out<TO>(vc);
-  ddtr_f[i] = to_out<TO>(vf);
-  ddtr_r[i] = to_out<TO>(vr);
+// The token sweeps below read their rows through a ring in shared memory: each
+// thread copies (cp.async) the Q channels it will use itself, kAhead tokens
+// before it uses them, so no barrier is needed and enough bytes are in flight
+// without holding them in registers.
+template <int BYTES>
+__device__ __forceinline__ void copy_async(void* smem, const void* gmem) {
+  const uint32_t s = (uint32_t)__cvta_generic_to_shared(smem);
+  asm volatile("cp.async.ca.shared.global [%0], [%1], %2;\n" ::"r"(s), "l"(gmem), "n"(BYTES) : "memory");
+}
+template <int PENDING>
+__device__ __forceinline__ void wait_async() {
+  asm volatile("cp.async.wait_group %0;\n" ::"n"(PENDING) : "memory");
 }
 
-// Gradients of the raw inputs from the pre-activation gradients (the
-// convolution's transpose): raw position u feeds tap j of token u + 3 - j; a
-// noisy token's taps before its block feed the clean stream. V channels per
-// thread (V = 16 / sizeof(TI), TI the input type).
-template <typename TO, int V>
-__global__ void __launch_bounds__(256) k_mix_dxr(int64_t Bt, int64_t L, int64_t D, int64_t Bs, const float* w,
-                                                 const float* gp_c, const float* gp_n, TO* dxr_c, TO* dxr_n) {
-  const int64_t d = ((int64_t)blockIdx.y * 256 + threadIdx.x) * V;
-  if (d >= D) return;
-  const int64_t bt = blockIdx.x, b = bt / L, u = bt - b * L, i = bt * D + d;
-  float wv[kW * V], ac[V], an[V];
-  ldf<kW * V>(w + d * kW, wv);
+// Scan inputs in fp32: x = SiLU(conv), dt = softplus(dt_raw + bias), for the
+// clean stream (if x_c) and the noisy stream (if x_n). A thread sweeps Ls
+// consecutive tokens of 4 channels with the convolution window in registers
+// (slot q holds the last row whose position is q modulo 4 of the sweep).
+// Bound by memory: 8 x 2048 x 1536 bf16 moves 755 MB; one element per thread,
+// each with its own window loads and two 64-bit divisions, took 391 us.
+constexpr int kPrepCta = 128, kPrepRing = 8, kPrepAhead = kPrepRing - 1;
+template <typename T>
+constexpr size_t prep_smem() {
+  return (size_t)kPrepRing * 5 * kPrepCta * 4 * sizeof(T);
+}
+template <typename T>
+__global__ void __launch_bounds__(kPrepCta) k_mix_prep(const MixIn<T> a, float* x_c, float* dt_c, float* x_n,
+                                                       float* dt_f, float* dt_r, int Ls) {
+  extern __shared__ __align__(16) unsigned char smem[];
+  constexpr int Q = 4, S = 4, W1 = kW - 1;
+  const int64_t d = ((int64_t)blockIdx.y * blockDim.x + threadIdx.x) * Q, b = blockIdx.z;
+  const int tb = (int)(blockIdx.x * blockDim.y + threadIdx.y) * Ls, L = (int)a.L, Bs = (int)a.Bs;
+  if (d >= a.D || tb >= L) return;
+  const int te = tb + Ls < L ? tb + Ls : L;
+  T* ring = reinterpret_cast<T*>(smem) + (threadIdx.y * blockDim.x + threadIdx.x) * Q;  // [slot][tensor][thread]
+  auto slot = [&](int t, int k) { return ring + ((t & (kPrepRing - 1)) * 5 + k) * (kPrepCta * Q); };
+  constexpr int BYTES = Q * (int)sizeof(T);
+  auto issue = [&](int t) {
+    if (t < te) {
+      const int64_t i = (b * a.L + t) * a.D + d;
+      if (a.xr_c != nullptr) {
+        copy_async<BYTES>(slot(t, 0), a.xr_c + i);
+        if (x_c != nullptr) copy_async<BYTES>(slot(t, 1), a.dtr_c + i);
+      }
+      if (x_n != nullptr) {
+        copy_async<BYTES>(slot(t, 2), a.xr_n + i);
+        copy_async<BYTES>(slot(t, 3), a.dtr_f + i);
+        copy_async<BYTES>(slot(t, 4), a.dtr_r + i);
+      }
+    }
+    cp_async_commit();
+  };
 #pragma unroll
-  for (int v = 0; v < V; ++v) ac[v] = an[v] = 0.f;
+  for (int q = 0; q < kPrepAhead; ++q) issue(tb + q);
+  float c[S][Q], n[S][Q];
 #pragma unroll
-  for (int j = 0; j < kW; ++j) {
-    const int64_t t = u + (kW - 1) - j;
-    if (t >= L) continue;
-    const int64_t o = (b * L + t) * D + d;
-    float pc[V], pn[V];
-    ldf<V>(gp_c + o, pc);
-    ldf<V>(gp_n + o, pn);
-    const bool inside = u >= t - t % Bs;  // the same block as the consuming noisy token
+  for (int q = 0; q < S; ++q) {
+    zeroq<Q>(c[q]);
+    zeroq<Q>(n[q]);
+  }
 #pragma unroll
-    for (int v = 0; v < V; ++v) {
-      const float wj = wv[v * kW + j];
-      ac[v] = __fmaf_rn(wj, pc[v], ac[v]);
-      if (inside)
-        an[v] = __fmaf_rn(wj, pn[v], an[v]);
-      else
-        ac[v] = __fmaf_rn(wj, pn[v], ac[v]);
+  for (int q = 1; q < S; ++q) {
+    raw_cq<T, Q>(a, b, tb - S + q, d, c[q]);
+    if (x_n != nullptr) raw_nq<T, Q>(a, b, tb - S + q, d, n[q]);
+  }
+  float w[kW * Q], cb[Q], bf[Q], br[Q];
+  ldf<kW * Q>(a.w + d * kW, w);
+  ldq<Q>(a.cb + d, cb);
+  ldq<Q>(a.bias_f + d, bf);
+  ldq<Q>(a.bias_r + d, br);
+  int off = block_off(a, tb);
+  for (int t0 = tb; t0 < te; t0 += S) {
+#pragma unroll
+    for (int q = 0; q < S; ++q) {
+      const int t = t0 + q;
+      if (t >= te) break;
+      issue(t + kPrepAhead);
+      wait_async<kPrepAhead>();
+      const int64_t i = (b * a.L + t) * a.D + d;
+      float o[Q], v[Q];
+      if (a.xr_c != nullptr) ldq<Q>(slot(t, 0), c[q]);
+      if (x_c != nullptr) {
+        ldq<Q>(slot(t, 1), v);
+#pragma unroll
+        for (int e = 0; e < Q; ++e) {
+          float pre = cb[e];
+#pragma unroll
+          for (int j = 0; j < kW; ++j) pre = __fmaf_rn(w[e * kW + j], c[(q + 1 + j) % S][e], pre);
+          o[e] = silu(pre);
+          v[e] = softplus(__fadd_rn(v[e], bf[e]));
+        }
+        stq<Q>(x_c + i, o);
+        stq<Q>(dt_c + i, v);
+      }
+      if (x_n != nullptr) {
+        ldq<Q>(slot(t, 2), n[q]);
+        ldq<Q>(slot(t, 3), v);
+#pragma unroll
+        for (int e = 0; e < Q; ++e) {
+          float pre = cb[e];
+#pragma unroll
+          for (int j = 0; j < kW; ++j)  // tap j is at t - 3 + j: inside the block from its first token on
+            pre = __fmaf_rn(w[e * kW + j], off >= W1 - j ? n[(q + 1 + j) % S][e] : c[(q + 1 + j) % S][e], pre);
+          o[e] = silu(pre);
+          v[e] = softplus(__fadd_rn(v[e], bf[e]));
+        }
+        stq<Q>(x_n + i, o);
+        stq<Q>(dt_f + i, v);
+        ldq<Q>(slot(t, 4), v);
+#pragma unroll
+        for (int e = 0; e < Q; ++e) v[e] = softplus(__fadd_rn(v[e], br[e]));
+        stq<Q>(dt_r + i, v);
+      }
+      off = off + 1 == Bs ? 0 : off + 1;
     }
   }
-  stv<V>(dxr_c + i, ac);
-  stv<V>(dxr_n + i, an);
 }
 
-// Partial sums of the parameter gradients over a slice of the token rows:
-// part[slice][v][d] for v = tap 0..3, conv bias, dt_bias_f, dt_bias_r; V
-// channels per thread.
+// The backward from the scan's fp32 gradients to the raw inputs, in one pass:
+// through SiLU (gp = gx SiLU'(pre)), softplus (the step-size gradients), the
+// convolution's transpose (raw position u feeds tap j of token u + 3 - j; a
+// noisy token's taps before its block feed the clean stream) and the partial
+// sums of the parameter gradients, part[slice][v][d] for v = tap 0..3, conv
+// bias, dt_bias_f, dt_bias_r. gp exists in registers only.
+// A warp sweeps segments of Ls consecutive tokens (and the three after each,
+// whose gp the transpose needs) for 64 channels, with windows of the last four
+// raw rows and gp rows (slot q: position q modulo 4 of the sweep); the eight
+// warps of a CTA share the channels and leave one slice of sums.
+// Bound by memory: 8 x 2048 x 1536 bf16 moves 1.0 GB; as three kernels that
+// exchanged gp through memory the same work took 795 us.
+constexpr int kBwdGroups = 8, kBwdRing = 4, kBwdAhead = kBwdRing - 1;  // warps per CTA; ring of token rows
 template <typename T>
-__global__ void __launch_bounds__(128) k_mix_par_part(const MixIn<T> a, const float* gp_c, const float* gp_n,
-                                                      const float* gdt_c, const float* gdt_f, const float* gdt_r,
-                                                      float* part) {
-  constexpr int V = Vec<T>::V;
-  const int64_t d = ((int64_t)blockIdx.x * 128 + threadIdx.x) * V;
-  const int slice = blockIdx.y;
-  if (d >= a.D) return;
-  float s[kW + 3][V];
+constexpr size_t mix_bwd_smem() {
+  return (size_t)kBwdRing * 5 * 32 * kBwdGroups * 2 * (sizeof(T) + 4);
+}
+template <typename T, typename TO>
+__global__ void __launch_bounds__(32 * kBwdGroups, 2)
+    k_mix_bwd(const MixIn<T> a, const float* gx_c, const float* gdt_c, const float* gx_n, const float* gdt_f,
+              const float* gdt_r, TO* dxr_c, TO* ddtr_c, TO* dxr_n, TO* ddtr_f, TO* ddtr_r, int Ls, int nseg,
+              float* part) {
+  extern __shared__ __align__(16) unsigned char smem[];
+  constexpr int Q = 2, W1 = kW - 1, S = 4, TH = 32 * kBwdGroups;
+  __shared__ float red[kBwdGroups][kW + 3][32 * Q];
+  const int lane = threadIdx.x, grp = threadIdx.y;
+  const int64_t d = ((int64_t)blockIdx.y * 32 + lane) * Q;
+  const int L = (int)a.L, Bs = (int)a.Bs;
+  // ring[slot][tensor][thread]: fp32 gx_c, gx_n, gdt_c, gdt_f, gdt_r, then xr_c, xr_n, dtr_c, dtr_f, dtr_r
+  float* fring = reinterpret_cast<float*>(smem) + (grp * 32 + lane) * Q;
+  T* tring = reinterpret_cast<T*>(smem + (size_t)kBwdRing * 5 * TH * Q * 4) + (grp * 32 + lane) * Q;
+  auto fslot = [&](int t, int k) { return fring + ((t & (kBwdRing - 1)) * 5 + k) * (TH * Q); };
+  auto tslot = [&](int t, int k) { return tring + ((t & (kBwdRing - 1)) * 5 + k) * (TH * Q); };
+  float s[kW + 3][Q];
+#pragma unroll
+  for (int q = 0; q < kW + 3; ++q) zeroq<Q>(s[q]);
+  if (d < a.D) {
+    float w[kW * Q], cb[Q], bf[Q], br[Q];
+    ldf<kW * Q>(a.w + d * kW, w);
+    ldq<Q>(a.cb + d, cb);
+    ldq<Q>(a.bias_f + d, bf);
+    ldq<Q>(a.bias_r + d, br);
+    const int64_t segs = a.Bt * nseg;
+    for (int64_t seg = (int64_t)blockIdx.x * kBwdGroups + grp; seg < segs; seg += (int64_t)gridDim.x * kBwdGroups) {
+      const int64_t b = seg / nseg;
+      const int tb = (int)(seg - b * nseg) * Ls, te = tb + Ls < L ? tb + Ls : L;
+      const int th = te + W1 < L ? te + W1 : L;  // tokens whose gp is needed
+      auto issue = [&](int t) {
+        if (t < th) {
+          const int64_t i = (b * a.L + t) * a.D + d;
+          copy_async<8>(fslot(t, 0), gx_c + i);
+          copy_async<8>(fslot(t, 1), gx_n + i);
+          copy_async<2 * sizeof(T)>(tslot(t, 0), a.xr_c + i);
+          copy_async<2 * sizeof(T)>(tslot(t, 1), a.xr_n + i);
+          if (t < te) {
+            copy_async<8>(fslot(t, 2), gdt_c + i);
+            copy_async<8>(fslot(t, 3), gdt_f + i);
+            copy_async<8>(fslot(t, 4), gdt_r + i);
+            copy_async<2 * sizeof(T)>(tslot(t, 2), a.dtr_c + i);
+            copy_async<2 * sizeof(T)>(tslot(t, 3), a.dtr_f + i);
+            copy_async<2 * sizeof(T)>(tslot(t, 4), a.dtr_r + i);
+          }
+        }
+        cp_async_commit();
+      };
+#pragma unroll
+      for (int q = 0; q < kBwdAhead; ++q) issue(tb + q);
+      float c[S][Q], n[S][Q], pc[S][Q], pn[S][Q];
+      int off[S];  // the token's offset in its block
+#pragma unroll
+      for (int q = 0; q < S; ++q) {
+        zeroq<Q>(c[q]);
+        zeroq<Q>(n[q]);
+        zeroq<Q>(pc[q]);
+        zeroq<Q>(pn[q]);
+        off[q] = 0;
+      }
+#pragma unroll
+      for (int q = 1; q < S; ++q) {
+        raw_cq<T, Q>(a, b, tb - S + q, d, c[q]);
+        raw_nq<T, Q>(a, b, tb - S + q, d, n[q]);
+      }
+      int o = block_off(a, tb);
+      for (int t0 = tb; t0 < te + W1; t0 += S) {
+#pragma unroll
+        for (int q = 0; q < S; ++q) {
+          const int t = t0 + q;
+          if (t >= te + W1) break;
+          issue(t + kBwdAhead);
+          wait_async<kBwdAhead>();
+          off[q] = o;
+          o = o + 1 == Bs ? 0 : o + 1;
+          if (t < L) {
+            ldq<Q>(tslot(t, 0), c[q]);
+            ldq<Q>(tslot(t, 1), n[q]);
+            ldq<Q>(fslot(t, 0), pc[q]);
+            ldq<Q>(fslot(t, 1), pn[q]);
+#pragma unroll
+            for (int e = 0; e < Q; ++e) {
+              float rc[kW], rn[kW], prc = cb[e], prn = cb[e];
+#pragma unroll
+              for (int j = 0; j < kW; ++j) {
+                rc[j] = c[(q + 1 + j) % S][e];
+                rn[j] = off[q] >= W1 - j ? n[(q + 1 + j) % S][e] : rc[j];
+                prc = __fmaf_rn(w[e * kW + j], rc[j], prc);
+                prn = __fmaf_rn(w[e * kW + j], rn[j], prn);
+              }
+              pc[q][e] = __fmul_rn(pc[q][e], dsilu(prc));
+              pn[q][e] = __fmul_rn(pn[q][e], dsilu(prn));
+              if (t < te) {
+#pragma unroll
+                for (int j = 0; j < kW; ++j) s[j][e] = __fmaf_rn(pn[q][e], rn[j], __fmaf_rn(pc[q][e], rc[j], s[j][e]));
+                s[kW][e] = __fadd_rn(s[kW][e], __fadd_rn(pc[q][e], pn[q][e]));
+              }
+            }
+            if (t < te) {
+              const int64_t i = (b * a.L + t) * a.D + d;
+              float v1[Q], v2[Q], v3[Q], r1[Q], r2[Q], r3[Q];
+              ldq<Q>(fslot(t, 2), v1);
+              ldq<Q>(fslot(t, 3), v2);
+              ldq<Q>(fslot(t, 4), v3);
+              ldq<Q>(tslot(t, 2), r1);
+              ldq<Q>(tslot(t, 3), r2);
+              ldq<Q>(tslot(t, 4), r3);
+#pragma unroll
+              for (int e = 0; e < Q; ++e) {
+                v1[e] = __fmul_rn(v1[e], sigm(__fadd_rn(r1[e], bf[e])));
+                v2[e] = __fmul_rn(v2[e], sigm(__fadd_rn(r2[e], bf[e])));
+                v3[e] = __fmul_rn(v3[e], sigm(__fadd_rn(r3[e], br[e])));
+                s[kW + 1][e] = __fadd_rn(s[kW + 1][e], __fadd_rn(v1[e], v2[e]));
+                s[kW + 2][e] = __fadd_rn(s[kW + 2][e], v3[e]);
+              }
+              stq<Q>(ddtr_c + i, v1);
+              stq<Q>(ddtr_f + i, v2);
+              stq<Q>(ddtr_r + i, v3);
+            }
+          }
+          // gp of tokens u ... u + 3 is complete: the raw gradients of u = t - 3
+          const int u = t - W1;
+          if (u >= tb) {
+            float ac[Q], an[Q];
+            zeroq<Q>(ac);
+            zeroq<Q>(an);
+#pragma unroll
+            for (int j = 0; j < kW; ++j) {
+              if (t - j >= L) continue;
+              const int k = (q + S - j) % S;
+              const bool inside = off[k] >= W1 - j;  // the same block as the consuming noisy token
+#pragma unroll
+              for (int e = 0; e < Q; ++e) {
+                const float wj = w[e * kW + j];
+                ac[e] = __fmaf_rn(wj, pc[k][e], ac[e]);
+                if (inside)
+                  an[e] = __fmaf_rn(wj, pn[k][e], an[e]);
+                else
+                  ac[e] = __fmaf_rn(wj, pn[k][e], ac[e]);
+              }
+            }
+            const int64_t i = (b * a.L + u) * a.D + d;
+            stq<Q>(dxr_c + i, ac);
+            stq<Q>(dxr_n + i, an);
+          }
+        }
+      }
+    }
+  }
 #pragma unroll
   for (int q = 0; q < kW + 3; ++q)
 #pragma unroll
-    for (int v = 0; v < V; ++v) s[q][v] = 0.f;
-  int64_t b = slice / a.L, t = slice - b * a.L;  // batch row and token of `row`, stepped without division
-  for (int64_t row = slice; row < a.Bt * a.L; row += kParSplit) {
-    const int64_t o = row * a.D + d, k0 = t - t % a.Bs;
-    float pc[V], pn[V], g1[V], g2[V], g3[V];
-    ldf<V>(gp_c + o, pc);
-    ldf<V>(gp_n + o, pn);
-    ldf<V>(gdt_c + o, g1);
-    ldf<V>(gdt_f + o, g2);
-    ldf<V>(gdt_r + o, g3);
+    for (int e = 0; e < Q; ++e) red[grp][q][lane * Q + e] = s[q][e];
+  __syncthreads();
+  for (int i = grp * 32 + lane; i < (kW + 3) * 32 * Q; i += TH) {
+    const int q = i / (32 * Q), k = i - q * (32 * Q);
+    const int64_t dk = (int64_t)blockIdx.y * 32 * Q + k;
+    float v = red[0][q][k];
 #pragma unroll
-    for (int j = 0; j < kW; ++j) {
-      const int64_t u = t - (kW - 1) + j;
-      float rc[V], rn[V];
-      raw_cv<T, V>(a, b, u, d, rc);
-      raw_nv<T, V>(a, b, u, k0, d, rn);
-#pragma unroll
-      for (int v = 0; v < V; ++v) {
-        s[j][v] = __fmaf_rn(pc[v], rc[v], s[j][v]);
-        s[j][v] = __fmaf_rn(pn[v], rn[v], s[j][v]);
-      }
-    }
-#pragma unroll
-    for (int v = 0; v < V; ++v) {
-      s[kW][v] = __fadd_rn(s[kW][v], __fadd_rn(pc[v], pn[v]));
-      s[kW + 1][v] = __fadd_rn(s[kW + 1][v], __fadd_rn(g1[v], g2[v]));
-      s[kW + 2][v] = __fadd_rn(s[kW + 2][v], g3[v]);
-    }
-    t += kParSplit;
-    while (t >= a.L) {
-      t -= a.L;
-      ++b;
-    }
+    for (int r = 1; r < kBwdGroups; ++r) v = __fadd_rn(v, red[r][q][k]);
+    if (dk < a.D) part[((int64_t)blockIdx.x * (kW + 3) + q) * a.D + dk] = v;
   }
-#pragma unroll
-  for (int q = 0; q < kW + 3; ++q) stv<V>(part + ((int64_t)slice * (kW + 3) + q) * a.D + d, s[q]);
 }
 
 // The slices summed in order: dconv_w [D][4], dconv_b, ddt_bias_f, ddt_bias_r [D].
-__global__ void __launch_bounds__(256) k_mix_par_red(int64_t D, const float* part, float* dw, float* db, float* dbf,
-                                                     float* dbr) {
+__global__ void __launch_bounds__(256) k_mix_par_red(int64_t D, int slices, const float* part, float* dw, float* db,
+                                                     float* dbf, float* dbr) {
   const int64_t i = (int64_t)blockIdx.x * 256 + threadIdx.x;
   if (i >= D * (kW + 3)) return;
   const int v = (int)(i / D);
   const int64_t d = i % D;
   float s = 0.f;
-  for (int sl = 0; sl < kParSplit; ++sl) s = __fadd_rn(s, part[((int64_t)sl * (kW + 3) + v) * D + d]);
+#pragma unroll 16
+  for (int sl = 0; sl < slices; ++sl) s = __fadd_rn(s, part[((int64_t)sl * (kW + 3) + v) * D + d]);
   if (v < kW)
     dw[d * kW + v] = s;
   else if (v == kW)
@@ -345,11 +537,20 @@ __global__ void __launch_bounds__(256) k_mix_gate_bwd(int64_t n, const float* y,
   stv<V>(dz + i, c);
 }
 
-// Element type conversion (B, C to fp32 for the scan; their gradients back).
+// Element type conversion of up to six tensors of n elements (B, C to fp32
+// for the scan; their gradients back), one per blockIdx.y; four elements per
+// thread (rows of d_state are multiples of 4).
+struct CvtSet {
+  const void* src[6];
+  void* dst[6];
+};
 template <typename TI, typename TO>
-__global__ void __launch_bounds__(256) k_mix_cvt(int64_t n, const TI* src, TO* dst) {
-  const int64_t i = (int64_t)blockIdx.x * 256 + threadIdx.x;
-  if (i < n) dst[i] = to_out<TO>(cvt(src[i]));
+__global__ void __launch_bounds__(256) k_mix_cvt(int64_t n, const __grid_constant__ CvtSet c) {
+  const int64_t i = ((int64_t)blockIdx.x * 256 + threadIdx.x) * 4;
+  if (i >= n) return;
+  float v[4];
+  ldq<4>((const TI*)c.src[blockIdx.y] + i, v);
+  stq<4>((TO*)c.dst[blockIdx.y] + i, v);
 }
 
 // Convolution part of the cache: the raw clean inputs of the three tokens
@@ -435,11 +636,6 @@ int check_mparams(const bdscan_mixer_params* m, const char* fn) {
 }
 
 unsigned blocks_of(int64_t n) { return (unsigned)((n + 255) / 256); }
-// one CTA row per token, 256 threads of V channels per CTA
-dim3 rows_grid(const Geo& g, int V) {
-  const int64_t span = 256 * (int64_t)V;
-  return dim3((unsigned)(g.Bt * g.L), (unsigned)((g.D + span - 1) / span));
-}
 template <typename T>
 unsigned vec_blocks(int64_t n) {
   constexpr int64_t span = 256 * Vec<T>::V;
@@ -472,15 +668,44 @@ MixIn<T> mix_in(const Geo& g, const bdscan_clean* c, const bdscan_noisy* n, cons
   return a;
 }
 
+template <typename TI, typename TO>
+cudaError_t cvt_all(const CvtSet& c, int count, int64_t n, cudaStream_t s) {
+  k_mix_cvt<TI, TO><<<dim3((unsigned)((n / 4 + 255) / 256), (unsigned)count), 256, 0, s>>>(n, c);
+  return api_launched(cudaGetLastError(), s);
+}
 // B and C of the given streams converted to fp32 into the workspace slots.
 template <typename T>
 cudaError_t to_f32(const void* const* src, const size_t* slot, int count, char* ws, int64_t n, cudaStream_t s) {
-  cudaError_t e = cudaSuccess;
-  for (int i = 0; i < count && e == cudaSuccess; ++i) {
-    k_mix_cvt<T, float><<<blocks_of(n), 256, 0, s>>>(n, (const T*)src[i], (float*)(ws + slot[i]));
-    e = api_launched(cudaGetLastError(), s);
+  CvtSet c;
+  memset(&c, 0, sizeof(c));
+  for (int i = 0; i < count; ++i) {
+    c.src[i] = src[i];
+    c.dst[i] = ws + slot[i];
   }
-  return e;
+  return cvt_all<T, float>(c, count, n, s);
+}
+
+// Tokens per sweep of the elementwise kernels: 32 where that still leaves two
+// CTAs to every SM, else 8 (shorter serial sweeps). `ctas(Ls)` is the CTA count.
+template <typename F>
+int sweep_len(F ctas) {
+  return ctas(32) >= 2 * (int64_t)sm_count_cached() ? 32 : 8;
+}
+
+template <typename T>
+cudaError_t prep(const Geo& g, const MixIn<T>& a, float* x_c, float* dt_c, float* x_n, float* dt_f, float* dt_r,
+                 cudaStream_t s) {
+  const int64_t quads = (g.D + 3) / 4;
+  unsigned tx = 8;  // threads along the channels, the rest along the sweeps
+  while (tx < kPrepCta && tx < quads) tx <<= 1;
+  const unsigned ty = kPrepCta / tx, tiles = (unsigned)((quads + tx - 1) / tx);
+  auto runs = [&](int ls) { return (unsigned)(((g.L + ls - 1) / ls + ty - 1) / ty); };
+  const int Ls = sweep_len([&](int ls) { return g.Bt * tiles * runs(ls); });
+  cudaError_t e = set_smem_cached((const void*)k_mix_prep<T>, (int)prep_smem<T>(), -1);
+  if (e != cudaSuccess) return e;
+  k_mix_prep<T><<<dim3(runs(Ls), tiles, (unsigned)g.Bt), dim3(tx, ty), prep_smem<T>(), s>>>(a, x_c, dt_c, x_n, dt_f,
+                                                                                           dt_r, Ls);
+  return api_launched(cudaGetLastError(), s);
 }
 
 // The forward of both streams up to the scan outputs: prep, B/C to fp32, the
@@ -493,8 +718,7 @@ cudaError_t mix_forward_core(const Geo& g, int N, const bdscan_clean* cl, const 
   const int64_t nn = g.Bt * g.L * N;
   float* X[5];
   for (int i = 0; i < 5; ++i) X[i] = (float*)(ws + w.x[i]);
-  k_mix_prep<T><<<rows_grid(g, 1), 256, 0, s>>>(a, X[0], X[1], X[2], X[3], X[4]);
-  cudaError_t e = api_launched(cudaGetLastError(), s);
+  cudaError_t e = prep<T>(g, a, X[0], X[1], X[2], X[3], X[4], s);
   const void* bc[6] = {cl->B, cl->C, nz->B_f, nz->C_f, nz->B_r, nz->C_r};
   if (e == cudaSuccess) e = to_f32<T>(bc, w.bc, 6, ws, nn, s);
   if (e != cudaSuccess) return e;
@@ -604,25 +828,26 @@ cudaError_t mix_backward_t(const Geo& g, int N, const bdscan_clean* cl, const vo
   if (e != cudaSuccess) return e;
   // through SiLU, softplus and the convolution
   const MixIn<T> a = mix_in<T>(g, cl, nz, mp, nullptr);
-  k_mix_dpre<T, TO><<<rows_grid(g, 1), 256, 0, s>>>(a, G[0], G[1], G[2], G[3], G[4], (TO*)gc->ddt, (TO*)gn->ddt_f,
-                                                 (TO*)gn->ddt_r);
-  e = api_launched(cudaGetLastError(), s);
-  if (e != cudaSuccess) return e;
-  k_mix_dxr<TO, Vec<T>::V><<<rows_grid(g, Vec<T>::V), 256, 0, s>>>(g.Bt, g.L, g.D, g.Bs, mp->conv_w, G[0], G[2], (TO*)gc->dx, (TO*)gn->dx);
-  e = api_launched(cudaGetLastError(), s);
-  if (e != cudaSuccess) return e;
-  void* gbc_out[6] = {gc->dB, gc->dC, gn->dB_f, gn->dC_f, gn->dB_r, gn->dC_r};
-  for (int i = 0; i < 6 && e == cudaSuccess; ++i) {
-    k_mix_cvt<float, TO><<<blocks_of(nn), 256, 0, s>>>(nn, (const float*)(ws + w.gbc[i]), (TO*)gbc_out[i]);
-    e = api_launched(cudaGetLastError(), s);
-  }
-  if (e != cudaSuccess) return e;
   float* part = (float*)(ws + w.part);
-  k_mix_par_part<T><<<dim3((unsigned)((g.D + 128 * Vec<T>::V - 1) / (128 * Vec<T>::V)), kParSplit), 128, 0, s>>>(a, G[0], G[2], G[1], G[3], G[4],
-                                                                                  part);
+  const int64_t tiles = (g.D + 63) / 64;
+  auto ctas = [&](int ls) { return (g.Bt * ((g.L + ls - 1) / ls) + kBwdGroups - 1) / kBwdGroups; };
+  const int Ls = sweep_len([&](int ls) { return ctas(ls) * tiles; });
+  const int64_t want = ctas(Ls);
+  const int slices = (int)(want < kParSplit ? want : kParSplit);
+  if ((e = set_smem_cached((const void*)k_mix_bwd<T, TO>, (int)mix_bwd_smem<T>(), -1)) != cudaSuccess) return e;
+  k_mix_bwd<T, TO><<<dim3((unsigned)slices, (unsigned)tiles), dim3(32, kBwdGroups), mix_bwd_smem<T>(), s>>>(
+      a, G[0], G[1], G[2], G[3], G[4], (TO*)gc->dx, (TO*)gc->ddt, (TO*)gn->dx, (TO*)gn->ddt_f, (TO*)gn->ddt_r, Ls,
+      (int)((g.L + Ls - 1) / Ls), part);
   e = api_launched(cudaGetLastError(), s);
   if (e != cudaSuccess) return e;
-  k_mix_par_red<<<blocks_of(g.D * (kW + 3)), 256, 0, s>>>(g.D, part, gm->dconv_w, gm->dconv_b, gm->ddt_bias_f,
+  CvtSet cv;
+  void* gbc_out[6] = {gc->dB, gc->dC, gn->dB_f, gn->dC_f, gn->dB_r, gn->dC_r};
+  for (int i = 0; i < 6; ++i) {
+    cv.src[i] = ws + w.gbc[i];
+    cv.dst[i] = gbc_out[i];
+  }
+  if ((e = cvt_all<float, TO>(cv, 6, nn, s)) != cudaSuccess) return e;
+  k_mix_par_red<<<blocks_of(g.D * (kW + 3)), 256, 0, s>>>(g.D, slices, part, gm->dconv_w, gm->dconv_b, gm->ddt_bias_f,
                                                           gm->ddt_bias_r);
   return api_launched(cudaGetLastError(), s);
 }
@@ -635,9 +860,7 @@ cudaError_t mix_boundary_t(const Geo& g, int N, const bdscan_clean* cl, const vo
   const MixWs w = mix_ws(g, N);
   const MixIn<T> a = mix_in<T>(g, cl, nullptr, mp, conv_init);
   const int64_t n = g.Bt * g.L * g.D, nn = g.Bt * g.L * N;
-  k_mix_prep<T><<<rows_grid(g, 1), 256, 0, s>>>(a, (float*)(ws + w.x[0]), (float*)(ws + w.x[1]), nullptr, nullptr,
-                                             nullptr);
-  cudaError_t e = api_launched(cudaGetLastError(), s);
+  cudaError_t e = prep<T>(g, a, (float*)(ws + w.x[0]), (float*)(ws + w.x[1]), nullptr, nullptr, nullptr, s);
   const void* bc[2] = {cl->B, cl->C};
   if (e == cudaSuccess) e = to_f32<T>(bc, w.bc, 2, ws, nn, s);
   if (e != cudaSuccess) return e;
@@ -671,9 +894,8 @@ cudaError_t mix_active_t(const Geo& g, int N, const float* seed, const float* co
   // convolution state
   const MixIn<T> a = mix_in<T>(g, nullptr, nz, mp, conv_seed);
   const int64_t n = g.Bt * g.L * g.D, nn = g.Bt * g.L * N;
-  k_mix_prep<T><<<rows_grid(g, 1), 256, 0, s>>>(a, nullptr, nullptr, (float*)(ws + w.x[2]), (float*)(ws + w.x[3]),
-                                             (float*)(ws + w.x[4]));
-  cudaError_t e = api_launched(cudaGetLastError(), s);
+  cudaError_t e = prep<T>(g, a, nullptr, nullptr, (float*)(ws + w.x[2]), (float*)(ws + w.x[3]),
+                          (float*)(ws + w.x[4]), s);
   const void* bc[4] = {nz->B_f, nz->C_f, nz->B_r, nz->C_r};
   if (e == cudaSuccess) e = to_f32<T>(bc, w.bc + 2, 4, ws, nn, s);
   if (e != cudaSuccess) return e;
