@@ -186,7 +186,7 @@ size_t fwd_ws(const bds::Geo& g, int N) {
 }
 
 struct BwdWs {
-  size_t dS, Lc, sdtc, part_tok, part_A, part_D, ck, total;
+  size_t dS, Lc, sdtc, part_tok, part_A, part_D, ck, dx_part, total;
 };
 BwdWs bwd_ws(const bds::Geo& g, int N) {
   BwdWs w;
@@ -207,6 +207,8 @@ BwdWs bwd_ws(const bds::Geo& g, int N) {
   // (grid G x nc x Bt), (Bs/16 - 1) x N x 128 floats each
   w.ck = o;
   if (g.Bs > bds::kCkSmemMaxBs) o += 2 * al256((size_t)g.G * g.nc * g.Bt * (g.Bs / 16 - 1) * N * bds::kCtaHost * 4);
+  w.dx_part = o;
+  if (bds::split_parts(g)) o += al256((size_t)2 * g.Bt * g.L * g.D * 4);
   w.total = o;
   return w;
 }
@@ -697,7 +699,7 @@ int bdscan_forward(const bdscan_dims* dims, const bdscan_clean* clean, const bds
   p.hst = (float*)workspace;
   p.sdt = (float*)((char*)workspace + al256((size_t)c.g.Bt * (c.g.nc + 1) * c.g.D * c.N * 4));
   if ((rc = run_chunk_states(c, p, s, fn))) return rc;
-  cudaError_t e = launched(bds::launch_block_scan(c.dt, c.N, 0, c.g.nc, p, s), s);
+  cudaError_t e = bds::api_run_blocks(c.dt, c.N, p, s);
   if (e != cudaSuccess) return cuda_fail(e, fn);
   return ok();
 }
@@ -1082,8 +1084,27 @@ cudaError_t api_run_boundary(int dt, int N, FwdParams& p, float* states, int emi
   return launched(launch_block_scan(dt, N, 1, 1, p, s), s);
 }
 
+// Where the fused block scan would leave SMs idle, the clean rescan and the
+// noisy blocks are launched apart: the noisy blocks then all run at once, each
+// with its two directions in two warps, instead of one after another behind
+// their chunk's clean tokens. Same per-channel arithmetic, so the same bits.
+// The line lies at two CTAs of the fused scan per SM, where both sides take
+// the same time (2 x 2048 x 1536, blocks of 16, 384 CTAs: 100 us fused, 106
+// apart; half the batch: 78 and 71; 256 x 32 in 2 CTAs: 49 and 31). A block
+// above 128 tokens fills an SM's shared memory with one 32-channel CTA: there
+// the fused scan is the faster one (8192 x 512, blocks of 256: 123 and 184 us).
+static bool noisy_apart(const Geo& g) {
+  return g.Bs <= 128 && (int64_t)g.G * g.nc * g.Bt < 2 * (int64_t)sm_count_cached();
+}
+
+cudaError_t api_run_blocks(int dt, int N, const FwdParams& p, cudaStream_t s) {
+  if (!noisy_apart(p.g)) return launched(launch_block_scan(dt, N, 0, p.g.nc, p, s), s);
+  const cudaError_t e = launched(launch_block_scan(dt, N, 1, p.g.nc, p, s), s);
+  return e == cudaSuccess ? launched(launch_active_block(dt, N, p, s), s) : e;
+}
+
 // The all-block forward's launches (chunk-local scan, chunk carry, block
-// scan) with p's tensors set; the workspace holds the chunk states.
+// scans) with p's tensors set; the workspace holds the chunk states.
 cudaError_t api_run_forward(int dt, int N, FwdParams& p, void* workspace, cudaStream_t s) {
   p.hst = (float*)workspace;
   p.sdt = (float*)((char*)workspace + al256((size_t)p.g.Bt * (p.g.nc + 1) * p.g.D * N * 4));
@@ -1091,7 +1112,7 @@ cudaError_t api_run_forward(int dt, int N, FwdParams& p, void* workspace, cudaSt
   cudaError_t e = cudaSuccess;
   if (p.g.nc_full > 0) e = launched(launch_chunk_local(dt, N, p, s), s);
   if (e == cudaSuccess) e = launched(launch_chunk_carry(N, p, s), s);
-  if (e == cudaSuccess) e = launched(launch_block_scan(dt, N, 0, p.g.nc, p, s), s);
+  if (e == cudaSuccess) e = api_run_blocks(dt, N, p, s);
   return e;
 }
 
@@ -1109,6 +1130,7 @@ cudaError_t api_run_backward(int dt, int N, BwdParams& p, void* workspace, cudaS
   p.part_tok = (float*)(ws + w.part_tok);
   p.part_A = (float*)(ws + w.part_A);
   p.part_D = (float*)(ws + w.part_D);
+  p.dx_part = split_parts(gb) ? (float*)(ws + w.dx_part) : nullptr;
   if (gb.Bs > kCkSmemMaxBs) {
     const size_t ckb = al256((size_t)gb.G * gb.nc * gb.Bt * (gb.Bs / 16 - 1) * N * kCtaHost * 4);
     p.ck_noisy = (float*)(ws + w.ck);

@@ -66,13 +66,29 @@ __global__ void __launch_bounds__(256) k_bwd_carry(const BwdParams p) {
 // Deterministic reductions
 // ---------------------------------------------------------------------------
 // One thread per 4 consecutive state indices of one row of one tensor: the
-// channel-group partials are summed in group order (16-byte loads).
-template <typename TO, int N>
+// channel-group partials are summed in group order (16-byte loads). Where the
+// noisy kernel's parts ran in CTAs of their own, the threads after those join
+// dx_n from the two directions' shares, with the unsplit kernel's operations.
+template <typename T, typename TO, int N>
 __global__ void __launch_bounds__(256) k_reduce_tok(const BwdParams p) {
   const Geo& g = p.g;
-  const int64_t rows = g.Bt * g.L;
+  const int64_t rows = g.Bt * g.L, ntok = 6 * rows * (N / 4);
   const int64_t idx = (int64_t)blockIdx.x * 256 + threadIdx.x;
-  if (idx >= 6 * rows * (N / 4)) return;
+  if (idx >= ntok) {
+    const int64_t i = (idx - ntok) * 4, n = rows * g.D;  // four channels of one token
+    if (p.dx_part == nullptr || i >= n || !dguard(kSiteReduceTok, i + 3, n)) return;
+    const float4 r = *reinterpret_cast<const float4*>(p.dx_part + i);
+    const float4 f = *reinterpret_cast<const float4*>(p.dx_part + n + i);
+    const T* dy = (const T*)p.dyn + i;
+    TO* o = (TO*)p.dxn + i;
+    const float* df = p.Df + i % g.D;
+    const float* dr = p.Dr + i % g.D;
+    o[0] = to_out<TO>(__fmaf_rn(__fadd_rn(df[0], dr[0]), cvt(dy[0]), __fadd_rn(r.x, f.x)));
+    o[1] = to_out<TO>(__fmaf_rn(__fadd_rn(df[1], dr[1]), cvt(dy[1]), __fadd_rn(r.y, f.y)));
+    o[2] = to_out<TO>(__fmaf_rn(__fadd_rn(df[2], dr[2]), cvt(dy[2]), __fadd_rn(r.z, f.z)));
+    o[3] = to_out<TO>(__fmaf_rn(__fadd_rn(df[3], dr[3]), cvt(dy[3]), __fadd_rn(r.w, f.w)));
+    return;
+  }
   const int n = (int)(idx % (N / 4)) * 4;
   const int64_t row = idx / (N / 4);
   const int tensor = (int)(row / rows);
@@ -176,13 +192,15 @@ cudaError_t launch_bwd_carry(int N, const BwdParams& p, cudaStream_t s) {
 }
 
 cudaError_t launch_bwd_reduce_tok(int dt, int N, const BwdParams& p, cudaStream_t s) {
-  const int64_t ntok = 6 * p.g.Bt * p.g.L * (N / 4);
-  if (ntok == 0) return cudaSuccess;
-  const unsigned blocks = (unsigned)((ntok + 255) / 256);
-  if (dt == 1) {
-    BDS_DISPATCH_N(N, k_reduce_tok<bf16, NN><<<blocks, 256, 0, s>>>(p); return cudaGetLastError();)
+  const int64_t rows = p.g.Bt * p.g.L;
+  const int64_t n = 6 * rows * (N / 4) + (p.dx_part != nullptr ? rows * p.g.D / 4 : 0);
+  if (n == 0) return cudaSuccess;
+  const unsigned blocks = (unsigned)((n + 255) / 256);
+  switch (dt) {
+    case 0: BDS_DISPATCH_N(N, k_reduce_tok<float, float, NN><<<blocks, 256, 0, s>>>(p); return cudaGetLastError();)
+    case 1: BDS_DISPATCH_N(N, k_reduce_tok<bf16, bf16, NN><<<blocks, 256, 0, s>>>(p); return cudaGetLastError();)
+    default: BDS_DISPATCH_N(N, k_reduce_tok<bf16, float, NN><<<blocks, 256, 0, s>>>(p); return cudaGetLastError();)
   }
-  BDS_DISPATCH_N(N, k_reduce_tok<float, NN><<<blocks, 256, 0, s>>>(p); return cudaGetLastError();)
 }
 
 cudaError_t launch_bwd_reduce_par(int N, const BwdParams& p, cudaStream_t s) {
@@ -200,6 +218,7 @@ cudaError_t launch_bwd_reduce_par(int N, const BwdParams& p, cudaStream_t s) {
 // sum is taken. Falls back to the forward chunking if the attribute queries
 // fail.
 int bwd_chunk_count(int dt, int N, const Geo& g) {
+  if (split_parts(g)) return g.nb;
   int dev = 0, sms = 0;
   if (cudaGetDevice(&dev) != cudaSuccess) return g.nc;
   if (cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev) != cudaSuccess || sms <= 0) return g.nc;

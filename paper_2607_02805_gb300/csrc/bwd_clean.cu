@@ -17,10 +17,10 @@ struct CleanBwdSmem {
   static __host__ __device__ size_t slot_off(int bufs, int TS, int Bs) {
     return ck_off(bufs) + (Bs > kCkSmemMaxBs ? 0 : (size_t)(Bs / TS - 1) * N * kCta * 4);
   }
-  // one-segment blocks: the seeds of the current and the next block
+  // one-segment blocks: the seed of each buffer's block
   static __host__ __device__ size_t seed_off(int bufs, int TS, int Bs) { return slot_off(bufs, TS, Bs) + 16; }
   static __host__ __device__ size_t bytes(int bufs, int TS, int Bs) {
-    return seed_off(bufs, TS, Bs) + (Bs / TS == 1 ? (size_t)2 * kCta * N * 4 : 0);
+    return seed_off(bufs, TS, Bs) + (Bs / TS == 1 ? (size_t)bufs * kCta * N * 4 : 0);
   }
 };
 
@@ -52,7 +52,7 @@ __global__ void __launch_bounds__(kCta, 3) k_bwd_clean(const BwdParams p) {
   st.row_src[BC] = (const T*)p.Bc;
   st.row_src[CC] = (const T*)p.Cc;
   const bool resident = NSEG > 1 && p.seg_resident;
-  const int bufs = NSEG == 1 ? 2 : (resident ? NSEG : 1);
+  const int bufs = NSEG == 1 ? (is_f32<T>::value ? p.stage_bufs : 2) : (resident ? NSEG : 1);
   float* red = reinterpret_cast<float*>(smem + L::red_off(bufs));
   float* mine = red_slot<N>(red);
   float* ck = Bs > kCkSmemMaxBs
@@ -156,39 +156,40 @@ __global__ void __launch_bounds__(kCta, 3) k_bwd_clean(const BwdParams p) {
     // flushed once.
     const int TB = kBwdTS / Bs;
     auto tile_lo = [&](int hi) { return hi - TB + 1 > k_lo ? hi - TB + 1 : k_lo; };
-    issue_seed<N>(seedb, p.states, g, b, k_hi, d0);  // same cp.async group as the tile
-    st.issue(0, b * g.L + (int64_t)tile_lo(k_hi) * Bs, (k_hi - tile_lo(k_hi) + 1) * Bs, g.D, d0);
+    auto issue_tile = [&](int buf, int lo, int hi) {
+      issue_seed<N>(seedb + buf * kCta * N, p.states, g, b, hi, d0);  // same cp.async group as the tile
+      st.issue(buf, b * g.L + (int64_t)lo * Bs, (hi - lo + 1) * Bs, g.D, d0);
+    };
+    if (bufs == 2) issue_tile(0, tile_lo(k_hi), k_hi);
     int tile = 0;
     for (int kt_hi = k_hi; kt_hi >= k_lo; ++tile) {
       const int kt_lo = tile_lo(kt_hi), nbk = kt_hi - kt_lo + 1;
-      const int buf = tile & 1;
-      __syncthreads();  // the other buffer is no longer read
-      if (kt_lo > k_lo) {
-        const int nhi = kt_lo - 1, nlo = tile_lo(nhi);
-        issue_seed<N>(seedb + (buf ^ 1) * kCta * N, p.states, g, b, nhi, d0);
-        st.issue(buf ^ 1, b * g.L + (int64_t)nlo * Bs, (nhi - nlo + 1) * Bs, g.D, d0);
-      }
-      st.complete(buf, nbk * Bs, kt_lo > k_lo ? 1 : 0);
+      const int buf = bufs == 2 ? tile & 1 : 0;
+      const bool ahead = bufs == 2 && kt_lo > k_lo;
+      __syncthreads();  // the buffer to fill is no longer read
+      if (bufs == 1) issue_tile(0, kt_lo, kt_hi);
+      if (ahead) issue_tile(buf ^ 1, tile_lo(kt_lo - 1), kt_lo - 1);
+      st.complete(buf, nbk * Bs, ahead ? 1 : 0);
       for (int k = kt_hi; k >= kt_lo; --k) block(k, (k - kt_lo) * Bs, buf, k == kt_hi);
       red_flush<N>(p, red, 0, 1, 0, 1, b, (int64_t)kt_lo * Bs, nbk * Bs);  // the tile's dB/dC
       kt_hi = kt_lo - 1;
     }
   } else {
-    // one-segment blocks: block k-1 (and its seed) is copied while block k is processed
-    if (NSEG == 1) {
-      issue_seed<N>(seedb, p.states, g, b, k_hi, d0);  // same cp.async group as the block
-      st.issue(0, b * g.L + (int64_t)k_hi * Bs, TS, g.D, d0);
-    }
+    // one-segment blocks, two buffers: block k-1 (and its seed) is copied while block k is processed
+    auto issue_block = [&](int buf, int k) {
+      issue_seed<N>(seedb + buf * kCta * N, p.states, g, b, k, d0);  // same cp.async group as the block
+      st.issue(buf, b * g.L + (int64_t)k * Bs, TS, g.D, d0);
+    };
+    if (NSEG == 1 && bufs == 2) issue_block(0, k_hi);
     for (int k = k_hi; k >= k_lo; --k) {
       const int64_t row0 = b * g.L + (int64_t)k * Bs;
-      const int buf = (k_hi - k) & 1;
+      const int buf = NSEG == 1 && bufs == 2 ? (k_hi - k) & 1 : 0;
       if (NSEG == 1) {
-        __syncthreads();  // the other buffer is no longer read
-        if (k > k_lo) {
-          issue_seed<N>(seedb + (buf ^ 1) * kCta * N, p.states, g, b, k - 1, d0);
-          st.issue(buf ^ 1, row0 - Bs, TS, g.D, d0);
-        }
-        st.complete(buf, TS, k > k_lo ? 1 : 0);
+        const bool ahead = bufs == 2 && k > k_lo;
+        __syncthreads();  // the buffer to fill is no longer read
+        if (bufs == 1) issue_block(0, k);
+        if (ahead) issue_block(buf ^ 1, k - 1);
+        st.complete(buf, TS, ahead ? 1 : 0);
       } else if (resident) {  // every segment of the block, once
         __syncthreads();  // the previous block is no longer read
         for (int s = 0; s < NSEG; ++s) st.issue(s, row0 + (int64_t)s * TS, TS, g.D, d0);
@@ -211,7 +212,7 @@ namespace {
 template <typename T, typename TO, int N, bool TILED>
 BwdLaunch clean_launch(int Bs, int dev) {
   const int TS = Bs < 16 ? Bs : 16;
-  return bwd_launch<CleanBwdSmem<T, N>>(k_bwd_clean<T, TO, N, TILED>, Bs, half_cols(TS, N), dev);
+  return bwd_launch<CleanBwdSmem<T, N>, is_f32<T>::value>(k_bwd_clean<T, TO, N, TILED>, Bs, half_cols(TS, N), dev);
 }
 
 template <typename T, typename TO, int N, bool TILED>
@@ -222,6 +223,7 @@ cudaError_t bwd_clean_tt(const BwdParams& p_in, cudaStream_t s) {
   const BwdLaunch l = clean_launch<T, TO, N, TILED>((int)p_in.g.Bs, dev);
   BwdParams p = p_in;
   p.seg_resident = l.resident;
+  p.stage_bufs = l.bufs;
   e = set_bwd_attrs(k_bwd_clean<T, TO, N, TILED>, l.smem);
   if (e != cudaSuccess) return e;
   dim3 grid((unsigned)p.g.G, (unsigned)p.g.nc, (unsigned)p.g.Bt);

@@ -364,19 +364,25 @@ int resident_ctas(K kernel, size_t smem, uint32_t tcols, int dev) {
   return n;
 }
 
-// Shared memory of a launch, and whether a block of several segments is
-// staged whole (one buffer per segment): only where that costs no resident CTA.
+// Shared memory of a launch, whether a block of several segments is staged
+// whole (one buffer per segment; only where that costs no resident CTA), and
+// the buffers of one-segment blocks: two, or, for fp32 inputs (ONE), one where
+// that leaves more CTAs on an SM (16 states: the noisy kernel's 132 KB admit
+// one CTA, its 78 KB with one buffer two; 8 x 2048 x 1536, blocks of 16: 1291
+// -> 855 us; the clean kernel gets three CTAs instead of two: 444 -> 378 us).
 struct BwdLaunch {
   size_t smem;
-  int resident;
+  int resident, bufs;
 };
-template <typename L, typename K>
+template <typename L, bool ONE, typename K>
 BwdLaunch bwd_launch(K kernel, int Bs, uint32_t cols, int dev) {
   const int TS = Bs < 16 ? Bs : 16, nseg = Bs / TS;
-  if (nseg == 1) return {pad_for_tmem(L::bytes(2, TS, Bs), cols), 0};
-  const size_t one = pad_for_tmem(L::bytes(1, TS, Bs), cols), all = pad_for_tmem(L::bytes(nseg, TS, Bs), cols);
+  if (nseg == 1 && !ONE) return {pad_for_tmem(L::bytes(2, TS, Bs), cols), 0, 2};
+  const size_t one = pad_for_tmem(L::bytes(1, TS, Bs), cols);
+  const size_t all = pad_for_tmem(L::bytes(nseg == 1 ? 2 : nseg, TS, Bs), cols);
   const int r1 = resident_ctas(kernel, one, cols, dev), ra = resident_ctas(kernel, all, cols, dev);
-  return ra >= r1 && ra > 0 ? BwdLaunch{all, 1} : BwdLaunch{one, 0};
+  if (ra >= r1 && ra > 0) return {all, nseg > 1, 2};
+  return {one, 0, 1};
 }
 }  // namespace
 

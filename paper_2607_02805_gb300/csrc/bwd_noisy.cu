@@ -11,9 +11,10 @@ template <typename T, int N>
 struct NoisyBwdSmem {
   // token-by-channel: x_n, dt_f, dt_r, dy_n, dt_c, dy_c; token-by-state: B_f, C_f, B_r, C_r, C_c
   using St = Stage<T, N, 6, 5, 2, kBwdTS>;
-  // `bufs` staging buffers: 2 for one-segment blocks (the next block is
-  // copied while the current one is used); for longer blocks one per segment
-  // (the whole block resident) or 1 (each segment copied when needed)
+  // `bufs` staging buffers: for one-segment blocks 2 (the next block is copied
+  // while the current one is used) or, where that leaves more CTAs on an SM, 1;
+  // for longer blocks one per segment (the whole block resident) or 1 (each
+  // segment copied when needed)
   static __host__ __device__ size_t dx_off(int bufs) { return align16(St::buf_bytes(kBwdTS) * bufs); }
   // dx partials of a tile (several short blocks) or of one long block
   static __host__ __device__ size_t red_off(int bufs, int Bs) { return dx_off(bufs) + (size_t)(Bs < kBwdTS ? kBwdTS : Bs) * kCta * 4; }
@@ -29,14 +30,19 @@ struct NoisyBwdSmem {
 };
 
 // TILED (blocks shorter than kBwdTS tokens): several blocks per staged tile.
-template <typename T, typename TO, int N, bool TILED>
+// SPLIT (small problems, split_parts): the chunk is one block, and a CTA does
+// one of the three parts of its work, none of which reads what another makes.
+template <typename T, typename TO, int N, bool TILED, bool SPLIT>
 __global__ void __launch_bounds__(kCta, 1) k_bwd_noisy(const BwdParams p) {
+  static_assert(!(TILED && SPLIT), "a split launch has one block per CTA");
   extern __shared__ __align__(16) unsigned char smem[];
   using L = NoisyBwdSmem<T, N>;
   const Geo& g = p.g;
   const int tid = threadIdx.x, warp = tid >> 5;
   const int sw = swz_of_lane<N>();
-  const int64_t b = blockIdx.z;
+  const unsigned part = SPLIT ? blockIdx.z % 3 : 0;
+  const bool do_clean = !SPLIT || part == 0, do_rev = !SPLIT || part == 1, do_fwd = !SPLIT || part == 2;
+  const int64_t b = SPLIT ? blockIdx.z / 3 : blockIdx.z;
   const int c = blockIdx.y;
   const int64_t d0 = (int64_t)blockIdx.x * kCta, d = d0 + tid;
   const bool act = d < g.D;
@@ -63,7 +69,9 @@ __global__ void __launch_bounds__(kCta, 1) k_bwd_noisy(const BwdParams p) {
   st.row_src[CR] = (const T*)p.Cr;
   st.row_src[CC] = (const T*)p.Cc;
   const bool resident = NSEG > 1 && p.seg_resident;
-  const int bufs = NSEG == 1 ? 2 : (resident ? NSEG : 1);
+  const int bufs = NSEG == 1 ? (is_f32<T>::value ? p.stage_bufs : 2) : (resident ? NSEG : 1);
+  float* dxr_part = p.dx_part;  // SPLIT: where the two directions leave their share of dx
+  float* dxf_part = SPLIT ? p.dx_part + g.Bt * g.L * g.D : nullptr;
   float* dxbuf = reinterpret_cast<float*>(smem + L::dx_off(bufs));
   float* red = reinterpret_cast<float*>(smem + L::red_off(bufs, Bs));
   float* mine = red_slot<N>(red);
@@ -125,7 +133,7 @@ __global__ void __launch_bounds__(kCta, 1) k_bwd_noisy(const BwdParams p) {
         for (int j = 0; j < N / 2; ++j) carry[j] = add2(carry[j], e[j]);
       }
     }
-    for (int s = NSEG - 1; s >= 0; --s) {
+    if (do_clean) for (int s = NSEG - 1; s >= 0; --s) {
       if (NSEG > 1) stage_seg(s);
 #pragma unroll 4
       for (int i = TS - 1; i >= 0; --i) {
@@ -140,7 +148,7 @@ __global__ void __launch_bounds__(kCta, 1) k_bwd_noisy(const BwdParams p) {
     }
 
     // ---- noisy block k, reverse direction (zero state at the block end) ----
-    {
+    if (do_rev) {
       if (NSEG > 1) {
         float2 h[N / 2];
         vzero2<N>(h);
@@ -166,14 +174,17 @@ __global__ void __launch_bounds__(kCta, 1) k_bwd_noisy(const BwdParams p) {
                             if (act)
                               reinterpret_cast<TO*>(p.ddtr)[(row0 + ib) * g.D + d] =
                                   to_out<TO>(__fmaf_rn(x, sgB, __fmul_rn(kLn2, sAq)));
-                            dxbuf[(off + ib) * kCta + tid] = __fmul_rn(dt, sgB);
+                            if (!SPLIT)
+                              dxbuf[(off + ib) * kCta + tid] = __fmul_rn(dt, sgB);
+                            else if (act)
+                              dxr_part[(row0 + ib) * g.D + d] = __fmul_rn(dt, sgB);
                           });
         if (!TILED) red_flush<N>(p, red, 0, 1, 4, 5, b, t0 + (int64_t)s * TS, TS);
       }
     }
 
     // ---- noisy block k, forward direction (seeded with states[k-1]) ----
-    {
+    if (do_fwd) {
       float2 seed[N / 2];
       vzero2<N>(seed);
       if (k > 0 && act) vload2<N>(seed, p.states + ((b * g.nb + (k - 1)) * g.D + d) * N, sw);
@@ -205,9 +216,12 @@ __global__ void __launch_bounds__(kCta, 1) k_bwd_noisy(const BwdParams p) {
                            const int64_t o = (row0 + ib) * g.D + d;
                            if (act) {
                              reinterpret_cast<TO*>(p.ddtf)[o] = to_out<TO>(__fmaf_rn(x, sgB, __fmul_rn(kLn2, sAq)));
-                             const float dxv =
-                                 __fmaf_rn(Dsum, dy, __fadd_rn(dxbuf[(off + ib) * kCta + tid], __fmul_rn(dt, sgB)));
-                             reinterpret_cast<TO*>(p.dxn)[o] = to_out<TO>(dxv);
+                             const float dxf = __fmul_rn(dt, sgB);
+                             if (SPLIT)
+                               dxf_part[o] = dxf;
+                             else
+                               reinterpret_cast<TO*>(p.dxn)[o] = to_out<TO>(
+                                   __fmaf_rn(Dsum, dy, __fadd_rn(dxbuf[(off + ib) * kCta + tid], dxf)));
                            }
                            dDn = __fmaf_rn(dy, x, dDn);
                          });
@@ -226,33 +240,35 @@ __global__ void __launch_bounds__(kCta, 1) k_bwd_noisy(const BwdParams p) {
     // partials of a tile are flushed once for both directions.
     const int TB = kBwdTS / Bs;
     auto tile_lo = [&](int hi) { return hi - TB + 1 > k_lo ? hi - TB + 1 : k_lo; };
-    st.issue(0, b * g.L + (int64_t)tile_lo(k_hi) * Bs, (k_hi - tile_lo(k_hi) + 1) * Bs, g.D, d0);
+    auto issue_tile = [&](int buf, int lo, int hi) { st.issue(buf, b * g.L + (int64_t)lo * Bs, (hi - lo + 1) * Bs, g.D, d0); };
+    if (bufs == 2) issue_tile(0, tile_lo(k_hi), k_hi);
     int tile = 0;
     for (int kt_hi = k_hi; kt_hi >= k_lo; ++tile) {
       const int kt_lo = tile_lo(kt_hi), nbk = kt_hi - kt_lo + 1;
-      const int buf = tile & 1;
-      __syncthreads();  // the other buffer is no longer read
-      if (kt_lo > k_lo) {
-        const int nhi = kt_lo - 1, nlo = tile_lo(nhi);
-        st.issue(buf ^ 1, b * g.L + (int64_t)nlo * Bs, (nhi - nlo + 1) * Bs, g.D, d0);
-      }
-      st.complete(buf, nbk * Bs, kt_lo > k_lo ? 1 : 0);
+      const int buf = bufs == 2 ? tile & 1 : 0;
+      const bool ahead = bufs == 2 && kt_lo > k_lo;
+      __syncthreads();  // the buffer to fill is no longer read
+      if (bufs == 1) issue_tile(0, kt_lo, kt_hi);
+      if (ahead) issue_tile(buf ^ 1, tile_lo(kt_lo - 1), kt_lo - 1);
+      st.complete(buf, nbk * Bs, ahead ? 1 : 0);
       for (int k = kt_hi; k >= kt_lo; --k) block(k, (k - kt_lo) * Bs);
       const int64_t ts0 = (int64_t)kt_lo * Bs;  // the tile's dB/dC partials, both directions
-      red_flush<N>(p, red, 0, 1, 4, 5, b, ts0, nbk * Bs);
-      red_flush<N>(p, red, 2, 3, 2, 3, b, ts0, nbk * Bs);
+      if (do_rev) red_flush<N>(p, red, 0, 1, 4, 5, b, ts0, nbk * Bs);
+      if (do_fwd) red_flush<N>(p, red, 2, 3, 2, 3, b, ts0, nbk * Bs);
       kt_hi = kt_lo - 1;
     }
   } else {
-    // one-segment blocks: block k-1 is copied while block k is processed
-    if (NSEG == 1) st.issue(0, b * g.L + (int64_t)k_hi * Bs, TS, g.D, d0);
+    // one-segment blocks, two buffers: block k-1 is copied while block k is processed
+    if (NSEG == 1 && bufs == 2) st.issue(0, b * g.L + (int64_t)k_hi * Bs, TS, g.D, d0);
     for (int k = k_hi; k >= k_lo; --k) {
       const int64_t row0 = b * g.L + (int64_t)k * Bs;
       if (NSEG == 1) {
-        const int buf = (k_hi - k) & 1;
-        __syncthreads();  // the other buffer is no longer read
-        if (k > k_lo) st.issue(buf ^ 1, row0 - Bs, TS, g.D, d0);
-        st.complete(buf, TS, k > k_lo ? 1 : 0);
+        const int buf = bufs == 2 ? (k_hi - k) & 1 : 0;
+        const bool ahead = bufs == 2 && k > k_lo;
+        __syncthreads();  // the buffer to fill is no longer read
+        if (bufs == 1) st.issue(0, row0, TS, g.D, d0);
+        if (ahead) st.issue(buf ^ 1, row0 - Bs, TS, g.D, d0);
+        st.complete(buf, TS, ahead ? 1 : 0);
       } else if (resident) {  // every segment of the block, once
         __syncthreads();  // the previous block is no longer read
         for (int s = 0; s < NSEG; ++s) st.issue(s, row0 + (int64_t)s * TS, TS, g.D, d0);
@@ -263,12 +279,16 @@ __global__ void __launch_bounds__(kCta, 1) k_bwd_noisy(const BwdParams p) {
   }
 
   if (act) {
-    vstore2<N>(p.Lc + ((b * g.nc + c) * g.D + d) * N, carry, sw);
-    p.sdtc[(b * g.nc + c) * g.D + d] = sdt;
     const int64_t u = b * g.nc + c, U = g.Bt * g.nc;
-    vstore2<N>(p.part_A + ((0 * U + u) * g.D + d) * N, dAf, sw);
-    vstore2<N>(p.part_A + ((1 * U + u) * g.D + d) * N, dAr, sw);
-    p.part_D[(0 * U + u) * g.D + d] = dDn;
+    if (do_clean) {
+      vstore2<N>(p.Lc + (u * g.D + d) * N, carry, sw);
+      p.sdtc[u * g.D + d] = sdt;
+    }
+    if (do_fwd) {
+      vstore2<N>(p.part_A + ((0 * U + u) * g.D + d) * N, dAf, sw);
+      p.part_D[(0 * U + u) * g.D + d] = dDn;
+    }
+    if (do_rev) vstore2<N>(p.part_A + ((1 * U + u) * g.D + d) * N, dAr, sw);
   }
   tmem_sync();
   if (warp == 0) tmem_dealloc(tbase, tcols);
@@ -276,36 +296,40 @@ __global__ void __launch_bounds__(kCta, 1) k_bwd_noisy(const BwdParams p) {
 
 namespace {
 
-template <typename T, typename TO, int N, bool TILED>
+template <typename T, typename TO, int N, bool TILED, bool SPLIT>
 BwdLaunch noisy_launch(int Bs, int dev) {
   const int TS = Bs < 16 ? Bs : 16;
-  return bwd_launch<NoisyBwdSmem<T, N>>(k_bwd_noisy<T, TO, N, TILED>, Bs, full_cols(TS, N), dev);
+  return bwd_launch<NoisyBwdSmem<T, N>, is_f32<T>::value>(k_bwd_noisy<T, TO, N, TILED, SPLIT>, Bs, full_cols(TS, N), dev);
 }
-template <typename T, typename TO, int N, bool TILED>
+template <typename T, typename TO, int N, bool TILED, bool SPLIT>
 cudaError_t bwd_noisy_tt(const BwdParams& p_in, cudaStream_t s) {
   int dev = 0;
   cudaError_t e = cudaGetDevice(&dev);
   if (e != cudaSuccess) return e;
-  const BwdLaunch l = noisy_launch<T, TO, N, TILED>((int)p_in.g.Bs, dev);
+  const BwdLaunch l = noisy_launch<T, TO, N, TILED, SPLIT>((int)p_in.g.Bs, dev);
   BwdParams p = p_in;
   p.seg_resident = l.resident;
-  e = set_bwd_attrs(k_bwd_noisy<T, TO, N, TILED>, l.smem);
+  p.stage_bufs = l.bufs;
+  e = set_bwd_attrs(k_bwd_noisy<T, TO, N, TILED, SPLIT>, l.smem);
   if (e != cudaSuccess) return e;
-  dim3 grid((unsigned)p.g.G, (unsigned)p.g.nc, (unsigned)p.g.Bt);
-  k_bwd_noisy<T, TO, N, TILED><<<grid, kCta, l.smem, s>>>(p);
+  dim3 grid((unsigned)p.g.G, (unsigned)p.g.nc, (unsigned)(SPLIT ? 3 * p.g.Bt : p.g.Bt));
+  k_bwd_noisy<T, TO, N, TILED, SPLIT><<<grid, kCta, l.smem, s>>>(p);
   return cudaGetLastError();
 }
 template <typename T, typename TO, int N>
 cudaError_t bwd_noisy_t(const BwdParams& p, cudaStream_t s) {
-  return p.g.Bs < kBwdTS ? bwd_noisy_tt<T, TO, N, true>(p, s) : bwd_noisy_tt<T, TO, N, false>(p, s);
+  if (p.dx_part != nullptr) return bwd_noisy_tt<T, TO, N, false, true>(p, s);
+  return p.g.Bs < kBwdTS ? bwd_noisy_tt<T, TO, N, true, false>(p, s) : bwd_noisy_tt<T, TO, N, false, false>(p, s);
 }
 
 template <typename T, typename TO, int N>
 int bwd_noisy_per_sm_t(int Bs, int dev) {
   const int TS = Bs < 16 ? Bs : 16;
   if (Bs < kBwdTS)
-    return resident_ctas(k_bwd_noisy<T, TO, N, true>, noisy_launch<T, TO, N, true>(Bs, dev).smem, full_cols(TS, N), dev);
-  return resident_ctas(k_bwd_noisy<T, TO, N, false>, noisy_launch<T, TO, N, false>(Bs, dev).smem, full_cols(TS, N), dev);
+    return resident_ctas(k_bwd_noisy<T, TO, N, true, false>, noisy_launch<T, TO, N, true, false>(Bs, dev).smem,
+                         full_cols(TS, N), dev);
+  return resident_ctas(k_bwd_noisy<T, TO, N, false, false>, noisy_launch<T, TO, N, false, false>(Bs, dev).smem,
+                       full_cols(TS, N), dev);
 }
 
 }  // namespace

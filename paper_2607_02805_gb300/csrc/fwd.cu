@@ -333,7 +333,9 @@ __global__ void __launch_bounds__(kCta, MODE == 0 ? 4 : 6) k_block_scan(const Fw
 
 // ---------------------------------------------------------------------------
 // Active block (the inference step): one noisy block per batch row from a
-// read-only cached seed. A CTA covers 32 channels of one row; warp 0 runs the
+// read-only cached seed; in the all-block forward of small problems (see
+// noisy_apart) every noisy block, seeded with the clean state before it. A CTA
+// covers 32 channels of one block; warp 0 runs the
 // seeded forward scan and warp 1 the block-local reverse scan at the same
 // time, each with the per-channel arithmetic of k_block_scan (scan_step,
 // with_skip, combine_dirs), so the outputs equal those of the all-block
@@ -369,7 +371,8 @@ __global__ void __launch_bounds__(2 * kActW, 1) k_active_block(const FwdParams p
   extern __shared__ __align__(16) unsigned char smem[];
   const Geo& g = p.g;
   const int Bs = (int)g.Bs;
-  const int64_t b = blockIdx.y, d0 = (int64_t)blockIdx.x * kActW;
+  const unsigned groups = (unsigned)((g.D + kActW - 1) / kActW), k = blockIdx.x / groups;  // the block of the row
+  const int64_t b = blockIdx.y, d0 = (int64_t)(blockIdx.x - k * groups) * kActW;
   const int lane = threadIdx.x & 31, dir = threadIdx.x >> 5;  // dir 0: forward, 1: reverse
   const int64_t d = d0 + lane;
   const bool act = d < g.D;
@@ -383,7 +386,7 @@ __global__ void __launch_bounds__(2 * kActW, 1) k_active_block(const FwdParams p
   // copies (16-byte chunks; channels past D read as zero)
   constexpr int E = 16 / (int)sizeof(T);
   constexpr int CPR = kActW / E;
-  const int64_t row0 = b * g.L;
+  const int64_t row0 = b * g.L + (int64_t)k * Bs;
   for (int q = threadIdx.x; q < 3 * Bs * CPR; q += 2 * kActW) {
     const int j = q / (Bs * CPR), r = q - j * (Bs * CPR), t = r / CPR, cc = (r - t * CPR) * E;
     const T* src = (const T*)(j == 0 ? p.xn : (j == 1 ? p.dtf : p.dtr));
@@ -409,7 +412,10 @@ __global__ void __launch_bounds__(2 * kActW, 1) k_active_block(const FwdParams p
 #pragma unroll
     for (int j = 0; j < N / 2; ++j) A2[j] = mul2(A2[j], f2(kLog2e));
     Dd = dir == 0 ? p.Df[d] : p.Dr[d];
-    if (dir == 0) vload2<N>(h, p.seed + (b * g.D + d) * N, 0);
+    const float* seed = p.seed != nullptr ? p.seed + (b * g.D + d) * N
+                        : k > 0           ? p.states + ((b * g.nb + k - 1) * g.D + d) * N
+                                          : nullptr;
+    if (dir == 0 && seed != nullptr) vload2<N>(h, seed, 0);
   }
   cp_async_wait_all();
   __syncthreads();
@@ -581,13 +587,14 @@ cudaError_t block_scan_mode(int mode, int nchunks, const FwdParams& p, cudaStrea
 
 template <typename T, typename TO, int N, bool ADA = false>
 cudaError_t active_block_t(const FwdParams& p, cudaStream_t s) {
-  const size_t smem = ADA ? ActiveLayout<T, N>::bytes_ada((int)p.g.Bs) : ActiveLayout<T, N>::bytes((int)p.g.Bs);
+  using Ly = ActiveLayout<T, N>;
+  const size_t smem = ADA ? Ly::bytes_ada((int)p.g.Bs) : Ly::bytes((int)p.g.Bs);
   if (smem > 48 * 1024) {
     cudaError_t e =
         cudaFuncSetAttribute(k_active_block<T, TO, N, ADA>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
     if (e != cudaSuccess) return e;
   }
-  dim3 grid((unsigned)((p.g.D + kActW - 1) / kActW), (unsigned)p.g.Bt);
+  dim3 grid((unsigned)((p.g.D + kActW - 1) / kActW * p.g.nb), (unsigned)p.g.Bt);
   k_active_block<T, TO, N, ADA><<<grid, 2 * kActW, smem, s>>>(p);
   return cudaGetLastError();
 }

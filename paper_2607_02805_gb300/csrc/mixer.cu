@@ -204,7 +204,7 @@ constexpr size_t prep_smem() {
   return (size_t)kPrepRing * 5 * kPrepCta * 4 * sizeof(T);
 }
 template <typename T>
-__global__ void __launch_bounds__(kPrepCta) k_mix_prep(const MixIn<T> a, float* x_c, float* dt_c, float* x_n,
+__global__ void __launch_bounds__(kPrepCta, 4) k_mix_prep(const MixIn<T> a, float* x_c, float* dt_c, float* x_n,
                                                        float* dt_f, float* dt_r, int Ls) {
   extern __shared__ __align__(16) unsigned char smem[];
   constexpr int Q = 4, S = 4, W1 = kW - 1;

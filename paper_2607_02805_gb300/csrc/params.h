@@ -65,6 +65,11 @@ struct BwdParams {
   float* part_A;    // [3][Bt*nc][D][N] dA partial sums: noisy fwd, noisy rev, clean
   float* part_D;    // [2][Bt*nc][D]    dD partial sums: noisy, clean
   int seg_resident;  // set per launch: blocks of several segments staged whole
+  int stage_bufs;    // set per launch: staging buffers of one-segment blocks
+  // noisy kernel with a CTA per part of a block (split_parts below): fp32
+  // partials of dx_n, [2][Bt][L][D] (reverse, forward direction), joined by
+  // the token reduction; null otherwise
+  float* dx_part;
   // segment checkpoints of blocks above kCkSmemMaxBs tokens, in global memory:
   // per CTA (linear block index) (Bs/16 - 1) x N x 128 floats; null otherwise
   float* ck_noisy;
@@ -76,7 +81,8 @@ cudaError_t launch_chunk_local(int dt, int N, const FwdParams& p, cudaStream_t s
 cudaError_t launch_chunk_carry(int N, const FwdParams& p, cudaStream_t s);
 // mode 0: all-block forward, 1: clean scan only (cache build), 2: clean scan right to left
 cudaError_t launch_block_scan(int dt, int N, int mode, int nchunks, const FwdParams& p, cudaStream_t s);
-// One noisy block per batch row from p.seed (len == block).
+// One noisy block per batch row from p.seed (len == block), or, without
+// p.seed, every noisy block of the rows from p.states (all written before).
 cudaError_t launch_active_block(int dt, int N, const FwdParams& p, cudaStream_t s);
 // Per-token layer-norm statistics of rows x D elements (dt: 0 f32, else bf16).
 // State groups of the diagonal form (groups.cu): d_state split into groups
@@ -111,6 +117,8 @@ cudaError_t api_launched(cudaError_t e, cudaStream_t s);
 cudaError_t set_smem_cached(const void* fn, int bytes, int carveout);  // carveout < 0: leave it
 int sm_count_cached();  // 0 if unknown
 int api_check_forward_dims(const void* dims, Geo* g, int* dt, int* N, const char* fn);
+// The block scans of the all-block forward, after the chunk carry.
+cudaError_t api_run_blocks(int dt, int N, const FwdParams& p, cudaStream_t s);
 size_t api_fwd_workspace(const Geo& g, int N);
 size_t api_bwd_workspace(const Geo& g, int N);
 // Launch sequences of bdscan_forward / bdscan_backward (counted by the
@@ -119,9 +127,19 @@ cudaError_t api_run_forward(int dt, int N, FwdParams& p, void* workspace, cudaSt
 cudaError_t api_run_boundary(int dt, int N, FwdParams& p, float* states, int emit_all, cudaStream_t s);
 cudaError_t api_run_backward(int dt, int N, BwdParams& p, void* workspace, cudaStream_t s);
 int bwd_chunk_count(int dt, int N, const Geo& g);
+// Small problems, bound by the length of the serial chain of a CTA: each block
+// is a chunk of its own, and the three independent parts of its noisy kernel
+// (the clean stream's local adjoint, the reverse and the forward direction)
+// run in a CTA each. The limit is three CTAs per SM of the part that this
+// library is written for (the rule sizes workspaces, so it does not ask the
+// device); beyond it the longer chains fill the SMs as well. Blocks whose
+// checkpoints are in global memory (one region per CTA of the unsplit kernel)
+// stay unsplit.
+constexpr int64_t kSplitCtas = 456;
+inline bool split_parts(const Geo& g) { return g.Bs <= kCkSmemMaxBs && 3 * g.Bt * g.G * g.nb <= kSplitCtas; }
 // Upper bound of the backward's chunks per batch row (sizes its workspace
-// independently of the device): twice the forward chunking, at most one
-// chunk per block.
-inline int bwd_max_chunks(const Geo& g) { return g.nb < 2 * g.nc ? g.nb : 2 * g.nc; }
+// independently of the device): one chunk per block for small problems, else
+// twice the forward chunking, at most one chunk per block.
+inline int bwd_max_chunks(const Geo& g) { return g.nb < 2 * g.nc || split_parts(g) ? g.nb : 2 * g.nc; }
 
 }  // namespace bds
