@@ -11,6 +11,7 @@ namespace bds {
 // ---------------------------------------------------------------------------
 template <int N>
 __global__ void __launch_bounds__(256) k_bwd_carry(const BwdParams p) {
+  pdl_sync();
   const Geo& g = p.g;
   const int64_t idx = (int64_t)blockIdx.x * 256 + threadIdx.x;
   if (idx >= g.Bt * g.D * N) return;
@@ -71,6 +72,7 @@ __global__ void __launch_bounds__(256) k_bwd_carry(const BwdParams p) {
 // dx_n from the two directions' shares, with the unsplit kernel's operations.
 template <typename T, typename TO, int N>
 __global__ void __launch_bounds__(256) k_reduce_tok(const BwdParams p) {
+  pdl_sync();
   const Geo& g = p.g;
   const int64_t rows = g.Bt * g.L, ntok = 6 * rows * (N / 4);
   const int64_t idx = (int64_t)blockIdx.x * 256 + threadIdx.x;
@@ -119,6 +121,7 @@ __global__ void __launch_bounds__(256) k_reduce_tok(const BwdParams p) {
 constexpr int kParSlices = 16;
 template <int N>
 __global__ void __launch_bounds__(32 * kParSlices) k_reduce_par(const BwdParams p) {
+  pdl_sync();
   // kParSlices slices (warps) of the chunk partials; each lane sums 4 adjacent columns
   __shared__ float4 part[3][kParSlices][32];
   const Geo& g = p.g;
@@ -188,7 +191,7 @@ __global__ void __launch_bounds__(32 * kParSlices) k_reduce_par(const BwdParams 
 cudaError_t launch_bwd_carry(int N, const BwdParams& p, cudaStream_t s) {
   const int64_t total = p.g.Bt * p.g.D * N;
   if (total == 0) return cudaSuccess;
-  BDS_DISPATCH_N(N, k_bwd_carry<NN><<<(unsigned)((total + 255) / 256), 256, 0, s>>>(p); return cudaGetLastError();)
+  BDS_DISPATCH_N(N, launch_pdl(k_bwd_carry<NN>, (unsigned)((total + 255) / 256), 256, 0, s, p); return cudaGetLastError();)
 }
 
 cudaError_t launch_bwd_reduce_tok(int dt, int N, const BwdParams& p, cudaStream_t s) {
@@ -197,15 +200,15 @@ cudaError_t launch_bwd_reduce_tok(int dt, int N, const BwdParams& p, cudaStream_
   if (n == 0) return cudaSuccess;
   const unsigned blocks = (unsigned)((n + 255) / 256);
   switch (dt) {
-    case 0: BDS_DISPATCH_N(N, k_reduce_tok<float, float, NN><<<blocks, 256, 0, s>>>(p); return cudaGetLastError();)
-    case 1: BDS_DISPATCH_N(N, k_reduce_tok<bf16, bf16, NN><<<blocks, 256, 0, s>>>(p); return cudaGetLastError();)
-    default: BDS_DISPATCH_N(N, k_reduce_tok<bf16, float, NN><<<blocks, 256, 0, s>>>(p); return cudaGetLastError();)
+    case 0: BDS_DISPATCH_N(N, launch_pdl(k_reduce_tok<float, float, NN>, blocks, 256, 0, s, p); return cudaGetLastError();)
+    case 1: BDS_DISPATCH_N(N, launch_pdl(k_reduce_tok<bf16, bf16, NN>, blocks, 256, 0, s, p); return cudaGetLastError();)
+    default: BDS_DISPATCH_N(N, launch_pdl(k_reduce_tok<bf16, float, NN>, blocks, 256, 0, s, p); return cudaGetLastError();)
   }
 }
 
 cudaError_t launch_bwd_reduce_par(int N, const BwdParams& p, cudaStream_t s) {
   const int64_t npar4 = (p.g.D * N + p.g.D) / 4;  // float4 columns
-  BDS_DISPATCH_N(N, k_reduce_par<NN><<<(unsigned)((npar4 + 31) / 32), 32 * kParSlices, 0, s>>>(p);
+  BDS_DISPATCH_N(N, launch_pdl(k_reduce_par<NN>, (unsigned)((npar4 + 31) / 32), 32 * kParSlices, 0, s, p);
                  return cudaGetLastError();)
 }
 

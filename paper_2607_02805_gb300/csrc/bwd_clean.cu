@@ -26,6 +26,7 @@ struct CleanBwdSmem {
 
 template <typename T, typename TO, int N, bool TILED>
 __global__ void __launch_bounds__(kCta, 3) k_bwd_clean(const BwdParams p) {
+  pdl_sync();
   extern __shared__ __align__(16) unsigned char smem[];
   using L = CleanBwdSmem<T, N>;
   const Geo& g = p.g;
@@ -227,7 +228,7 @@ cudaError_t bwd_clean_tt(const BwdParams& p_in, cudaStream_t s) {
   e = set_bwd_attrs(k_bwd_clean<T, TO, N, TILED>, l.smem);
   if (e != cudaSuccess) return e;
   dim3 grid((unsigned)p.g.G, (unsigned)p.g.nc, (unsigned)p.g.Bt);
-  k_bwd_clean<T, TO, N, TILED><<<grid, kCta, l.smem, s>>>(p);
+  launch_pdl(k_bwd_clean<T, TO, N, TILED>, grid, kCta, l.smem, s, p);
   return cudaGetLastError();
 }
 template <typename T, typename TO, int N>

@@ -34,6 +34,7 @@ struct NoisyBwdSmem {
 // one of the three parts of its work, none of which reads what another makes.
 template <typename T, typename TO, int N, bool TILED, bool SPLIT>
 __global__ void __launch_bounds__(kCta, 1) k_bwd_noisy(const BwdParams p) {
+  pdl_sync();
   static_assert(!(TILED && SPLIT), "a split launch has one block per CTA");
   extern __shared__ __align__(16) unsigned char smem[];
   using L = NoisyBwdSmem<T, N>;
@@ -313,7 +314,7 @@ cudaError_t bwd_noisy_tt(const BwdParams& p_in, cudaStream_t s) {
   e = set_bwd_attrs(k_bwd_noisy<T, TO, N, TILED, SPLIT>, l.smem);
   if (e != cudaSuccess) return e;
   dim3 grid((unsigned)p.g.G, (unsigned)p.g.nc, (unsigned)(SPLIT ? 3 * p.g.Bt : p.g.Bt));
-  k_bwd_noisy<T, TO, N, TILED, SPLIT><<<grid, kCta, l.smem, s>>>(p);
+  launch_pdl(k_bwd_noisy<T, TO, N, TILED, SPLIT>, grid, kCta, l.smem, s, p);
   return cudaGetLastError();
 }
 template <typename T, typename TO, int N>

@@ -43,6 +43,7 @@ constexpr int kScanSeg = 16;
 // run-time stride and half the unroll).
 template <typename T, int N, bool REV>
 __global__ void __launch_bounds__(kCta) k_chunk_local(const FwdParams p) {
+  pdl_sync();
   extern __shared__ __align__(16) unsigned char smem[];
   const Geo& g = p.g;
   const int64_t b = blockIdx.z;
@@ -108,6 +109,7 @@ __global__ void __launch_bounds__(kCta) k_chunk_local(const FwdParams p) {
 constexpr int kCarryW = 64, kCarryRows = 16, kCarryStages = 4;
 template <int N>
 __global__ void __launch_bounds__(kCarryW) k_chunk_carry(const FwdParams p) {
+  pdl_sync();
   constexpr int CH = kCarryW / N;        // channels of the CTA's elements
   constexpr int HQ = kCarryW / 4, SQ = CH / 4;  // 16-byte pieces of one row of states, of dt sums
   __shared__ __align__(16) float hbuf[kCarryStages][kCarryRows][kCarryW];
@@ -186,6 +188,7 @@ struct ScanLayout {
 // mode 1: 545 us with four, 528 with five, 520 with six, 610 with seven).
 template <typename T, typename TO, int N, int MODE, bool TILED>
 __global__ void __launch_bounds__(kCta, MODE == 0 ? 4 : 6) k_block_scan(const FwdParams p) {
+  pdl_sync();
   using Ly = ScanLayout<MODE>;
   extern __shared__ __align__(16) unsigned char smem[];
   const Geo& g = p.g;
@@ -367,6 +370,7 @@ struct ActiveLayout {
 // the output is x + gate * y_n. The seed, the cache, is never modulated.
 template <typename T, typename TO, int N, bool ADA = false>
 __global__ void __launch_bounds__(2 * kActW, 1) k_active_block(const FwdParams p) {
+  pdl_sync();
   using Ly = ActiveLayout<T, N>;
   extern __shared__ __align__(16) unsigned char smem[];
   const Geo& g = p.g;
@@ -479,6 +483,7 @@ __global__ void __launch_bounds__(2 * kActW, 1) k_active_block(const FwdParams p
 // mean, then 1/sqrt(var + eps) from the centred second moment, in fp32.
 template <typename T>
 __global__ void __launch_bounds__(256) k_ln_stats(const T* h, int64_t rows, int64_t D, float eps, float2* stats) {
+  pdl_sync();
   const int64_t row = (int64_t)blockIdx.x * 8 + (threadIdx.x >> 5);
   const int lane = threadIdx.x & 31;
   if (row >= rows) return;
@@ -504,6 +509,7 @@ __global__ void __launch_bounds__(256) k_ln_stats(const T* h, int64_t rows, int6
 // ---------------------------------------------------------------------------
 template <typename TO>
 __global__ void __launch_bounds__(256) k_combine(const float* yf, const float* yr, TO* y, int64_t n4) {
+  pdl_sync();
   const int64_t i = (int64_t)blockIdx.x * 256 + threadIdx.x;  // four elements each
   if (i >= n4) return;
   const float4 a = reinterpret_cast<const float4*>(yf)[i], r = reinterpret_cast<const float4*>(yr)[i];
@@ -526,7 +532,7 @@ cudaError_t chunk_local_rt(const FwdParams& p, cudaStream_t s) {
       cudaFuncSetAttribute(k_chunk_local<T, N, REV>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
   if (e != cudaSuccess) return e;
   dim3 grid((unsigned)p.g.G, (unsigned)p.g.nc_full, (unsigned)p.g.Bt);
-  k_chunk_local<T, N, REV><<<grid, kCta, smem, s>>>(p);
+  launch_pdl(k_chunk_local<T, N, REV>, grid, kCta, smem, s, p);
   return cudaGetLastError();
 }
 template <typename T, int N>
@@ -565,12 +571,12 @@ cudaError_t block_scan_t(int nchunks, const FwdParams& p_in, cudaStream_t s) {
     cudaError_t e = cudaFuncSetAttribute(k_block_scan<T, TO, N, MODE, true>,
                                          cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
     if (e != cudaSuccess) return e;
-    k_block_scan<T, TO, N, MODE, true><<<grid, kCta, smem, s>>>(p);
+    launch_pdl(k_block_scan<T, TO, N, MODE, true>, grid, kCta, smem, s, p);
   } else {
     cudaError_t e = cudaFuncSetAttribute(k_block_scan<T, TO, N, MODE, false>,
                                          cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
     if (e != cudaSuccess) return e;
-    k_block_scan<T, TO, N, MODE, false><<<grid, kCta, smem, s>>>(p);
+    launch_pdl(k_block_scan<T, TO, N, MODE, false>, grid, kCta, smem, s, p);
   }
   return cudaGetLastError();
 }
@@ -595,7 +601,7 @@ cudaError_t active_block_t(const FwdParams& p, cudaStream_t s) {
     if (e != cudaSuccess) return e;
   }
   dim3 grid((unsigned)((p.g.D + kActW - 1) / kActW * p.g.nb), (unsigned)p.g.Bt);
-  k_active_block<T, TO, N, ADA><<<grid, 2 * kActW, smem, s>>>(p);
+  launch_pdl(k_active_block<T, TO, N, ADA>, grid, 2 * kActW, smem, s, p);
   return cudaGetLastError();
 }
 
@@ -619,7 +625,7 @@ cudaError_t launch_chunk_local(int dt, int N, const FwdParams& p, cudaStream_t s
 cudaError_t launch_chunk_carry(int N, const FwdParams& p, cudaStream_t s) {
   if (p.g.Bt * p.g.D * N == 0) return cudaSuccess;
   const dim3 grid((unsigned)((p.g.D * N + kCarryW - 1) / kCarryW), (unsigned)p.g.Bt);
-  BDS_DISPATCH_N(N, k_chunk_carry<NN><<<grid, kCarryW, 0, s>>>(p); return cudaGetLastError();)
+  BDS_DISPATCH_N(N, launch_pdl(k_chunk_carry<NN>, grid, kCarryW, 0, s, p); return cudaGetLastError();)
 }
 
 cudaError_t launch_block_scan(int dt, int N, int mode, int nchunks, const FwdParams& p, cudaStream_t s) {
@@ -653,9 +659,9 @@ cudaError_t launch_ln_stats(int dt, const void* h, int64_t rows, int64_t D, floa
   if (rows == 0) return cudaSuccess;
   const unsigned blocks = (unsigned)((rows + 7) / 8);
   if (dt == 0)
-    k_ln_stats<float><<<blocks, 256, 0, s>>>(reinterpret_cast<const float*>(h), rows, D, eps, stats);
+    launch_pdl(k_ln_stats<float>, blocks, 256, 0, s, reinterpret_cast<const float*>(h), rows, D, eps, stats);
   else
-    k_ln_stats<bf16><<<blocks, 256, 0, s>>>(reinterpret_cast<const bf16*>(h), rows, D, eps, stats);
+    launch_pdl(k_ln_stats<bf16>, blocks, 256, 0, s, reinterpret_cast<const bf16*>(h), rows, D, eps, stats);
   return cudaGetLastError();
 }
 
@@ -664,9 +670,9 @@ cudaError_t launch_combine(int out_f32, const float* yf, const float* yr, void* 
   if (n4 == 0) return cudaSuccess;
   const unsigned blocks = (unsigned)((n4 + 255) / 256);
   if (out_f32)
-    k_combine<float><<<blocks, 256, 0, s>>>(yf, yr, reinterpret_cast<float*>(y), n4);
+    launch_pdl(k_combine<float>, blocks, 256, 0, s, yf, yr, reinterpret_cast<float*>(y), n4);
   else
-    k_combine<bf16><<<blocks, 256, 0, s>>>(yf, yr, reinterpret_cast<bf16*>(y), n4);
+    launch_pdl(k_combine<bf16>, blocks, 256, 0, s, yf, yr, reinterpret_cast<bf16*>(y), n4);
   return cudaGetLastError();
 }
 

@@ -17,6 +17,7 @@ namespace {
 // element type of both.
 template <typename T>
 __global__ void __launch_bounds__(256) k_group_gather(const T* src, int64_t rows, int N, int n0, int gs, T* dst) {
+  pdl_sync();
   const int64_t i = (int64_t)blockIdx.x * 256 + threadIdx.x;
   if (i >= rows * gs) return;
   const int64_t r = i / gs;
@@ -27,6 +28,7 @@ __global__ void __launch_bounds__(256) k_group_gather(const T* src, int64_t rows
 // dst[r][n0 + k] = src[r][k] (fp32 to the output type) for k < gs, n0 + k < N.
 template <typename TO>
 __global__ void __launch_bounds__(256) k_group_scatter(const float* src, int64_t rows, int N, int n0, int gs, TO* dst) {
+  pdl_sync();
   const int64_t i = (int64_t)blockIdx.x * 256 + threadIdx.x;
   if (i >= rows * gs) return;
   const int64_t r = i / gs;
@@ -36,6 +38,7 @@ __global__ void __launch_bounds__(256) k_group_scatter(const float* src, int64_t
 
 // acc += add (fp32)
 __global__ void __launch_bounds__(256) k_group_add(float* acc, const float* add, int64_t n) {
+  pdl_sync();
   const int64_t i = (int64_t)blockIdx.x * 256 + threadIdx.x;
   if (i < n) acc[i] = __fadd_rn(acc[i], add[i]);
 }
@@ -43,6 +46,7 @@ __global__ void __launch_bounds__(256) k_group_add(float* acc, const float* add,
 // out = acc in the output type
 template <typename TO>
 __global__ void __launch_bounds__(256) k_group_out(const float* acc, TO* out, int64_t n) {
+  pdl_sync();
   const int64_t i = (int64_t)blockIdx.x * 256 + threadIdx.x;
   if (i < n) out[i] = to_out<TO>(acc[i]);
 }
@@ -55,9 +59,9 @@ cudaError_t launch_group_gather(const void* src, int elt, int64_t rows, int N, i
                                 cudaStream_t s) {
   if (rows * gs == 0) return cudaSuccess;
   if (elt == 2)
-    k_group_gather<bf16><<<nblk(rows * gs), 256, 0, s>>>((const bf16*)src, rows, N, n0, gs, (bf16*)dst);
+    launch_pdl(k_group_gather<bf16>, nblk(rows * gs), 256, 0, s, (const bf16*)src, rows, N, n0, gs, (bf16*)dst);
   else
-    k_group_gather<float><<<nblk(rows * gs), 256, 0, s>>>((const float*)src, rows, N, n0, gs, (float*)dst);
+    launch_pdl(k_group_gather<float>, nblk(rows * gs), 256, 0, s, (const float*)src, rows, N, n0, gs, (float*)dst);
   return cudaGetLastError();
 }
 
@@ -65,24 +69,24 @@ cudaError_t launch_group_scatter(const float* src, int64_t rows, int N, int n0, 
                                  cudaStream_t s) {
   if (rows * gs == 0) return cudaSuccess;
   if (out_elt == 2)
-    k_group_scatter<bf16><<<nblk(rows * gs), 256, 0, s>>>(src, rows, N, n0, gs, (bf16*)dst);
+    launch_pdl(k_group_scatter<bf16>, nblk(rows * gs), 256, 0, s, src, rows, N, n0, gs, (bf16*)dst);
   else
-    k_group_scatter<float><<<nblk(rows * gs), 256, 0, s>>>(src, rows, N, n0, gs, (float*)dst);
+    launch_pdl(k_group_scatter<float>, nblk(rows * gs), 256, 0, s, src, rows, N, n0, gs, (float*)dst);
   return cudaGetLastError();
 }
 
 cudaError_t launch_group_add(float* acc, const float* add, int64_t n, cudaStream_t s) {
   if (n == 0) return cudaSuccess;
-  k_group_add<<<nblk(n), 256, 0, s>>>(acc, add, n);
+  launch_pdl(k_group_add, nblk(n), 256, 0, s, acc, add, n);
   return cudaGetLastError();
 }
 
 cudaError_t launch_group_out(const float* acc, void* out, int out_elt, int64_t n, cudaStream_t s) {
   if (n == 0) return cudaSuccess;
   if (out_elt == 2)
-    k_group_out<bf16><<<nblk(n), 256, 0, s>>>(acc, (bf16*)out, n);
+    launch_pdl(k_group_out<bf16>, nblk(n), 256, 0, s, acc, (bf16*)out, n);
   else
-    k_group_out<float><<<nblk(n), 256, 0, s>>>(acc, (float*)out, n);
+    launch_pdl(k_group_out<float>, nblk(n), 256, 0, s, acc, (float*)out, n);
   return cudaGetLastError();
 }
 

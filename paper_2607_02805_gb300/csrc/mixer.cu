@@ -206,6 +206,7 @@ constexpr size_t prep_smem() {
 template <typename T>
 __global__ void __launch_bounds__(kPrepCta, 4) k_mix_prep(const MixIn<T> a, float* x_c, float* dt_c, float* x_n,
                                                        float* dt_f, float* dt_r, int Ls) {
+  pdl_sync();
   extern __shared__ __align__(16) unsigned char smem[];
   constexpr int Q = 4, S = 4, W1 = kW - 1;
   const int64_t d = ((int64_t)blockIdx.y * blockDim.x + threadIdx.x) * Q, b = blockIdx.z;
@@ -318,6 +319,7 @@ __global__ void __launch_bounds__(32 * kBwdGroups, 2)
     k_mix_bwd(const MixIn<T> a, const float* gx_c, const float* gdt_c, const float* gx_n, const float* gdt_f,
               const float* gdt_r, TO* dxr_c, TO* ddtr_c, TO* dxr_n, TO* ddtr_f, TO* ddtr_r, int Ls, int nseg,
               float* part) {
+  pdl_sync();
   extern __shared__ __align__(16) unsigned char smem[];
   constexpr int Q = 2, W1 = kW - 1, S = 4, TH = 32 * kBwdGroups;
   __shared__ float red[kBwdGroups][kW + 3][32 * Q];
@@ -480,6 +482,7 @@ __global__ void __launch_bounds__(32 * kBwdGroups, 2)
 // The slices summed in order: dconv_w [D][4], dconv_b, ddt_bias_f, ddt_bias_r [D].
 __global__ void __launch_bounds__(256) k_mix_par_red(int64_t D, int slices, const float* part, float* dw, float* db,
                                                      float* dbf, float* dbr) {
+  pdl_sync();
   const int64_t i = (int64_t)blockIdx.x * 256 + threadIdx.x;
   if (i >= D * (kW + 3)) return;
   const int v = (int)(i / D);
@@ -500,6 +503,7 @@ __global__ void __launch_bounds__(256) k_mix_par_red(int64_t D, int slices, cons
 // out = y * SiLU(z), V elements per thread.
 template <typename T, typename TO>
 __global__ void __launch_bounds__(256) k_mix_gate(int64_t n, const float* y, const T* z, TO* out) {
+  pdl_sync();
   constexpr int V = Vec<T>::V;
   const int64_t i = ((int64_t)blockIdx.x * 256 + threadIdx.x) * V;
   if (i >= n) return;
@@ -516,6 +520,7 @@ __global__ void __launch_bounds__(256) k_mix_gate(int64_t n, const float* y, con
 template <typename T, typename TO>
 __global__ void __launch_bounds__(256) k_mix_gate_bwd(int64_t n, const float* y, const T* z, const T* dout, float* dy,
                                                       TO* dz) {
+  pdl_sync();
   constexpr int V = Vec<T>::V;
   const int64_t i = ((int64_t)blockIdx.x * 256 + threadIdx.x) * V;
   if (i >= n) return;
@@ -546,6 +551,7 @@ struct CvtSet {
 };
 template <typename TI, typename TO>
 __global__ void __launch_bounds__(256) k_mix_cvt(int64_t n, const __grid_constant__ CvtSet c) {
+  pdl_sync();
   const int64_t i = ((int64_t)blockIdx.x * 256 + threadIdx.x) * 4;
   if (i >= n) return;
   float v[4];
@@ -557,6 +563,7 @@ __global__ void __launch_bounds__(256) k_mix_cvt(int64_t n, const __grid_constan
 // before each emitted boundary (every block end, or the end of the stream).
 template <typename T>
 __global__ void __launch_bounds__(256) k_mix_conv_states(const MixIn<T> a, int emit_all, float* cs) {
+  pdl_sync();
   const int64_t nS = emit_all ? a.L / a.Bs : 1;
   const int64_t i = (int64_t)blockIdx.x * 256 + threadIdx.x;
   if (i >= a.Bt * nS * (kW - 1) * a.D) return;
@@ -670,7 +677,7 @@ MixIn<T> mix_in(const Geo& g, const bdscan_clean* c, const bdscan_noisy* n, cons
 
 template <typename TI, typename TO>
 cudaError_t cvt_all(const CvtSet& c, int count, int64_t n, cudaStream_t s) {
-  k_mix_cvt<TI, TO><<<dim3((unsigned)((n / 4 + 255) / 256), (unsigned)count), 256, 0, s>>>(n, c);
+  launch_pdl(k_mix_cvt<TI, TO>, dim3((unsigned)((n / 4 + 255) / 256), (unsigned)count), 256, 0, s, n, c);
   return api_launched(cudaGetLastError(), s);
 }
 // B and C of the given streams converted to fp32 into the workspace slots.
@@ -703,7 +710,7 @@ cudaError_t prep(const Geo& g, const MixIn<T>& a, float* x_c, float* dt_c, float
   const int Ls = sweep_len([&](int ls) { return g.Bt * tiles * runs(ls); });
   cudaError_t e = set_smem_cached((const void*)k_mix_prep<T>, (int)prep_smem<T>(), -1);
   if (e != cudaSuccess) return e;
-  k_mix_prep<T><<<dim3(runs(Ls), tiles, (unsigned)g.Bt), dim3(tx, ty), prep_smem<T>(), s>>>(a, x_c, dt_c, x_n, dt_f,
+  launch_pdl(k_mix_prep<T>, dim3(runs(Ls), tiles, (unsigned)g.Bt), dim3(tx, ty), prep_smem<T>(), s, a, x_c, dt_c, x_n, dt_f,
                                                                                            dt_r, Ls);
   return api_launched(cudaGetLastError(), s);
 }
@@ -748,7 +755,7 @@ cudaError_t mix_forward_core(const Geo& g, int N, const bdscan_clean* cl, const 
 
 template <typename T, typename TO>
 cudaError_t gate(int64_t n, const char* ws, size_t yslot, const void* z, void* out, cudaStream_t s) {
-  k_mix_gate<T, TO><<<vec_blocks<T>(n), 256, 0, s>>>(n, (const float*)(ws + yslot), (const T*)z, (TO*)out);
+  launch_pdl(k_mix_gate<T, TO>, vec_blocks<T>(n), 256, 0, s, n, (const float*)(ws + yslot), (const T*)z, (TO*)out);
   return api_launched(cudaGetLastError(), s);
 }
 
@@ -777,11 +784,11 @@ cudaError_t mix_backward_t(const Geo& g, int N, const bdscan_clean* cl, const vo
   if (e != cudaSuccess) return e;
   const int64_t n = g.Bt * g.L * g.D, nn = g.Bt * g.L * N;
   float* dy[2] = {(float*)(ws + w.dy[0]), (float*)(ws + w.dy[1])};
-  k_mix_gate_bwd<T, TO><<<vec_blocks<T>(n), 256, 0, s>>>(n, (const float*)(ws + w.y[0]), (const T*)z_c, (const T*)dout_c,
+  launch_pdl(k_mix_gate_bwd<T, TO>, vec_blocks<T>(n), 256, 0, s, n, (const float*)(ws + w.y[0]), (const T*)z_c, (const T*)dout_c,
                                                      dy[0], (TO*)dz_c);
   e = api_launched(cudaGetLastError(), s);
   if (e != cudaSuccess) return e;
-  k_mix_gate_bwd<T, TO><<<vec_blocks<T>(n), 256, 0, s>>>(n, (const float*)(ws + w.y[1]), (const T*)z_n, (const T*)dout_n,
+  launch_pdl(k_mix_gate_bwd<T, TO>, vec_blocks<T>(n), 256, 0, s, n, (const float*)(ws + w.y[1]), (const T*)z_n, (const T*)dout_n,
                                                      dy[1], (TO*)dz_n);
   e = api_launched(cudaGetLastError(), s);
   if (e != cudaSuccess) return e;
@@ -835,7 +842,7 @@ cudaError_t mix_backward_t(const Geo& g, int N, const bdscan_clean* cl, const vo
   const int64_t want = ctas(Ls);
   const int slices = (int)(want < kParSplit ? want : kParSplit);
   if ((e = set_smem_cached((const void*)k_mix_bwd<T, TO>, (int)mix_bwd_smem<T>(), -1)) != cudaSuccess) return e;
-  k_mix_bwd<T, TO><<<dim3((unsigned)slices, (unsigned)tiles), dim3(32, kBwdGroups), mix_bwd_smem<T>(), s>>>(
+  launch_pdl(k_mix_bwd<T, TO>, dim3((unsigned)slices, (unsigned)tiles), dim3(32, kBwdGroups), mix_bwd_smem<T>(), s, 
       a, G[0], G[1], G[2], G[3], G[4], (TO*)gc->dx, (TO*)gc->ddt, (TO*)gn->dx, (TO*)gn->ddt_f, (TO*)gn->ddt_r, Ls,
       (int)((g.L + Ls - 1) / Ls), part);
   e = api_launched(cudaGetLastError(), s);
@@ -847,7 +854,7 @@ cudaError_t mix_backward_t(const Geo& g, int N, const bdscan_clean* cl, const vo
     cv.dst[i] = gbc_out[i];
   }
   if ((e = cvt_all<float, TO>(cv, 6, nn, s)) != cudaSuccess) return e;
-  k_mix_par_red<<<blocks_of(g.D * (kW + 3)), 256, 0, s>>>(g.D, slices, part, gm->dconv_w, gm->dconv_b, gm->ddt_bias_f,
+  launch_pdl(k_mix_par_red, blocks_of(g.D * (kW + 3)), 256, 0, s, g.D, slices, part, gm->dconv_w, gm->dconv_b, gm->ddt_bias_f,
                                                           gm->ddt_bias_r);
   return api_launched(cudaGetLastError(), s);
 }
@@ -881,7 +888,7 @@ cudaError_t mix_boundary_t(const Geo& g, int N, const bdscan_clean* cl, const vo
   if (e == cudaSuccess && out_c != nullptr) e = gate<T, TO>(n, ws, w.y[0], z_c, out_c, s);
   if (e != cudaSuccess) return e;
   const int64_t nc = g.Bt * (emit_all ? g.nb : 1) * (kW - 1) * g.D;
-  k_mix_conv_states<T><<<blocks_of(nc), 256, 0, s>>>(a, emit_all, conv_states);
+  launch_pdl(k_mix_conv_states<T>, blocks_of(nc), 256, 0, s, a, emit_all, conv_states);
   return api_launched(cudaGetLastError(), s);
 }
 

@@ -69,6 +69,7 @@ constexpr int kStateIssuer = 64;  // the thread that issues a head's MMAs (k_ssd
 // written out (two accumulators, TMEM columns 0..63 and 64..127).
 template <int N>
 __global__ void __launch_bounds__(kStateThreads, 1) k_ssd_block_state(const SsdStateParams p) {
+  pdl_sync();
   extern __shared__ unsigned char smraw[];
   unsigned char* sm = align1024(smraw);
   __shared__ uint64_t bar[2];
@@ -212,6 +213,7 @@ __global__ void __launch_bounds__(kStateThreads, 1) k_ssd_block_state(const SsdS
 
 // One thread per (batch row, head, channel, state index), sequential in k.
 __global__ void __launch_bounds__(256) k_ssd_state_pass(const SsdPassParams p) {
+  pdl_sync();
   const SsdGeo& g = p.g;
   const int64_t per_b = (int64_t)g.H * kSsdP * g.N;
   const int64_t idx = (int64_t)blockIdx.x * 256 + threadIdx.x;
@@ -381,6 +383,7 @@ __device__ __forceinline__ void setup_dir(const T* dt, int hs, int n, float A2, 
 template <int N, bool NOISY>
 __global__ void __launch_bounds__(kScanThreads, 1) k_ssd_block_scan(const SsdScanParams p,
                                                                     const __grid_constant__ CUtensorMap xmap) {
+  pdl_sync();
   extern __shared__ unsigned char smraw[];
   unsigned char* sm = align1024(smraw);
   __shared__ uint64_t bar[3];  // [0]: a head's MMAs, [1]: the Gram products, [2]: a head's loads (TMA)
@@ -803,10 +806,10 @@ cudaError_t launch_ssd_block_state(const SsdStateParams& p, cudaStream_t s) {
   cudaError_t e;
   if (p.g.N == 64) {
     if ((e = set_smem(k_ssd_block_state<64>, bytes)) != cudaSuccess) return e;
-    k_ssd_block_state<64><<<grid, kStateThreads, bytes, s>>>(p);
+    launch_pdl(k_ssd_block_state<64>, grid, kStateThreads, bytes, s, p);
   } else {
     if ((e = set_smem(k_ssd_block_state<128>, bytes)) != cudaSuccess) return e;
-    k_ssd_block_state<128><<<grid, kStateThreads, bytes, s>>>(p);
+    launch_pdl(k_ssd_block_state<128>, grid, kStateThreads, bytes, s, p);
   }
   return cudaGetLastError();
 }
@@ -814,7 +817,7 @@ cudaError_t launch_ssd_block_state(const SsdStateParams& p, cudaStream_t s) {
 cudaError_t launch_ssd_state_pass(const SsdPassParams& p, cudaStream_t s) {
   const int64_t n = p.g.Bt * p.g.H * kSsdP * p.g.N;
   if (n == 0) return cudaSuccess;
-  k_ssd_state_pass<<<(unsigned)((n + 255) / 256), 256, 0, s>>>(p);
+  launch_pdl(k_ssd_state_pass, (unsigned)((n + 255) / 256), 256, 0, s, p);
   return cudaGetLastError();
 }
 
@@ -869,7 +872,7 @@ cudaError_t scan_t(const SsdScanParams& p_in, cudaStream_t s) {
   // streams read right to left keep the cp.async path (a box cannot reverse rows)
   p.tma = !p.rev && encode_head_map(&xmap, p.x, p.g.Bt * p.g.L, p.g.H) ? 1 : 0;
   const dim3 grid((unsigned)tiles, (unsigned)((p.g.H + p.hg - 1) / p.hg));
-  k_ssd_block_scan<N, NOISY><<<grid, kScanThreads, L.total, s>>>(p, xmap);
+  launch_pdl(k_ssd_block_scan<N, NOISY>, grid, kScanThreads, L.total, s, p, xmap);
   return cudaGetLastError();
 }
 

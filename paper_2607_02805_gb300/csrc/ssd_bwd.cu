@@ -179,6 +179,7 @@ template <int N, bool UPPER, bool SEED>
 __global__ void __launch_bounds__(kTileThreads, 1) k_ssd_bwd_tile(const SsdBwdTileParams p,
                                                                   const __grid_constant__ CUtensorMap xmap,
                                                                   const __grid_constant__ CUtensorMap dymap) {
+  pdl_sync();
   extern __shared__ unsigned char smraw[];
   unsigned char* sm = align1024(smraw);
   __shared__ uint64_t bar, bar_ld;  // MMAs; a head's x and dy tiles (TMA)
@@ -690,6 +691,7 @@ __device__ __forceinline__ void warp_scan_f32(float* a, int n) {
 // rowdot_t), ddt_r = colsum'_r + sum of dc over the tokens whose cumulative dt
 // includes dt_r (t >= r forward, t <= r reverse), dA = sum_t c_t (dc_t / A).
 __global__ void __launch_bounds__(128) k_ssd_bwd_vec(const SsdBwdVecParams p) {
+  pdl_sync();
   __shared__ float s_c[4][256], s_q[4][256], s_col[4][256];
   const SsdGeo& g = p.g;
   const int w = threadIdx.x >> 5, lane = threadIdx.x & 31, Bs = (int)g.Bs, m = g.m, H = g.H;
@@ -734,6 +736,7 @@ __global__ void __launch_bounds__(128) k_ssd_bwd_vec(const SsdBwdVecParams p) {
 
 // One thread per (batch row, head, channel, state index), blocks last to first.
 __global__ void __launch_bounds__(256) k_ssd_bwd_pass(const SsdBwdPassParams p) {
+  pdl_sync();
   const SsdGeo& g = p.g;
   const int64_t PN = (int64_t)kSsdP * g.N, per_b = (int64_t)g.H * PN;
   const int64_t idx = (int64_t)blockIdx.x * 256 + threadIdx.x;
@@ -800,6 +803,7 @@ struct StateBwdSmem {
 // the block decay.
 template <int N>
 __global__ void __launch_bounds__(kBwdThreads, 1) k_ssd_bwd_state(const SsdBwdStateParams p) {
+  pdl_sync();
   extern __shared__ unsigned char smraw[];
   unsigned char* sm = align1024(smraw);
   __shared__ uint64_t bar;
@@ -992,6 +996,7 @@ __global__ void __launch_bounds__(256) k_ssd_bwd_dx(const SsdGeo g, const float*
                                                     const float* dxp_f, const float* dxp_r, const __nv_bfloat16* dyc,
                                                     const __nv_bfloat16* dyn, const float* Df, const float* Dr,
                                                     __nv_bfloat16* dxc, __nv_bfloat16* dxn) {
+  pdl_sync();
   constexpr int Q = kSsdP / 4;  // 4-channel groups per head
   const int64_t i = (int64_t)blockIdx.x * 256 + threadIdx.x;
   if (i >= g.Bt * g.L * g.H * Q) return;
@@ -1038,6 +1043,7 @@ __global__ void __launch_bounds__(256) k_ssd_bwd_dbc(const SsdGeo g, int ngrp, c
                                                      const float* dBp_r, const float* dCp_r, __nv_bfloat16* dBc,
                                                      __nv_bfloat16* dCc, __nv_bfloat16* dBf, __nv_bfloat16* dCf,
                                                      __nv_bfloat16* dBr, __nv_bfloat16* dCr) {
+  pdl_sync();
   const int N = g.N, m = g.m, Q = N / 4;
   const int64_t i = (int64_t)blockIdx.x * 256 + threadIdx.x;
   if (i >= g.Bt * g.L * Q) return;
@@ -1089,6 +1095,7 @@ __global__ void __launch_bounds__(256) k_ssd_bwd_par(const SsdGeo g, const float
                                                      const float* dA_c, const float* dA_f, const float* dA_s,
                                                      const float* dA_r, float* dAf, float* dDf, float* dAr,
                                                      float* dDr) {
+  pdl_sync();
   __shared__ float4 red[256];
   const int h = blockIdx.x, t = threadIdx.x, nd = g.m * 8;
   float af = 0.f, ar = 0.f, df = 0.f, dr = 0.f;
@@ -1136,7 +1143,7 @@ cudaError_t bwd_tile_t(const SsdBwdTileParams& p_in, cudaStream_t s) {
               ? 1
               : 0;
   dim3 grid((unsigned)(p.g.Bt * p.g.nb * p.g.m), (unsigned)((p.g.H + p.hg - 1) / p.hg));
-  k_ssd_bwd_tile<N, UPPER, SEED><<<grid, kTileThreads, smem, s>>>(p, xmap, dymap);
+  launch_pdl(k_ssd_bwd_tile<N, UPPER, SEED>, grid, kTileThreads, smem, s, p, xmap, dymap);
   return cudaGetLastError();
 }
 
@@ -1146,7 +1153,7 @@ cudaError_t bwd_state_t(const SsdBwdStateParams& p, cudaStream_t s) {
   cudaError_t e = set_smem_cached((const void*)k_ssd_bwd_state<N>, smem, -1);
   if (e != cudaSuccess) return e;
   dim3 grid((unsigned)(p.g.Bt * p.g.nb), (unsigned)p.g.H);
-  k_ssd_bwd_state<N><<<grid, kBwdThreads, smem, s>>>(p);
+  launch_pdl(k_ssd_bwd_state<N>, grid, kBwdThreads, smem, s, p);
   return cudaGetLastError();
 }
 
@@ -1163,13 +1170,13 @@ cudaError_t launch_ssd_bwd_tile(bool upper, bool seeded, const SsdBwdTileParams&
 
 cudaError_t launch_ssd_bwd_vec(const SsdBwdVecParams& p, cudaStream_t s) {
   const int64_t warps = p.g.Bt * p.g.nb * p.g.H;
-  k_ssd_bwd_vec<<<(unsigned)((warps + 3) / 4), 128, 0, s>>>(p);
+  launch_pdl(k_ssd_bwd_vec, (unsigned)((warps + 3) / 4), 128, 0, s, p);
   return cudaGetLastError();
 }
 
 cudaError_t launch_ssd_bwd_pass(const SsdBwdPassParams& p, cudaStream_t s) {
   const int64_t n = p.g.Bt * p.g.H * kSsdP * p.g.N;
-  k_ssd_bwd_pass<<<(unsigned)((n + 255) / 256), 256, 0, s>>>(p);
+  launch_pdl(k_ssd_bwd_pass, (unsigned)((n + 255) / 256), 256, 0, s, p);
   return cudaGetLastError();
 }
 
@@ -1182,7 +1189,7 @@ cudaError_t launch_ssd_bwd_dx(const SsdGeo& g, const float* dxp_c, const float* 
                               const float* Dr, __nv_bfloat16* dxc, __nv_bfloat16* dxn, cudaStream_t s) {
   const int64_t n = g.Bt * g.L * g.H * (kSsdP / 4);
   if (n == 0) return cudaSuccess;
-  k_ssd_bwd_dx<<<(unsigned)((n + 255) / 256), 256, 0, s>>>(g, dxp_c, dxs, dxp_f, dxp_r, dyc, dyn, Df, Dr, dxc, dxn);
+  launch_pdl(k_ssd_bwd_dx, (unsigned)((n + 255) / 256), 256, 0, s, g, dxp_c, dxs, dxp_f, dxp_r, dyc, dyn, Df, Dr, dxc, dxn);
   return cudaGetLastError();
 }
 
@@ -1192,7 +1199,7 @@ cudaError_t launch_ssd_bwd_dbc(const SsdGeo& g, int ngrp, const float* dBp_c, co
                                __nv_bfloat16* dBr, __nv_bfloat16* dCr, cudaStream_t s) {
   const int64_t n = g.Bt * g.L * (g.N / 4);
   if (n == 0) return cudaSuccess;
-  k_ssd_bwd_dbc<<<(unsigned)((n + 255) / 256), 256, 0, s>>>(g, ngrp, dBp_c, dBs, dCp_c, dBp_f, dCp_f, dBp_r, dCp_r, dBc,
+  launch_pdl(k_ssd_bwd_dbc, (unsigned)((n + 255) / 256), 256, 0, s, g, ngrp, dBp_c, dBs, dCp_c, dBp_f, dCp_f, dBp_r, dCp_r, dBc,
                                                               dCc, dBf, dCf, dBr, dCr);
   return cudaGetLastError();
 }
@@ -1200,7 +1207,7 @@ cudaError_t launch_ssd_bwd_dbc(const SsdGeo& g, int ngrp, const float* dBp_c, co
 cudaError_t launch_ssd_bwd_params(const SsdGeo& g, const float* dd_c, const float* dd_n, const float* dA_c,
                                   const float* dA_f, const float* dA_s, const float* dA_r, float* dAf, float* dDf,
                                   float* dAr, float* dDr, cudaStream_t s) {
-  k_ssd_bwd_par<<<(unsigned)g.H, 256, 0, s>>>(g, dd_c, dd_n, dA_c, dA_f, dA_s, dA_r, dAf, dDf, dAr, dDr);
+  launch_pdl(k_ssd_bwd_par, (unsigned)g.H, 256, 0, s, g, dd_c, dd_n, dA_c, dA_f, dA_s, dA_r, dAf, dDf, dAr, dDr);
   return cudaGetLastError();
 }
 

@@ -50,3 +50,31 @@ def test_small_problems_match_oracle(Bt, L, Bs, D, N, dt, od):
     ref = P.oracle_backward(wl, st, use_dstates=True)
     for k, v in lay.g.items():
         P.assert_close("d" + k, to_numpy(v), ref[k], P.GRAD_TOL, 0.0 if k in P.PARAMS else u)
+
+
+def test_back_to_back_small_steps_keep_their_order():
+    """Small launches may be placed before their predecessor has ended; two
+    steps that share every buffer but the inputs, enqueued without a wait,
+    give the bits of the same steps run one at a time."""
+    wls = [Workload(1, 256, 16, 32, 8, dtype="f32", seed=s) for s in (5, 6)]
+    lay = Layer(wls[0])
+    lay.alloc_backward()
+    ins = [lay.t, Layer(wls[1]).t]
+
+    def outputs():
+        return [lay.y_c, lay.y_n, lay.states] + list(lay.g.values())
+
+    def step(t):
+        lay.t = t
+        lay.forward()
+        lay.backward(use_dstates=False)
+
+    step(ins[1])
+    torch.cuda.synchronize()
+    alone = [v.clone() for v in outputs()]
+    torch.cuda.synchronize()
+    for _ in range(20):
+        step(ins[0])
+        step(ins[1])
+    torch.cuda.synchronize()
+    assert all(torch.equal(a, v) for a, v in zip(alone, outputs()))
