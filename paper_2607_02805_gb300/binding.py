@@ -200,7 +200,8 @@ class BdscanError(RuntimeError):
 
 
 def _call(name, *args):
-    lib = load()
+    # a loaded library is never unloaded, so the load lock is only for the first call
+    lib = _libs[_use_debug] or load()
     rc = getattr(lib, name)(*args)
     if rc != BDSCAN_OK:
         raise BdscanError(name, rc, lib.bdscan_last_error().decode())
@@ -410,9 +411,16 @@ def _ptr(t):
 
 
 def _stream(stream):
+    """The CUDA stream handle of `stream`, by default of the current device's
+    current stream (asked for as a raw handle where this PyTorch has the query:
+    0.2 us against 3 us for a Stream object, of an 11 us active-block call)."""
+    if stream is not None:
+        return stream.cuda_stream
     import torch
-    s = torch.cuda.current_stream() if stream is None else stream
-    return s.cuda_stream
+    raw = getattr(torch._C, "_cuda_getCurrentRawStream", None)
+    if raw is not None and torch.cuda.is_initialized():
+        return raw(torch._C._cuda_getDevice())
+    return torch.cuda.current_stream().cuda_stream
 
 
 def _dtype_code(t):
