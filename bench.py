@@ -590,19 +590,23 @@ def run_ssd(args):
         torch.cuda.empty_cache()
 
 
-SSD_BWD_KERNELS = ("bwd_tile_clean", "bwd_tile_fwd", "bwd_tile_rev", "bwd_vec_clean", "bwd_vec_fwd", "bwd_vec_rev",
-                   "bwd_state_pass", "bwd_block_state", "bwd_dx", "bwd_dbc", "bwd_par")
+SSD_BWD_KERNELS = ("bwd_tile_clean", "bwd_tile_fwd", "bwd_tile_rev", "bwd_vec", "bwd_state_pass", "bwd_block_state",
+                   "bwd_dx", "bwd_dbc", "bwd_par")
 
 
 def ssd_bwd_head_groups(Bt, L, Bs, H):
-    """Heads per tile CTA and the number of head groups the backward picks
-    (about 1024 CTAs per launch, at most 16 heads per CTA)."""
+    """Heads per tile CTA and the number of head groups the backward picks: the
+    fewest waves over 152 SMs times (one and a half heads of set-up + heads per
+    CTA), at most 16 heads per CTA."""
     units = Bt * (L // Bs) * (Bs // 128)
-    want = -(-1024 // units) if units > 0 else 1
-    want = min(max(want, -(-H // 16)), H)
-    want = max(want, 1)
-    hg = -(-H // want)
-    return hg, -(-H // hg)
+    best = None
+    for n in range(-(-H // 16), H + 1):
+        per = -(-H // n)
+        groups = -(-H // per)
+        cost = -(-units * groups // 152) * (3 + 2 * per)
+        if best is None or cost < best[0]:
+            best = (cost, per, groups)
+    return best[1:] if best else (1, 1)
 
 
 def ssd_bwd_tile_flops(Bt, L, Bs, H, N, seeded):

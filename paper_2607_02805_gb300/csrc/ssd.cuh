@@ -91,10 +91,9 @@ struct SsdBwdTileParams {
   int tma;              // set by the launcher: x and dy tiles arrive by TMA
 };
 
-// The dt and A gradients of one stream and direction from the row and column
+// The dt and A gradients of each stream and direction from the row and column
 // sums: dc = A (rowsum - dt colsum' + rowdot), then a scan inside the block.
-struct SsdBwdVecParams {
-  SsdGeo g;
+struct SsdBwdVecStream {
   const __nv_bfloat16* dt;
   const float* A;
   const float *col_part, *rowsum, *rowdot;  // rowdot null: zero
@@ -103,6 +102,10 @@ struct SsdBwdVecParams {
   __nv_bfloat16* ddt_out;    // [Bt][L][H] or null: the stream's final dt gradient (no other term adds to it)
   float* dA;                 // [Bt*nb][H]
   float* sumdt;              // [Bt*nb][H] or null: the block's sum of dt
+};
+struct SsdBwdVecParams {
+  SsdGeo g;
+  SsdBwdVecStream s[3];  // clean, noisy forward, noisy reverse
 };
 
 // Reverse pass over the clean stream's block-end states: gS_k = dstates_k +
@@ -116,6 +119,9 @@ struct SsdBwdPassParams {
   float* gS;                 // [Bt][nb][H][P][N]
 };
 
+// Most heads of a k_ssd_bwd_state CTA (its vectors beside 192 KB of operands).
+constexpr int kMaxStateBwdHeads = 13;
+
 // Transpose of the clean block-state product T_k = sum_s w_s x_s B_s^T, and
 // the gradient of the block decay exp(A sumdt_k) S_{k-1}.
 struct SsdBwdStateParams {
@@ -126,7 +132,8 @@ struct SsdBwdStateParams {
   const float* states;  // [Bt][nb][H][P][N]
   const float* sumdt;   // [Bt*nb][H]
   float* dx_state;          // [Bt*nb][H][Bs][P]
-  float* dB_state;          // [Bt*nb][H][Bs][N]
+  float* dB_state;          // [Bt*nb][head groups][Bs][N]
+  int hg;                   // heads per CTA, at most kMaxStateBwdHeads
   const float* ddt_tile;    // [Bt][L][H] the tile side of the clean dt gradient
   __nv_bfloat16* ddt;       // [Bt][L][H] output: ddt_tile + this kernel's terms
   float* dA;                // [Bt*nb][H]
@@ -142,7 +149,8 @@ cudaError_t launch_ssd_bwd_state(const SsdBwdStateParams& p, cudaStream_t s);
 cudaError_t launch_ssd_bwd_dx(const SsdGeo& g, const float* dxp_c, const float* dxs, const float* dxp_f,
                               const float* dxp_r, const __nv_bfloat16* dyc, const __nv_bfloat16* dyn, const float* Df,
                               const float* Dr, __nv_bfloat16* dxc, __nv_bfloat16* dxn, cudaStream_t s);
-cudaError_t launch_ssd_bwd_dbc(const SsdGeo& g, int ngrp, const float* dBp_c, const float* dBs, const float* dCp_c,
+cudaError_t launch_ssd_bwd_dbc(const SsdGeo& g, int ngrp, int ngrp_state, const float* dBp_c, const float* dBs,
+                               const float* dCp_c,
                                const float* dBp_f, const float* dCp_f, const float* dBp_r, const float* dCp_r,
                                __nv_bfloat16* dBc, __nv_bfloat16* dCc, __nv_bfloat16* dBf, __nv_bfloat16* dCf,
                                __nv_bfloat16* dBr, __nv_bfloat16* dCr, cudaStream_t s);

@@ -397,24 +397,36 @@ namespace {
 struct SsdBwdWs {
   size_t dxp[3], dBp[3], dCp[3], colp[3], rows[3], rowdot[3], dSp[3], ddtv[3], dAv[3];
   size_t sumdt, gS, dxs, dBs, dAs, dd, total;
-  int hg, ngrp;  // heads per tile CTA, head groups
+  int hg, ngrp;      // heads per tile CTA, head groups
+  int hg_s, ngrp_s;  // the same of the block-state kernel
 };
-// Head groups of the tile kernel: enough CTAs for about 1024 (several waves
-// over the SMs), at most 16 heads per CTA; a function of the dimensions only,
-// so the workspace size does not depend on the device.
-void ssd_bwd_groups(const bds::SsdGeo& g, int* hg, int* ngrp) {
-  const int64_t units = g.Bt * g.nb * g.m;
-  int64_t want = units > 0 ? (1024 + units - 1) / units : 1;
-  const int64_t lo = (g.H + 15) / 16;
-  if (want < lo) want = lo;
-  if (want > g.H) want = g.H;
-  if (want < 1) want = 1;
-  *hg = (int)((g.H + want - 1) / want);
-  *ngrp = g.H > 0 ? (g.H + *hg - 1) / *hg : 1;
+// Head groups of the tile kernel (units: tiles of 128 tokens, at most 16 heads
+// per CTA) and of the block-state kernel (units: blocks), both one CTA per SM.
+// A CTA pays a set-up of about one and a half heads (operands, the Gram
+// product, the group's dB and dC), so the group count minimises (waves over
+// the 152 SMs this library is written for) x (set-up + heads per CTA); ties
+// keep fewer groups, whose partials the combine reads. A function of the
+// dimensions only, so the workspace size does not depend on the device.
+// 63 tiles of 14 heads: two groups in one wave instead of fourteen in six
+// (tile kernels 93 + 89 + 71 -> 66 + 63 + 40 us, combine 57 -> 16 us).
+void ssd_bwd_groups(const bds::SsdGeo& g, int64_t units, int maxg, int* hg, int* ngrp) {
+  constexpr int64_t kSms = 152;
+  *hg = *ngrp = 1;
+  int64_t best = -1;
+  for (int n = (g.H + maxg - 1) / maxg; n <= g.H; ++n) {
+    const int per = (g.H + n - 1) / n, groups = (g.H + per - 1) / per;
+    const int64_t cost = (units * groups + kSms - 1) / kSms * (3 + 2 * per);
+    if (best < 0 || cost < best) {
+      best = cost;
+      *hg = per;
+      *ngrp = groups;
+    }
+  }
 }
 SsdBwdWs ssd_bwd_ws(const bds::SsdGeo& g) {
   SsdBwdWs w;
-  ssd_bwd_groups(g, &w.hg, &w.ngrp);
+  ssd_bwd_groups(g, g.Bt * g.nb * g.m, 16, &w.hg, &w.ngrp);
+  ssd_bwd_groups(g, g.Bt * g.nb, bds::kMaxStateBwdHeads, &w.hg_s, &w.ngrp_s);
   const size_t bkg = (size_t)g.Bt * g.nb * w.ngrp;
   const size_t bkh = (size_t)g.Bt * g.nb * g.H, P = 64, N = (size_t)g.N, m = (size_t)g.m, Bs = (size_t)g.Bs;
   size_t o = 0;
@@ -437,7 +449,7 @@ SsdBwdWs ssd_bwd_ws(const bds::SsdGeo& g) {
   w.sumdt = take(bkh);
   w.gS = take(bkh * P * N);
   w.dxs = take(bkh * Bs * P);
-  w.dBs = take(bkh * Bs * N);
+  w.dBs = take((size_t)g.Bt * g.nb * w.ngrp_s * Bs * N);
   w.dAs = take(bkh);
   w.dd = take(bkh * m * 8 * 2);  // dy . x partials of the clean, then the noisy stream
   w.total = o;
@@ -540,10 +552,11 @@ extern "C" int bdscan_ssd_backward(const bdscan_ssd_dims* dims, const bdscan_cle
     e = bds::api_launched(bds::launch_ssd_bwd_tile(st == 2, st < 2, p, s), s);
   }
   // 2. dt and A gradients of each stream from the row and column sums
-  for (int st = 0; st < 3 && e == cudaSuccess; ++st) {
-    bds::SsdBwdVecParams v;
-    memset(&v, 0, sizeof(v));
-    v.g = g;
+  bds::SsdBwdVecParams vp;
+  memset(&vp, 0, sizeof(vp));
+  vp.g = g;
+  for (int st = 0; st < 3; ++st) {
+    bds::SsdBwdVecStream& v = vp.s[st];
     v.dt = dts[st];
     v.A = As[st];
     v.col_part = F(w.colp[st]);
@@ -554,8 +567,8 @@ extern "C" int bdscan_ssd_backward(const bdscan_ssd_dims* dims, const bdscan_cle
     v.ddt_out = st == 1 ? (bf*)gnoisy->ddt_f : st == 2 ? (bf*)gnoisy->ddt_r : nullptr;
     v.dA = F(w.dAv[st]);
     v.sumdt = st == 0 ? F(w.sumdt) : nullptr;
-    e = bds::api_launched(bds::launch_ssd_bwd_vec(v, s), s);
   }
+  if (e == cudaSuccess) e = bds::api_launched(bds::launch_ssd_bwd_vec(vp, s), s);
   // 3. reverse pass over the clean block-end states
   if (e == cudaSuccess) {
     bds::SsdBwdPassParams q;
@@ -583,6 +596,7 @@ extern "C" int bdscan_ssd_backward(const bdscan_ssd_dims* dims, const bdscan_cle
     r.sumdt = F(w.sumdt);
     r.dx_state = F(w.dxs);
     r.dB_state = F(w.dBs);
+    r.hg = w.hg_s;
     r.ddt_tile = F(w.ddtv[0]);
     r.ddt = (bf*)gclean->ddt;
     r.dA = F(w.dAs);
@@ -595,7 +609,7 @@ extern "C" int bdscan_ssd_backward(const bdscan_ssd_dims* dims, const bdscan_cle
                                                  params->D_f, params->D_r, (bf*)gclean->dx, (bf*)gnoisy->dx, s),
                           s);
   if (e == cudaSuccess)
-    e = bds::api_launched(bds::launch_ssd_bwd_dbc(g, w.ngrp, F(w.dBp[0]), F(w.dBs), F(w.dCp[0]), F(w.dBp[1]), F(w.dCp[1]),
+    e = bds::api_launched(bds::launch_ssd_bwd_dbc(g, w.ngrp, w.ngrp_s, F(w.dBp[0]), F(w.dBs), F(w.dCp[0]), F(w.dBp[1]), F(w.dCp[1]),
                                                   F(w.dBp[2]), F(w.dCp[2]), (bf*)gclean->dB, (bf*)gclean->dC,
                                                   (bf*)gnoisy->dB_f, (bf*)gnoisy->dC_f, (bf*)gnoisy->dB_r,
                                                   (bf*)gnoisy->dC_r, s),

@@ -36,7 +36,7 @@ namespace {
 
 using umma::sw128;
 
-constexpr int kBwdThreads = 128;   // k_ssd_bwd_state
+constexpr int kStateBwdThreads = 256;  // k_ssd_bwd_state
 constexpr int kTileThreads = 256;  // k_ssd_bwd_tile: two threads per token row
 
 // Copies `rows` rows of `ncols` (64 or 128) bf16 into 128-byte-swizzled atom
@@ -84,12 +84,6 @@ __device__ __forceinline__ void stage_f32_hilo(unsigned char* dhi, unsigned char
     *reinterpret_cast<uint4*>(dhi + off) = make_uint4(hi[0], hi[1], hi[2], hi[3]);
     *reinterpret_cast<uint4*>(dlo + off) = make_uint4(lo[0], lo[1], lo[2], lo[3]);
   }
-}
-
-// Element `col` of row `row` of a bf16 tile in swizzled atom columns of 128 rows.
-__device__ __forceinline__ float tile_at(const unsigned char* tile, int row, int col) {
-  const uint32_t off = (uint32_t)(col >> 6) * kTile16 + sw128((uint32_t)row, (uint32_t)((col & 63) >> 3)) + (uint32_t)(col & 7) * 2u;
-  return __bfloat162float(*reinterpret_cast<const __nv_bfloat16*>(tile + off));
 }
 
 // Stores a warp's 32 x 32 fp32 block (lane r holds row r in v) to rows
@@ -687,13 +681,14 @@ __device__ __forceinline__ void warp_scan_f32(float* a, int n) {
 }
 
 
-// One warp per (batch row, block, head): dc_t = A (rowsum_t - dt_t colsum'_t +
+// One warp per (batch row, block, head) and stream (blockIdx.y): dc_t = A (rowsum_t - dt_t colsum'_t +
 // rowdot_t), ddt_r = colsum'_r + sum of dc over the tokens whose cumulative dt
 // includes dt_r (t >= r forward, t <= r reverse), dA = sum_t c_t (dc_t / A).
-__global__ void __launch_bounds__(128) k_ssd_bwd_vec(const SsdBwdVecParams p) {
+__global__ void __launch_bounds__(128) k_ssd_bwd_vec(const __grid_constant__ SsdBwdVecParams prm) {
   pdl_sync();
   __shared__ float s_c[4][256], s_q[4][256], s_col[4][256];
-  const SsdGeo& g = p.g;
+  const SsdGeo& g = prm.g;
+  const SsdBwdVecStream& p = prm.s[blockIdx.y];
   const int w = threadIdx.x >> 5, lane = threadIdx.x & 31, Bs = (int)g.Bs, m = g.m, H = g.H;
   const int64_t u = (int64_t)blockIdx.x * 4 + w;
   if (u >= g.Bt * g.nb * H) return;  // whole warps
@@ -787,187 +782,258 @@ __global__ void __launch_bounds__(256) k_ssd_bwd_pass(const SsdBwdPassParams p) 
   }
 }
 
-// Shared memory of k_ssd_bwd_state (from a 1024-aligned base): the state
-// gradient's bf16 high and low parts ([64 p][N], atom columns of 8 KB), x and
-// B of one s-tile, per-token vectors of the block.
+// Shared memory of k_ssd_bwd_state (from a 1024-aligned base):
+//   G     the state gradient's bf16 high and low parts ([64 p][N] each, atom
+//         columns of 8 KB); after the products per-warp 32 x 32 fp32
+//         transposition blocks of the stores
+//   RAW   the next state gradient as loaded (fp32)
+//   X     two buffers of a head's x tiles; BT the block's B tiles
+//   SUF   per head of the CTA the dt after each token, DT its dt (bf16), DW
+//         x . U (one tile per block: of each half of the channels)
 struct StateBwdSmem {
-  static constexpr uint32_t GH = 0, GL = 16384, X = 32768, BT = 49152, VEC = 81920;
-  static constexpr uint32_t TR = VEC + 6u * 256u * 4u;  // per-warp 32 x 32 fp32 transposition blocks
-  static constexpr uint32_t total = TR + 4u * 4096u + 1024u;
+  uint32_t g, raw, x, bt, suf, dt, dw, total;
+  __host__ __device__ StateBwdSmem(int N, int m, int hg) {
+    g = 0;
+    raw = 32768u;
+    x = raw + 256u * (uint32_t)N;
+    bt = x + 2u * (uint32_t)m * 16384u;
+    suf = bt + (uint32_t)(m * (N / 64)) * kTile16;
+    dw = suf + (uint32_t)hg * (uint32_t)m * 512u;
+    dt = dw + (uint32_t)hg * 1024u;
+    total = dt + (uint32_t)hg * (uint32_t)m * 256u + 1024u;
+  }
 };
 
-// One CTA of 4 warps per (batch row, block, head) of the clean stream, with
-// gS = the gradient of the state after the block: U = B gS^T and V = x gS per
-// s-tile on the tensor core (gS split into bf16 high and low parts), then
-// dx += w U, dB += w V, dw = x . U, and the dt and A gradients of w and of
-// the block decay.
-template <int N>
-__global__ void __launch_bounds__(kBwdThreads, 1) k_ssd_bwd_state(const SsdBwdStateParams p) {
+// One CTA of 8 warps per (batch row, block) of the clean stream and group of
+// heads, with gS = the gradient of the state after the block. Per head and
+// 128-token tile U = B gS^T and V = x gS on the tensor core (gS split into
+// bf16 high and low parts), then dx = w U, dw = x . U, and the dt and A
+// gradients of w and of the block decay. dB is shared by the heads: w V is
+// summed over the group's heads in registers, one row (two tiles) or half a
+// row (one tile) per thread, and leaves once per group. The next head's gS, x
+// and previous state arrive under the current head's products and epilogue.
+// Bound by memory and the chain of a head's steps: 8 x 8192 x 26 heads x 128
+// moves 1.1 GB in 342 us. A CTA per head, with 0.87 GB of per-head dB written
+// here and read back by k_ssd_bwd_dbc, took 518 us (and the combine 241 for 109).
+template <int N, bool TWO>
+__global__ void __launch_bounds__(kStateBwdThreads, 1) k_ssd_bwd_state(const SsdBwdStateParams p) {
   pdl_sync();
   extern __shared__ unsigned char smraw[];
   unsigned char* sm = align1024(smraw);
   __shared__ uint64_t bar;
   __shared__ uint32_t tslot;
-  __shared__ float red[4];
-  using S = StateBwdSmem;
+  __shared__ float red[kMaxStateBwdHeads][kStateBwdThreads / 32];
+  constexpr int NT = kStateBwdThreads, m = TWO ? 2 : 1, Bs = 128 * m;
+  constexpr int UC = TWO ? 64 : 32, VC = TWO ? N : N / 2;  // columns of U and V per thread
   const SsdGeo& g = p.g;
-  const int Bs = (int)g.Bs, H = g.H, m = g.m, t = threadIdx.x, w = t >> 5, lane = t & 31;
+  const int H = g.H, tid = threadIdx.x, w = tid >> 5, lane = tid & 31, t = tid & 127, half = tid >> 7;
   const int64_t bk = blockIdx.x, b = bk / g.nb;
-  const int k = (int)(bk % g.nb), h = blockIdx.y;
-  // debug build: the block and the head lie inside the sizes
-  if (!(dguard(kSiteSsdBwdState, bk, g.Bt * g.nb) && dguard(kSiteSsdBwdState, h, H))) return;
+  const int k = (int)(bk % g.nb);
+  const int grp = blockIdx.y, h0 = grp * p.hg, hg = min(H, h0 + p.hg) - h0;
+  // debug build: the block and the heads lie inside the sizes
+  if (!(dguard(kSiteSsdBwdState, bk, g.Bt * g.nb) && dguard(kSiteSsdBwdState, h0 + hg - 1, H))) return;
+  const StateBwdSmem S(N, m, p.hg);
   const int64_t tok0 = b * g.L + (int64_t)k * Bs, HP = (int64_t)H * kSsdP, PN = (int64_t)kSsdP * N;
-  float* s_suf = reinterpret_cast<float*>(sm + S::VEC);  // inclusive suffix sums of dt, then exclusive
-  float* s_dt = s_suf + 256;
-  float* s_w = s_dt + 256;
-  float* s_dw = s_w + 256;
-  float* s_e = s_dw + 256;
-  float* s_vt = s_e + 256;  // the tile side of the dt gradient, added at the end
-  const float* gS = p.gS + (bk * H + h) * PN;
-  for (int s = t; s < Bs; s += kBwdThreads)
-    cp_async4(s_vt + s, p.ddt_tile + (tok0 + s) * H + h);  // completes with the first tile's staging
-  if (w == 0) warp_scan_dt<true>(p.dt + tok0 * H + h, H, Bs, s_suf, s_dt);
-  // gS as bf16 high and low parts, and the block decay's da = sum over (p, n)
-  // of gS o S_{k-1}: the loads of both matrices are issued first
-  float da = 0.f;
-  {
-    constexpr int cpr = N / 8, per = 64 * cpr / kBwdThreads;
-    const float* prev = k > 0 ? p.states + ((b * g.nb + k - 1) * H + h) * PN : nullptr;
-    float4 ga[per], gb[per], pa[per], pb[per];
+  float* s_suf = reinterpret_cast<float*>(sm + S.suf);                  // [hh][Bs]
+  float* s_dw = reinterpret_cast<float*>(sm + S.dw);                    // [hh][256]
+  __nv_bfloat16* s_dt = reinterpret_cast<__nv_bfloat16*>(sm + S.dt);    // [hh][Bs]
+  const float* gS = p.gS + (bk * H + h0) * PN;                          // head h0 + hh at hh PN
+  const float* prev = k > 0 ? p.states + ((bk - 1) * H + h0) * PN : nullptr;
+
+  auto load_head = [&](int hh) {  // gS and x of head h0 + hh
+    for (int c = tid; c < kSsdP * N / 4; c += NT) cp_async16(sm + S.raw + c * 16, gS + hh * PN + c * 4, 16);
+#pragma unroll
+    for (int j = 0; j < m; ++j)
+      stage_bf16<NT>(sm + S.x + (uint32_t)((hh & 1) * m + j) * 16384u, p.x + ((tok0 + j * kSsdT) * H + h0 + hh) * kSsdP,
+                     HP, 128, 64);
+    cp_async_commit();
+  };
+  constexpr int cpr = N / 8, per = kSsdP * cpr / NT;  // 8-element pieces of a state matrix per thread
+  float4 pa[per], pb[per];                            // the previous state's, for the block decay's gradient
+  auto load_prev = [&](int hh) {
 #pragma unroll
     for (int q = 0; q < per; ++q) {
-      const int c = t + q * kBwdThreads, r = c / cpr, ch = c % cpr;
-      ga[q] = *reinterpret_cast<const float4*>(gS + r * N + ch * 8);
-      gb[q] = *reinterpret_cast<const float4*>(gS + r * N + ch * 8 + 4);
-      pa[q] = prev != nullptr ? *reinterpret_cast<const float4*>(prev + r * N + ch * 8) : make_float4(0.f, 0.f, 0.f, 0.f);
-      pb[q] = prev != nullptr ? *reinterpret_cast<const float4*>(prev + r * N + ch * 8 + 4) : make_float4(0.f, 0.f, 0.f, 0.f);
+      const float* src = prev + hh * PN + (tid + q * NT) * 8;
+      pa[q] = prev != nullptr ? *reinterpret_cast<const float4*>(src) : make_float4(0.f, 0.f, 0.f, 0.f);
+      pb[q] = prev != nullptr ? *reinterpret_cast<const float4*>(src + 4) : make_float4(0.f, 0.f, 0.f, 0.f);
     }
+  };
 #pragma unroll
-    for (int q = 0; q < per; ++q) {
-      const int c = t + q * kBwdThreads, r = c / cpr, ch = c % cpr;
-      const float v[8] = {ga[q].x, ga[q].y, ga[q].z, ga[q].w, gb[q].x, gb[q].y, gb[q].z, gb[q].w};
-      const float u[8] = {pa[q].x, pa[q].y, pa[q].z, pa[q].w, pb[q].x, pb[q].y, pb[q].z, pb[q].w};
-      uint32_t hi[4], lo[4];
-#pragma unroll
-      for (int e = 0; e < 4; ++e) {
-        const __nv_bfloat162 hv = __floats2bfloat162_rn(v[2 * e], v[2 * e + 1]);
-        hi[e] = *reinterpret_cast<const uint32_t*>(&hv);
-        lo[e] = pack_bf16(__fsub_rn(v[2 * e], __low2float(hv)), __fsub_rn(v[2 * e + 1], __high2float(hv)));
-      }
-#pragma unroll
-      for (int e = 0; e < 8; ++e) da = __fmaf_rn(v[e], u[e], da);
-      const uint32_t off = (uint32_t)(ch >> 3) * 64u * 128u + sw128((uint32_t)r, (uint32_t)(ch & 7));
-      *reinterpret_cast<uint4*>(sm + S::GH + off) = make_uint4(hi[0], hi[1], hi[2], hi[3]);
-      *reinterpret_cast<uint4*>(sm + S::GL + off) = make_uint4(lo[0], lo[1], lo[2], lo[3]);
+  for (int j = 0; j < m; ++j)
+    stage_bf16<NT>(sm + S.bt + (uint32_t)(j * (N / 64)) * kTile16, p.B + (tok0 + j * kSsdT) * N, N, 128, N);
+  load_head(0);
+  load_prev(0);
+  for (int hh = w; hh < hg; hh += NT / 32) {  // dt and the dt after each token
+    const __nv_bfloat16* dth = p.dt + tok0 * H + h0 + hh;
+    float* suf = s_suf + hh * Bs;
+    warp_scan_dt<true>(dth, H, Bs, suf);
+    __syncwarp();
+    for (int s = lane; s < Bs; s += 32) {
+      const __nv_bfloat16 d = dth[(int64_t)s * H];
+      s_dt[hh * Bs + s] = d;
+      suf[s] = __fsub_rn(suf[s], __bfloat162float(d));
     }
   }
-  da = warp_sum(da);
-  if (lane == 0) red[w] = da;
-  if (t == 0) umma::bar_init(&bar, 1);
-  if (w == 0) tmem_alloc(&tslot, 256);
+  if (tid == 0) umma::bar_init(&bar, 1);
+  constexpr uint32_t kCols = m * (N + 64) <= 128 ? 128 : m * (N + 64) <= 256 ? 256 : 512;
+  if (w == 0) tmem_alloc(&tslot, kCols);
   umma::fence_before_sync();
   __syncthreads();
   umma::fence_after_sync();
-  da = __fadd_rn(__fadd_rn(red[0], red[1]), __fadd_rn(red[2], red[3]));
-  for (int s = t; s < Bs; s += kBwdThreads) s_suf[s] = __fsub_rn(s_suf[s], s_dt[s]);  // dt after s
-  const uint32_t tm = tslot, lane_base = tm + ((uint32_t)(32 * w) << 16);
-  const float A = p.A[h], A2 = __fmul_rn(A, kLog2e);
-  const uint32_t gh = umma::smem_u32(sm + S::GH), gl = umma::smem_u32(sm + S::GL), x0 = umma::smem_u32(sm + S::X),
-                 b0 = umma::smem_u32(sm + S::BT);
+  const uint32_t tm = tslot, lane_base = tm + ((uint32_t)(32 * (w & 3)) << 16);
+  const uint32_t gh = umma::smem_u32(sm + S.g), x0 = umma::smem_u32(sm + S.x), b0 = umma::smem_u32(sm + S.bt);
+  constexpr uint32_t kGLow = 64u * (uint32_t)N * 2u;                        // low parts after the high ones
+  constexpr uint32_t kU = m * N;                                            // TMEM: V_j at N j, U_j at kU + 64 j
   constexpr uint32_t id_u = umma::idesc_bf16(128, 64, false, false);
   constexpr uint32_t id_v = umma::idesc_bf16(128, N, false, true);
-  uint32_t phase = 0;
+  const int tile = TWO ? half : 0, row = tile * kSsdT + t;                  // this thread's token
+  const uint32_t ucol = kU + (TWO ? 64u * (uint32_t)half : 32u * (uint32_t)half);
+  const uint32_t vcol = TWO ? (uint32_t)(N * half) : (uint32_t)(VC * half);
+  const int u0 = TWO ? 0 : 32 * half;                                       // first channel of the thread's U columns
+  const int64_t row0 = tile * kSsdT + 32 * (w & 3);                         // the warp's first token
+  float* tb = reinterpret_cast<float*>(sm + S.g) + w * 1024;
+  float acc[VC];
+#pragma unroll
+  for (int e = 0; e < VC; ++e) acc[e] = 0.f;
   bool alive = true;
-  for (int j = 0; j < m; ++j) {
-    const int64_t sr0 = tok0 + (int64_t)j * kSsdT;
-    stage_bf16<kBwdThreads>(sm + S::X, p.x + (sr0 * H + h) * kSsdP, HP, 128, 64);
-    stage_bf16<kBwdThreads>(sm + S::BT, p.B + sr0 * N, N, 128, N);
-    cp_async_commit();
+  for (int hh = 0; hh < hg; ++hh) {
     cp_async_wait_all();
+    __syncthreads();  // the head's gS and x have landed; the transposition blocks are no longer read
+    float da = 0.f;   // the block decay's: sum over (p, n) of gS o S_{k-1}
+#pragma unroll
+    for (int q = 0; q < per; ++q) {
+      const int c = tid + q * NT, r = c / cpr, ch = c % cpr;
+      const float4 ga = *reinterpret_cast<const float4*>(sm + S.raw + c * 32);
+      const float4 gb = *reinterpret_cast<const float4*>(sm + S.raw + c * 32 + 16);
+      const float v[8] = {ga.x, ga.y, ga.z, ga.w, gb.x, gb.y, gb.z, gb.w};
+      const float u[8] = {pa[q].x, pa[q].y, pa[q].z, pa[q].w, pb[q].x, pb[q].y, pb[q].z, pb[q].w};
+      uint32_t hi[4], lo[4];
+#pragma unroll
+      for (int e = 0; e < 4; ++e) split_pair(v[2 * e], v[2 * e + 1], hi[e], lo[e]);
+#pragma unroll
+      for (int e = 0; e < 8; ++e) da = __fmaf_rn(v[e], u[e], da);
+      const uint32_t off = (uint32_t)(ch >> 3) * 64u * 128u + sw128((uint32_t)r, (uint32_t)(ch & 7));
+      *reinterpret_cast<uint4*>(sm + S.g + off) = make_uint4(hi[0], hi[1], hi[2], hi[3]);
+      *reinterpret_cast<uint4*>(sm + S.g + kGLow + off) = make_uint4(lo[0], lo[1], lo[2], lo[3]);
+    }
     umma::fence_async_smem();
     umma::fence_before_sync();
     __syncthreads();
-    if (t == 0) {
+    const uint32_t xo = (uint32_t)((hh & 1) * m) * 16384u;
+    if (tid == 0) {
       umma::fence_after_sync();
-      const uint64_t db = umma::sdesc(b0, 16, 1024), dx = umma::sdesc(x0, 16, 1024);
 #pragma unroll
-      for (int half = 0; half < 2; ++half) {
-        const uint32_t gs0 = half ? gl : gh;
-        const uint64_t dgk = umma::sdesc(gs0, 16, 1024), dgm = umma::sdesc(gs0, 8192, 1024);
+      for (int j = 0; j < m; ++j) {
+        const uint64_t db = umma::sdesc(b0 + (uint32_t)(j * (N / 64)) * kTile16, 16, 1024),
+                       dx = umma::sdesc(x0 + xo + (uint32_t)j * 16384u, 16, 1024);
 #pragma unroll
-        for (int kk = 0; kk < N / 16; ++kk)  // U = B_j gS^T: gS K-major [p][n]
-          umma::mma_bf16(tm, umma::sdesc_adv(db, (kk >> 2) * kTile16 + (kk & 3) * 32u),
-                         umma::sdesc_adv(dgk, (kk >> 2) * 8192u + (kk & 3) * 32u), id_u, half > 0 || kk > 0);
+        for (int part = 0; part < 2; ++part) {
+          const uint32_t gs0 = gh + (part ? kGLow : 0u);
+          const uint64_t dgk = umma::sdesc(gs0, 16, 1024), dgm = umma::sdesc(gs0, 8192, 1024);
 #pragma unroll
-        for (int kk = 0; kk < 4; ++kk)  // V = x_j gS: gS MN-major [p][n]
-          umma::mma_bf16(tm + 64u, umma::sdesc_adv(dx, kk * 32u), umma::sdesc_adv(dgm, kk * 2048u), id_v,
-                         half > 0 || kk > 0);
+          for (int kk = 0; kk < N / 16; ++kk)  // U = B_j gS^T: gS K-major [p][n]
+            umma::mma_bf16(tm + kU + 64u * j, umma::sdesc_adv(db, (kk >> 2) * kTile16 + (kk & 3) * 32u),
+                           umma::sdesc_adv(dgk, (kk >> 2) * 8192u + (kk & 3) * 32u), id_u, part > 0 || kk > 0);
+#pragma unroll
+          for (int kk = 0; kk < 4; ++kk)  // V = x_j gS: gS MN-major [p][n]
+            umma::mma_bf16(tm + (uint32_t)(N * j), umma::sdesc_adv(dx, kk * 32u), umma::sdesc_adv(dgm, kk * 2048u), id_v,
+                           part > 0 || kk > 0);
+        }
       }
       umma::mma_commit(&bar);
     }
-    if (!cta_wait(&bar, phase, p.flag)) {
+    if (hh + 1 < hg) {
+      load_head(hh + 1);
+      load_prev(hh + 1);
+    }
+    da = warp_sum(da);
+    if (lane == 0) red[hh][w] = da;
+    if (!cta_wait(&bar, (uint32_t)(hh & 1), p.flag)) {
       alive = false;
       break;
     }
-    phase ^= 1u;
     umma::fence_after_sync();
-    {
-      const int s = j * kSsdT + t;
-      const float e = ex2(__fmul_rn(A2, s_suf[s])), ws = __fmul_rn(e, s_dt[s]);
-      float v[32], dw = 0.f;
-      float* tb = reinterpret_cast<float*>(sm + S::TR) + w * 1024;
-      const int s0 = j * kSsdT + 32 * w;  // the warp's first row
-      float* dxo = p.dx_state + ((bk * H + h) * Bs + s0) * kSsdP;
+    const float A2 = __fmul_rn(p.A[h0 + hh], kLog2e);
+    const float ws = __fmul_rn(ex2(__fmul_rn(A2, s_suf[hh * Bs + row])), __bfloat162float(s_dt[hh * Bs + row]));
+    float v[32], dw = 0.f;
+    float* dxo = p.dx_state + ((bk * H + h0 + hh) * Bs + row0) * kSsdP + u0;
 #pragma unroll
-      for (int q = 0; q < 2; ++q) {
-        umma::tmem_ld32(lane_base + 32u * (uint32_t)q, v);
+    for (int q = 0; q < UC / 32; ++q) {
+      umma::tmem_ld32(lane_base + ucol + 32u * (uint32_t)q, v);
+      const unsigned char* xr = sm + S.x + xo + (uint32_t)tile * 16384u;
 #pragma unroll
-        for (int e2 = 0; e2 < 32; ++e2) {
-          dw = __fmaf_rn(tile_at(sm + S::X, t, 32 * q + e2), v[e2], dw);
-          v[e2] = __fmul_rn(ws, v[e2]);
+      for (int cq = 0; cq < 4; ++cq) {
+        const uint4 xv = *reinterpret_cast<const uint4*>(xr + sw128((uint32_t)t, (uint32_t)(u0 / 8 + 4 * q + cq)));
+        const __nv_bfloat162* x2 = reinterpret_cast<const __nv_bfloat162*>(&xv);
+#pragma unroll
+        for (int e = 0; e < 4; ++e) {
+          const float2 f = __bfloat1622float2(x2[e]);
+          dw = __fmaf_rn(f.x, v[8 * cq + 2 * e], dw);
+          dw = __fmaf_rn(f.y, v[8 * cq + 2 * e + 1], dw);
         }
-        store_block32(dxo + 32 * q, kSsdP, v, tb);
       }
-      float* dbo = p.dB_state + ((bk * H + h) * Bs + s0) * N;
 #pragma unroll
-      for (int q = 0; q < N / 32; ++q) {
-        umma::tmem_ld32(lane_base + 64u + 32u * (uint32_t)q, v);
-#pragma unroll
-        for (int e2 = 0; e2 < 32; ++e2) v[e2] = __fmul_rn(ws, v[e2]);
-        store_block32(dbo + 32 * q, N, v, tb);
-      }
-      s_w[s] = ws;
-      s_dw[s] = dw;
-      s_e[s] = e;
+      for (int e = 0; e < 32; ++e) v[e] = __fmul_rn(ws, v[e]);
+      store_block32(dxo + 32 * q, kSsdP, v, tb);
     }
+#pragma unroll
+    for (int q = 0; q < VC / 32; ++q) {
+      umma::tmem_ld32(lane_base + vcol + 32u * (uint32_t)q, v);
+#pragma unroll
+      for (int e = 0; e < 32; ++e) acc[32 * q + e] = __fmaf_rn(ws, v[e], acc[32 * q + e]);
+    }
+    s_dw[hh * 256 + half * 128 + t] = dw;
     umma::fence_before_sync();
   }
-  __syncthreads();
-  if (alive && w == 0) {
-    // the exponent of w_s is A times the dt after s: dt_r feeds every s < r
-    float dA = 0.f;
-    for (int s = lane; s < Bs; s += 32) {
-      const float wdw = __fmul_rn(s_w[s], s_dw[s]);
-      dA = __fmaf_rn(s_suf[s], wdw, dA);
-      s_suf[s] = __fmul_rn(A, wdw);
-    }
-    __syncwarp();
-    warp_scan_f32<false>(s_suf, Bs);  // inclusive prefix sums of A w dw
-    const float sd = p.sumdt[bk * H + h], ak = ex2(__fmul_rn(A2, sd));
-    const float blk = __fmul_rn(__fmul_rn(A, ak), da);  // block decay exp(A sumdt) of S_{k-1}
-    for (int r = lane; r < Bs; r += 32) {
-      const float before = r > 0 ? s_suf[r - 1] : 0.f;  // exclusive: s < r
-      const float vs = __fadd_rn(__fadd_rn(__fmul_rn(s_e[r], s_dw[r]), before), blk);
-      const int64_t o = (tok0 + r) * H + h;
-      p.ddt[o] = __float2bfloat16_rn(__fadd_rn(s_vt[r], vs));
-    }
-    dA = warp_sum(dA);
-    if (lane == 0) p.dA[bk * H + h] = __fadd_rn(dA, __fmul_rn(__fmul_rn(sd, ak), da));
-  }
   cp_async_wait_all();
+  __syncthreads();
+  if (alive) {
+    float* dbo = p.dB_state + ((bk * gridDim.y + grp) * Bs + row0) * N + (TWO ? 0 : VC * half);
+    float v[32];
+#pragma unroll
+    for (int q = 0; q < VC / 32; ++q) {
+#pragma unroll
+      for (int e = 0; e < 32; ++e) v[e] = acc[32 * q + e];
+      store_block32(dbo + 32 * q, N, v, tb);
+    }
+    // the exponent of w_s is A times the dt after s: dt_r feeds every s < r
+    for (int hh = w; hh < hg; hh += NT / 32) {
+      const int h = h0 + hh;
+      float* suf = s_suf + hh * Bs;
+      const float* dwv = s_dw + hh * 256;
+      const float A = p.A[h], A2 = __fmul_rn(A, kLog2e);
+      float da = red[hh][0], dA = 0.f, ev[Bs / 32], dv[Bs / 32];
+#pragma unroll
+      for (int q = 1; q < NT / 32; ++q) da = __fadd_rn(da, red[hh][q]);
+#pragma unroll
+      for (int q = 0; q < Bs / 32; ++q) {
+        const int s = lane + 32 * q;
+        const float dw = TWO ? dwv[s] : __fadd_rn(dwv[s], dwv[128 + s]);
+        ev[q] = ex2(__fmul_rn(A2, suf[s]));
+        dv[q] = dw;
+        const float wdw = __fmul_rn(__fmul_rn(ev[q], __bfloat162float(s_dt[hh * Bs + s])), dw);
+        dA = __fmaf_rn(suf[s], wdw, dA);
+        suf[s] = __fmul_rn(A, wdw);
+      }
+      __syncwarp();
+      warp_scan_f32<false>(suf, Bs);  // inclusive prefix sums of A w dw
+      const float sd = p.sumdt[bk * H + h], ak = ex2(__fmul_rn(A2, sd));
+      const float blk = __fmul_rn(__fmul_rn(A, ak), da);  // block decay exp(A sumdt) of S_{k-1}
+#pragma unroll
+      for (int q = 0; q < Bs / 32; ++q) {
+        const int r = lane + 32 * q;
+        const float before = r > 0 ? suf[r - 1] : 0.f;  // exclusive: s < r
+        const float vs = __fadd_rn(__fadd_rn(__fmul_rn(ev[q], dv[q]), before), blk);
+        const int64_t o = (tok0 + r) * H + h;
+        p.ddt[o] = __float2bfloat16_rn(__fadd_rn(p.ddt_tile[o], vs));
+      }
+      dA = warp_sum(dA);
+      if (lane == 0) p.dA[bk * H + h] = __fadd_rn(dA, __fmul_rn(__fmul_rn(sd, ak), da));
+    }
+  }
   umma::fence_before_sync();
   __syncthreads();
-  if (w == 0) tmem_dealloc(tm, 256);
+  if (w == 0) tmem_dealloc(tm, kCols);
 }
 
 }  // namespace
@@ -1034,11 +1100,12 @@ __global__ void __launch_bounds__(256) k_ssd_bwd_dx(const SsdGeo g, const float*
 }
 
 // dB and dC of the three streams: the tile partials of every head group (and
-// the clean state term of every head), summed in order. One thread per
+// the clean state term of its own head groups), summed in order. One thread per
 // (token, 4 state indices); the tile index j of a token is the same across
 // a warp but at the ends of 128-token tiles, and only the tile partials that
 // reach the token are read.
-__global__ void __launch_bounds__(256) k_ssd_bwd_dbc(const SsdGeo g, int ngrp, const float* dBp_c, const float* dBs,
+__global__ void __launch_bounds__(256) k_ssd_bwd_dbc(const SsdGeo g, int ngrp, int ngrp_state, const float* dBp_c,
+                                                     const float* dBs,
                                                      const float* dCp_c, const float* dBp_f, const float* dCp_f,
                                                      const float* dBp_r, const float* dCp_r, __nv_bfloat16* dBc,
                                                      __nv_bfloat16* dCc, __nv_bfloat16* dBf, __nv_bfloat16* dCf,
@@ -1077,8 +1144,8 @@ __global__ void __launch_bounds__(256) k_ssd_bwd_dbc(const SsdGeo g, int ngrp, c
     cf = add4(cf, cf0);
     cr = add4(cr, cr0);
   }
-  const float* st = dBs + (bk * g.H * g.Bs + s) * N + n;
-  for (int h = 0; h < g.H; ++h) bc = add4(bc, ld4(st + (int64_t)h * g.Bs * N));
+  const float* st = dBs + (bk * ngrp_state * g.Bs + s) * N + n;
+  for (int q = 0; q < ngrp_state; ++q) bc = add4(bc, ld4(st + (int64_t)q * g.Bs * N));
   st_bf4(dBc + idx, bc);
   st_bf4(dCc + idx, cc);
   st_bf4(dBf + idx, bf);
@@ -1147,13 +1214,13 @@ cudaError_t bwd_tile_t(const SsdBwdTileParams& p_in, cudaStream_t s) {
   return cudaGetLastError();
 }
 
-template <int N>
+template <int N, bool TWO>
 cudaError_t bwd_state_t(const SsdBwdStateParams& p, cudaStream_t s) {
-  const int smem = (int)StateBwdSmem::total;
-  cudaError_t e = set_smem_cached((const void*)k_ssd_bwd_state<N>, smem, -1);
+  const int smem = (int)StateBwdSmem(N, p.g.m, p.hg).total;
+  cudaError_t e = set_smem_cached((const void*)k_ssd_bwd_state<N, TWO>, smem, -1);
   if (e != cudaSuccess) return e;
-  dim3 grid((unsigned)(p.g.Bt * p.g.nb), (unsigned)p.g.H);
-  launch_pdl(k_ssd_bwd_state<N>, grid, kBwdThreads, smem, s, p);
+  dim3 grid((unsigned)(p.g.Bt * p.g.nb), (unsigned)((p.g.H + p.hg - 1) / p.hg));
+  launch_pdl(k_ssd_bwd_state<N, TWO>, grid, kStateBwdThreads, smem, s, p);
   return cudaGetLastError();
 }
 
@@ -1170,7 +1237,7 @@ cudaError_t launch_ssd_bwd_tile(bool upper, bool seeded, const SsdBwdTileParams&
 
 cudaError_t launch_ssd_bwd_vec(const SsdBwdVecParams& p, cudaStream_t s) {
   const int64_t warps = p.g.Bt * p.g.nb * p.g.H;
-  launch_pdl(k_ssd_bwd_vec, (unsigned)((warps + 3) / 4), 128, 0, s, p);
+  launch_pdl(k_ssd_bwd_vec, dim3((unsigned)((warps + 3) / 4), 3), 128, 0, s, p);
   return cudaGetLastError();
 }
 
@@ -1181,7 +1248,8 @@ cudaError_t launch_ssd_bwd_pass(const SsdBwdPassParams& p, cudaStream_t s) {
 }
 
 cudaError_t launch_ssd_bwd_state(const SsdBwdStateParams& p, cudaStream_t s) {
-  return p.g.N == 64 ? bwd_state_t<64>(p, s) : bwd_state_t<128>(p, s);
+  if (p.g.N == 64) return p.g.m == 2 ? bwd_state_t<64, true>(p, s) : bwd_state_t<64, false>(p, s);
+  return p.g.m == 2 ? bwd_state_t<128, true>(p, s) : bwd_state_t<128, false>(p, s);
 }
 
 cudaError_t launch_ssd_bwd_dx(const SsdGeo& g, const float* dxp_c, const float* dxs, const float* dxp_f,
@@ -1193,13 +1261,14 @@ cudaError_t launch_ssd_bwd_dx(const SsdGeo& g, const float* dxp_c, const float* 
   return cudaGetLastError();
 }
 
-cudaError_t launch_ssd_bwd_dbc(const SsdGeo& g, int ngrp, const float* dBp_c, const float* dBs, const float* dCp_c,
+cudaError_t launch_ssd_bwd_dbc(const SsdGeo& g, int ngrp, int ngrp_state, const float* dBp_c, const float* dBs,
+                               const float* dCp_c,
                                const float* dBp_f, const float* dCp_f, const float* dBp_r, const float* dCp_r,
                                __nv_bfloat16* dBc, __nv_bfloat16* dCc, __nv_bfloat16* dBf, __nv_bfloat16* dCf,
                                __nv_bfloat16* dBr, __nv_bfloat16* dCr, cudaStream_t s) {
   const int64_t n = g.Bt * g.L * (g.N / 4);
   if (n == 0) return cudaSuccess;
-  launch_pdl(k_ssd_bwd_dbc, (unsigned)((n + 255) / 256), 256, 0, s, g, ngrp, dBp_c, dBs, dCp_c, dBp_f, dCp_f, dBp_r, dCp_r, dBc,
+  launch_pdl(k_ssd_bwd_dbc, (unsigned)((n + 255) / 256), 256, 0, s, g, ngrp, ngrp_state, dBp_c, dBs, dCp_c, dBp_f, dCp_f, dBp_r, dCp_r, dBc,
                                                               dCc, dBf, dCf, dBr, dCr);
   return cudaGetLastError();
 }
