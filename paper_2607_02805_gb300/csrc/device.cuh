@@ -113,19 +113,20 @@ template <typename T, bool REV = false>
 __device__ __forceinline__ void issue_td(T* tile, const T* g, int64_t row0, int nsteps, int64_t D,
                                          int64_t d0) {
   constexpr int E = 16 / (int)sizeof(T);
-  constexpr int CPR = kCta / E;
-  const int total = nsteps * CPR;
-  for (int i = threadIdx.x; i < total; i += kCta) {
-    const int r = i / CPR, q = i - r * CPR;
-    const int64_t d = d0 + (int64_t)q * E;
-    T* dst = tile + r * kCta + q * E;
-    if (g == nullptr) {
-      *reinterpret_cast<uint4*>(dst) = make_uint4(0u, 0u, 0u, 0u);
-    } else {
-      const bool ok = d < D;
-      cp_async16(dst, ok ? (const void*)(g + (REV ? row0 - r : row0 + r) * D + d) : (const void*)g, ok ? 16 : 0);
-    }
+  constexpr int CPR = kCta / E, RPP = kCta / CPR;  // 16-byte pieces of a row, rows per pass over the CTA
+  const int r0 = (int)threadIdx.x / CPR, q = (int)threadIdx.x % CPR;
+  T* dst = tile + r0 * kCta + q * E;
+  if (g == nullptr) {
+    for (int r = r0; r < nsteps; r += RPP, dst += RPP * kCta) *reinterpret_cast<uint4*>(dst) = make_uint4(0u, 0u, 0u, 0u);
+    return;
   }
+  // a thread's pieces lie in one column, RPP rows apart: one address, stepped
+  const int64_t d = d0 + (int64_t)q * E;
+  const bool ok = d < D;
+  const T* src = ok ? g + (REV ? row0 - r0 : row0 + r0) * D + d : g;
+  const int64_t step = ok ? (REV ? -RPP * D : RPP * D) : 0;
+  const int bytes = ok ? 16 : 0;
+  for (int r = r0; r < nsteps; r += RPP, dst += RPP * kCta, src += step) cp_async16(dst, src, bytes);
 }
 
 // Copies nsteps token-by-state rows [N] into dst[step][N]: step r is row
