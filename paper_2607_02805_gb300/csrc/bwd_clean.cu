@@ -137,14 +137,15 @@ __global__ void __launch_bounds__(kCta, 3) k_bwd_clean(const BwdParams p) {
       } else {
         ck_load<N>(h, ck, s - 1);
       }
+      int64_t o = (row0 + (int64_t)(s + 1) * TS - 1) * g.D + d;  // the token's element, stepped
       seg_bwd_half<N, true>(st, TS, XC, DTC, DYC, BC, CC, A2, sw, h, gc, dA, tb, mine, off, 0,
                        [&](int i, float dt, float x, float dy, float sgB, float sAq) {
-                         const int64_t o = (row0 + s * TS + i) * g.D + d;
                          if (act) {
                            reinterpret_cast<TO*>(p.ddtc)[o] = to_out<TO>(__fmaf_rn(x, sgB, __fmul_rn(kLn2, sAq)));
                            reinterpret_cast<TO*>(p.dxc)[o] = to_out<TO>(__fmaf_rn(Df, dy, __fmul_rn(dt, sgB)));
                          }
                          dDc = __fmaf_rn(dy, x, dDc);
+                         o -= g.D;
                        });
       if (!TILED) red_flush<N>(p, red, 0, 1, 0, 1, b, t0 + (int64_t)s * TS, TS);
     }

@@ -89,6 +89,9 @@ __device__ void red_flush(const BwdParams& p, const float* red, int sB, int sC, 
                           int64_t tstart, int TS) {
   __syncthreads();
   const Geo& g = p.g;
+  const int64_t GN = g.G * N;
+  float* outB = p.part_tok + (((int64_t)tensB * g.Bt + b) * g.L + tstart) * GN + blockIdx.x * N;
+  float* outC = p.part_tok + (((int64_t)tensC * g.Bt + b) * g.L + tstart) * GN + blockIdx.x * N;
 #pragma unroll
   for (int j0 = 0; j0 < 2 * kBwdTS * N; j0 += kCta) {
     const int j = j0 + threadIdx.x;
@@ -100,8 +103,7 @@ __device__ void red_flush(const BwdParams& p, const float* red, int sB, int sC, 
       for (int w = 0; w < kWarps; ++w)
 #pragma unroll
         for (int r = 0; r < 32 / N; ++r) s += src[w * 32 + r * N];
-      const int tensor = which == 0 ? tensB : tensC;
-      p.part_tok[((((int64_t)tensor * g.Bt + b) * g.L + tstart + i) * g.G + blockIdx.x) * N + n] = s;
+      (which == 0 ? outB : outC)[i * GN + n] = s;
     }
   }
   __syncthreads();

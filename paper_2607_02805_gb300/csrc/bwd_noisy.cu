@@ -169,16 +169,18 @@ __global__ void __launch_bounds__(kCta, 1) k_bwd_noisy(const BwdParams p) {
           vzero2<N>(h);
         else
           ck_load<N>(h, ck, s);
+        int64_t o = (row0 + (int64_t)s * TS) * g.D + d;  // the token's element, stepped
         seg_bwd<N, false>(st, TS, XN, DTR, DYN, BR, CR, A2r, sw, h, gr, dAr, tb, mine, off, 0,
                           [&](int i, float dt, float x, float dy, float sgB, float sAq) {
                             const int ib = s * TS + i;
                             if (act)
-                              reinterpret_cast<TO*>(p.ddtr)[(row0 + ib) * g.D + d] =
+                              reinterpret_cast<TO*>(p.ddtr)[o] =
                                   to_out<TO>(__fmaf_rn(x, sgB, __fmul_rn(kLn2, sAq)));
                             if (!SPLIT)
                               dxbuf[(off + ib) * kCta + tid] = __fmul_rn(dt, sgB);
                             else if (act)
-                              dxr_part[(row0 + ib) * g.D + d] = __fmul_rn(dt, sgB);
+                              dxr_part[o] = __fmul_rn(dt, sgB);
+                            o += g.D;
                           });
         if (!TILED) red_flush<N>(p, red, 0, 1, 4, 5, b, t0 + (int64_t)s * TS, TS);
       }
@@ -211,10 +213,10 @@ __global__ void __launch_bounds__(kCta, 1) k_bwd_noisy(const BwdParams p) {
         } else {
           ck_load<N>(h, ck, s - 1);
         }
+        int64_t o = (row0 + (int64_t)(s + 1) * TS - 1) * g.D + d;
         seg_bwd<N, true>(st, TS, XN, DTF, DYN, BF, CF, A2f, sw, h, gf, dAf, tb, mine, off, TILED ? 2 : 0,
                          [&](int i, float dt, float x, float dy, float sgB, float sAq) {
                            const int ib = s * TS + i;
-                           const int64_t o = (row0 + ib) * g.D + d;
                            if (act) {
                              reinterpret_cast<TO*>(p.ddtf)[o] = to_out<TO>(__fmaf_rn(x, sgB, __fmul_rn(kLn2, sAq)));
                              const float dxf = __fmul_rn(dt, sgB);
@@ -225,6 +227,7 @@ __global__ void __launch_bounds__(kCta, 1) k_bwd_noisy(const BwdParams p) {
                                    __fmaf_rn(Dsum, dy, __fadd_rn(dxbuf[(off + ib) * kCta + tid], dxf)));
                            }
                            dDn = __fmaf_rn(dy, x, dDn);
+                           o -= g.D;
                          });
         if (!TILED) red_flush<N>(p, red, 0, 1, 2, 3, b, t0 + (int64_t)s * TS, TS);
       }

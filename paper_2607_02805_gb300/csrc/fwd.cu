@@ -276,10 +276,10 @@ __global__ void __launch_bounds__(kCta, MODE == 0 ? 4 : 6) k_block_scan(const Fw
       for (int sg = 0; sg < NSEG; ++sg) {  // segments left to right
         const int i0 = sg * SEG, ns = Bs - i0 < SEG ? Bs - i0 : SEG;
         if (NSEG > 1) st.load(prow(row0 + i0), ns, g.D, d0);
+        int64_t o = prow(row0 + i0) * g.D + d;  // the token's element, stepped
 #pragma unroll 2
-        for (int ii = 0; ii < ns; ++ii) {
+        for (int ii = 0; ii < ns; ++ii, o += kRev ? -g.D : g.D) {
           const int i = i0 + ii;
-          const int64_t o = prow(row0 + i) * g.D + d;
           if (Ly::kClean) {
             const float x = st.at(Ly::XC, toff + ii), dt = st.at(Ly::DTC, toff + ii);
             const float y = scan_step<N>(hc, A2f, dt, x, st.row(Ly::BC, toff + ii), st.row(Ly::CC, toff + ii));
@@ -308,10 +308,10 @@ __global__ void __launch_bounds__(kCta, MODE == 0 ? 4 : 6) k_block_scan(const Fw
         for (int sg = NSEG - 1; sg >= 0; --sg) {  // segments right to left; the last is still staged
           const int i0 = sg * SEG, ns = Bs - i0 < SEG ? Bs - i0 : SEG;
           if (sg < NSEG - 1) st.load(prow(row0 + i0), ns, g.D, d0);
+          int64_t o = prow(row0 + i0 + ns - 1) * g.D + d;
 #pragma unroll 2
-          for (int ii = ns - 1; ii >= 0; --ii) {
+          for (int ii = ns - 1; ii >= 0; --ii, o -= g.D) {  // noisy streams are never reversed
             const int i = i0 + ii;
-            const int64_t o = prow(row0 + i) * g.D + d;
             const float x = st.at(Ly::XN, toff + ii), dt = st.at(Ly::DTR, toff + ii);
             const float y = scan_step<N>(hr, A2r, dt, x, st.row(Ly::BR, toff + ii), st.row(Ly::CR, toff + ii));
             if (act)
