@@ -24,11 +24,15 @@ struct CleanBwdSmem {
   }
 };
 
-template <typename T, typename TO, int N, bool TILED>
+// KIND: how the chunk is walked (bwd_common.cuh). Blocks of several segments
+// make two passes, the checkpoints and the segments, each staging what it
+// reads, one segment ahead.
+template <typename T, typename TO, int N, int KIND>
 __global__ void __launch_bounds__(kCta, 3) k_bwd_clean(const BwdParams p) {
   pdl_sync();
   extern __shared__ __align__(16) unsigned char smem[];
   using L = CleanBwdSmem<T, N>;
+  constexpr bool TILED = KIND == kTiles, SEGS = KIND == kSegs;
   const Geo& g = p.g;
   const int tid = threadIdx.x, warp = tid >> 5;
   const int sw = swz_of_lane<N>();
@@ -36,7 +40,7 @@ __global__ void __launch_bounds__(kCta, 3) k_bwd_clean(const BwdParams p) {
   const int c = blockIdx.y;
   const int64_t d0 = (int64_t)blockIdx.x * kCta, d = d0 + tid;
   const bool act = d < g.D;
-  const int Bs = (int)g.Bs, TS = Bs < 16 ? Bs : 16, NSEG = Bs / TS;
+  const int Bs = KIND == kOneSeg ? 16 : (int)g.Bs, TS = TILED ? Bs : 16, NSEG = SEGS ? Bs / 16 : 1;
   const int k_lo = chunk_lo(g, c), k_hi = chunk_lo(g, c + 1) - 1;
   // debug build: the chunk's last token and the channel group lie inside the sizes
   if (!(dguard(kSiteBwdClean, b, g.Bt) && dguard(kSiteBwdClean, (int64_t)(k_hi + 1) * Bs - 1, g.L) &&
@@ -52,8 +56,7 @@ __global__ void __launch_bounds__(kCta, 3) k_bwd_clean(const BwdParams p) {
   st.td_src[DYC] = (const T*)p.dyc;
   st.row_src[BC] = (const T*)p.Bc;
   st.row_src[CC] = (const T*)p.Cc;
-  const bool resident = NSEG > 1 && p.seg_resident;
-  const int bufs = NSEG == 1 ? (is_f32<T>::value ? p.stage_bufs : 2) : (resident ? NSEG : 1);
+  const int bufs = is_f32<T>::value ? p.stage_bufs : 2;
   float* red = reinterpret_cast<float*>(smem + L::red_off(bufs));
   float* mine = red_slot<N>(red);
   float* ck = Bs > kCkSmemMaxBs
@@ -84,18 +87,37 @@ __global__ void __launch_bounds__(kCta, 3) k_bwd_clean(const BwdParams p) {
   float2 gc[N / 2];  // a_{t+1} gbar_{t+1} (+ injections) entering token t from the right
   vzero2<N>(gc);
 
+  // SEGS: the steps (pass, segment) of a block in the order they are used, one
+  // step staged ahead: checkpoints of segments 0 .. NSEG-2, then every segment
+  // from the last.
+  int nk = k_hi, ns = 0, fill = 0, cur = 0;  // next step to copy, buffers
+  bool nadj = false;                         // the next step is of the second pass
+  auto copy_step = [&]() {
+    if (nk < k_lo) return false;
+    st.issue_first(fill, b * g.L + (int64_t)nk * Bs + ns * TS, TS, g.D, d0, nadj ? 3 : 2, nadj ? 2 : 1);
+    fill ^= bufs - 1;
+    if (!nadj) {
+      nadj = ++ns > NSEG - 2;  // ns is the last segment then
+    } else if (--ns < 0) {
+      nadj = false;
+      ns = 0;
+      --nk;
+    }
+    return true;
+  };
+  auto next_step = [&](int nrow) {  // the next step's tiles become current
+    __syncthreads();                // the buffer to fill is no longer read
+    const bool ahead = copy_step() && bufs == 2;
+    st.complete(cur, TS, ahead ? 1 : 0, nrow);
+    cur ^= bufs - 1;
+  };
+  if (SEGS && bufs == 2) copy_step();
+
   // everything for block k, whose tokens start at `off` in the staged tile;
   // seed_staged: its seed is in seedb[buf]
   auto block = [&](int k, int off, int buf, bool seed_staged) {
     const int64_t t0 = (int64_t)k * Bs;
     const int64_t row0 = b * g.L + t0;
-    // make segment s current: staged now, or already resident
-    auto stage_seg = [&](int s) {
-      if (resident)
-        st.select(s);
-      else
-        st.load(row0 + (int64_t)s * TS, TS, g.D, d0);
-    };
     if (k == k_hi) {
       if (act) vload2<N>(gc, p.Lc + ((b * g.nc + c) * g.D + d) * N, sw);
     } else if (act) {
@@ -112,24 +134,22 @@ __global__ void __launch_bounds__(kCta, 3) k_bwd_clean(const BwdParams p) {
     float2 seed[N / 2];
     vzero2<N>(seed);
     if (seed_staged)
-        vload2<N>(seed, seedb + (buf * kCta + tid) * N, sw);  // staged with the tile
-      else if (NSEG == 1 && k > 0 && act)
-        vload2<N>(seed, p.states + ((b * g.nb + (k - 1)) * g.D + d) * N, sw);
-      else if (k > 0 && act)
-        vload2<N>(seed, p.states + ((b * g.nb + (k - 1)) * g.D + d) * N, sw);
-    if (NSEG > 1) {
+      vload2<N>(seed, seedb + (buf * kCta + tid) * N, sw);  // staged with the tile
+    else if (k > 0 && act)
+      vload2<N>(seed, p.states + ((b * g.nb + (k - 1)) * g.D + d) * N, sw);
+    if (SEGS) {
       float2 h[N / 2];
 #pragma unroll
       for (int j = 0; j < N / 2; ++j) h[j] = seed[j];
       for (int s = 0; s < NSEG - 1; ++s) {
-        stage_seg(s);
+        next_step(1);
 #pragma unroll 4
         for (int i = 0; i < TS; ++i) scan_state_swz<N>(h, A2, st.at(DTC, i), st.at(XC, i), st.row(BC, i), sw);
         ck_store<N>(ck, s, h);
       }
     }
     for (int s = NSEG - 1; s >= 0; --s) {
-      if (NSEG > 1) stage_seg(s);
+      if (SEGS) next_step(2);
       float2 h[N / 2];
       if (s == 0) {
 #pragma unroll
@@ -176,28 +196,23 @@ __global__ void __launch_bounds__(kCta, 3) k_bwd_clean(const BwdParams p) {
       red_flush<N>(p, red, 0, 1, 0, 1, b, (int64_t)kt_lo * Bs, nbk * Bs);  // the tile's dB/dC
       kt_hi = kt_lo - 1;
     }
+  } else if (SEGS) {
+    for (int k = k_hi; k >= k_lo; --k) block(k, 0, 0, false);
   } else {
-    // one-segment blocks, two buffers: block k-1 (and its seed) is copied while block k is processed
+    // two buffers: block k-1 (and its seed) is copied while block k is processed
     auto issue_block = [&](int buf, int k) {
       issue_seed<N>(seedb + buf * kCta * N, p.states, g, b, k, d0);  // same cp.async group as the block
       st.issue(buf, b * g.L + (int64_t)k * Bs, TS, g.D, d0);
     };
-    if (NSEG == 1 && bufs == 2) issue_block(0, k_hi);
+    if (bufs == 2) issue_block(0, k_hi);
     for (int k = k_hi; k >= k_lo; --k) {
-      const int64_t row0 = b * g.L + (int64_t)k * Bs;
-      const int buf = NSEG == 1 && bufs == 2 ? (k_hi - k) & 1 : 0;
-      if (NSEG == 1) {
-        const bool ahead = bufs == 2 && k > k_lo;
-        __syncthreads();  // the buffer to fill is no longer read
-        if (bufs == 1) issue_block(0, k);
-        if (ahead) issue_block(buf ^ 1, k - 1);
-        st.complete(buf, TS, ahead ? 1 : 0);
-      } else if (resident) {  // every segment of the block, once
-        __syncthreads();  // the previous block is no longer read
-        for (int s = 0; s < NSEG; ++s) st.issue(s, row0 + (int64_t)s * TS, TS, g.D, d0);
-        for (int s = 0; s < NSEG; ++s) st.complete(s, TS, 0);
-      }
-      block(k, 0, buf, NSEG == 1);
+      const int buf = bufs == 2 ? (k_hi - k) & 1 : 0;
+      const bool ahead = bufs == 2 && k > k_lo;
+      __syncthreads();  // the buffer to fill is no longer read
+      if (bufs == 1) issue_block(0, k);
+      if (ahead) issue_block(buf ^ 1, k - 1);
+      st.complete(buf, TS, ahead ? 1 : 0);
+      block(k, 0, buf, true);
     }
   }
   if (act) {
@@ -211,38 +226,47 @@ __global__ void __launch_bounds__(kCta, 3) k_bwd_clean(const BwdParams p) {
 
 namespace {
 
-template <typename T, typename TO, int N, bool TILED>
+template <typename T, typename TO, int N, int KIND>
 BwdLaunch clean_launch(int Bs, int dev) {
-  const int TS = Bs < 16 ? Bs : 16;
-  return bwd_launch<CleanBwdSmem<T, N>, is_f32<T>::value>(k_bwd_clean<T, TO, N, TILED>, Bs, half_cols(TS, N), dev);
+  return bwd_launch<CleanBwdSmem<T, N>, is_f32<T>::value>(k_bwd_clean<T, TO, N, KIND>, Bs,
+                                                          half_cols(Bs < 16 ? Bs : 16, N), dev);
 }
 
-template <typename T, typename TO, int N, bool TILED>
+template <typename T, typename TO, int N, int KIND>
 cudaError_t bwd_clean_tt(const BwdParams& p_in, cudaStream_t s) {
   int dev = 0;
   cudaError_t e = cudaGetDevice(&dev);
   if (e != cudaSuccess) return e;
-  const BwdLaunch l = clean_launch<T, TO, N, TILED>((int)p_in.g.Bs, dev);
+  const BwdLaunch l = clean_launch<T, TO, N, KIND>((int)p_in.g.Bs, dev);
   BwdParams p = p_in;
-  p.seg_resident = l.resident;
   p.stage_bufs = l.bufs;
-  e = set_bwd_attrs(k_bwd_clean<T, TO, N, TILED>, l.smem);
+  e = set_bwd_attrs(k_bwd_clean<T, TO, N, KIND>, l.smem);
   if (e != cudaSuccess) return e;
   dim3 grid((unsigned)p.g.G, (unsigned)p.g.nc, (unsigned)p.g.Bt);
-  launch_pdl(k_bwd_clean<T, TO, N, TILED>, grid, kCta, l.smem, s, p);
+  launch_pdl(k_bwd_clean<T, TO, N, KIND>, grid, kCta, l.smem, s, p);
   return cudaGetLastError();
 }
 template <typename T, typename TO, int N>
 cudaError_t bwd_clean_t(const BwdParams& p, cudaStream_t s) {
-  return p.g.Bs < kBwdTS ? bwd_clean_tt<T, TO, N, true>(p, s) : bwd_clean_tt<T, TO, N, false>(p, s);
+  switch (bwd_kind(p.g.Bs, false)) {
+    case kTiles: return bwd_clean_tt<T, TO, N, kTiles>(p, s);
+    case kSegs: return bwd_clean_tt<T, TO, N, kSegs>(p, s);
+    default: return bwd_clean_tt<T, TO, N, kOneSeg>(p, s);
+  }
 }
 
+template <typename T, typename TO, int N, int KIND>
+int clean_resident(int Bs, int dev) {
+  return resident_ctas(k_bwd_clean<T, TO, N, KIND>, clean_launch<T, TO, N, KIND>(Bs, dev).smem,
+                       half_cols(Bs < 16 ? Bs : 16, N), dev);
+}
 template <typename T, typename TO, int N>
 int bwd_clean_per_sm_t(int Bs, int dev) {
-  const int TS = Bs < 16 ? Bs : 16;
-  if (Bs < kBwdTS)
-    return resident_ctas(k_bwd_clean<T, TO, N, true>, clean_launch<T, TO, N, true>(Bs, dev).smem, half_cols(TS, N), dev);
-  return resident_ctas(k_bwd_clean<T, TO, N, false>, clean_launch<T, TO, N, false>(Bs, dev).smem, half_cols(TS, N), dev);
+  switch (bwd_kind(Bs, false)) {
+    case kTiles: return clean_resident<T, TO, N, kTiles>(Bs, dev);
+    case kSegs: return clean_resident<T, TO, N, kSegs>(Bs, dev);
+    default: return clean_resident<T, TO, N, kOneSeg>(Bs, dev);
+  }
 }
 
 }  // namespace

@@ -63,6 +63,12 @@ __device__ __forceinline__ void ck_load(float2 (&h)[N / 2], const float* ck, int
                        ck[((size_t)slot * N + 2 * j + 1) * kCta + threadIdx.x]);
 }
 
+// How a TMEM kernel walks a chunk: blocks of one segment, one at a time; tiles
+// of several shorter blocks; blocks of several 16-token segments, staged
+// segment by segment and pass by pass.
+constexpr int kOneSeg = 0, kTiles = 1, kSegs = 2;
+inline int bwd_kind(int64_t Bs, bool split) { return Bs > 16 ? kSegs : Bs < 16 && !split ? kTiles : kOneSeg; }
+
 // Tokens per backward segment; also the fixed stride of the staged tiles and
 // of the reduction buffer, so that their addresses are immediates.
 constexpr int kBwdTS = 16;
@@ -366,25 +372,23 @@ int resident_ctas(K kernel, size_t smem, uint32_t tcols, int dev) {
   return n;
 }
 
-// Shared memory of a launch, whether a block of several segments is staged
-// whole (one buffer per segment; only where that costs no resident CTA), and
-// the buffers of one-segment blocks: two, or, for fp32 inputs (ONE), one where
-// that leaves more CTAs on an SM (16 states: the noisy kernel's 132 KB admit
-// one CTA, its 78 KB with one buffer two; 8 x 2048 x 1536, blocks of 16: 1291
-// -> 855 us; the clean kernel gets three CTAs instead of two: 444 -> 378 us).
+// Shared memory of a launch and its staging buffers: two, or, for fp32 inputs
+// (ONE), one where that leaves more CTAs on an SM (16 states: the noisy
+// kernel's 132 KB admit one CTA, its 78 KB with one buffer two; 8 x 2048 x
+// 1536, blocks of 16: 1291 -> 855 us; the clean kernel gets three CTAs instead
+// of two: 444 -> 378 us; 4 x 2048 x 1024, blocks of 64: the step 851 -> 736 us).
 struct BwdLaunch {
   size_t smem;
-  int resident, bufs;
+  int bufs;
 };
 template <typename L, bool ONE, typename K>
 BwdLaunch bwd_launch(K kernel, int Bs, uint32_t cols, int dev) {
-  const int TS = Bs < 16 ? Bs : 16, nseg = Bs / TS;
-  if (nseg == 1 && !ONE) return {pad_for_tmem(L::bytes(2, TS, Bs), cols), 0, 2};
+  const int TS = Bs < 16 ? Bs : 16;
+  const size_t two = pad_for_tmem(L::bytes(2, TS, Bs), cols);
+  if (!ONE) return {two, 2};
   const size_t one = pad_for_tmem(L::bytes(1, TS, Bs), cols);
-  const size_t all = pad_for_tmem(L::bytes(nseg == 1 ? 2 : nseg, TS, Bs), cols);
-  const int r1 = resident_ctas(kernel, one, cols, dev), ra = resident_ctas(kernel, all, cols, dev);
-  if (ra >= r1 && ra > 0) return {all, nseg > 1, 2};
-  return {one, 0, 1};
+  return resident_ctas(kernel, one, cols, dev) > resident_ctas(kernel, two, cols, dev) ? BwdLaunch{one, 1}
+                                                                                      : BwdLaunch{two, 2};
 }
 }  // namespace
 

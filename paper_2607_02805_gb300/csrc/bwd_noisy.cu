@@ -7,14 +7,15 @@ namespace bds {
 // ---------------------------------------------------------------------------
 // Noisy blocks (both directions) + the clean stream's chunk-local adjoint
 // ---------------------------------------------------------------------------
-template <typename T, int N>
+template <typename T, int N, int KIND>
 struct NoisyBwdSmem {
-  // token-by-channel: x_n, dt_f, dt_r, dy_n, dt_c, dy_c; token-by-state: B_f, C_f, B_r, C_r, C_c
-  using St = Stage<T, N, 6, 5, 2, kBwdTS>;
-  // `bufs` staging buffers: for one-segment blocks 2 (the next block is copied
-  // while the current one is used) or, where that leaves more CTAs on an SM, 1;
-  // for longer blocks one per segment (the whole block resident) or 1 (each
-  // segment copied when needed)
+  // token-by-channel: x_n, dt_f, dt_r, dy_n, dt_c, dy_c; token-by-state: B_f, C_f, B_r, C_r, C_c.
+  // Blocks of several segments stage what one pass over a segment reads: at
+  // most three of the first (x_n, dt, dy_n; or dt_c, dy_c) and two of the
+  // second (B, C; or C_c)
+  using St = Stage<T, N, KIND == kSegs ? 3 : 6, KIND == kSegs ? 2 : 5, 2, kBwdTS>;
+  // `bufs` staging buffers: 2 (the next block, tile or segment is copied while
+  // the current one is used) or, where that leaves more CTAs on an SM, 1
   static __host__ __device__ size_t dx_off(int bufs) { return align16(St::buf_bytes(kBwdTS) * bufs); }
   // dx partials of a tile (several short blocks) or of one long block
   static __host__ __device__ size_t red_off(int bufs, int Bs) { return dx_off(bufs) + (size_t)(Bs < kBwdTS ? kBwdTS : Bs) * kCta * 4; }
@@ -29,15 +30,22 @@ struct NoisyBwdSmem {
   static __host__ __device__ size_t bytes(int bufs, int TS, int Bs) { return slot_off(bufs, TS, Bs) + 16; }
 };
 
-// TILED (blocks shorter than kBwdTS tokens): several blocks per staged tile.
+// KIND: how the chunk is walked (bwd_common.cuh). Blocks of several segments
+// make five passes over each: the clean local adjoint, and per direction the
+// checkpoints and the segments themselves. Each pass stages what it reads, and
+// the next pass's or segment's copies run under the current one's work (8 x
+// 2048 x 2048, blocks of 64: 1419 -> 1199 us against staging every tensor for
+// each pass). Blocks of one segment have their sizes at compile time (8 x 2048
+// x 1536, blocks of 16: 801 -> 738 us).
 // SPLIT (small problems, split_parts): the chunk is one block, and a CTA does
 // one of the three parts of its work, none of which reads what another makes.
-template <typename T, typename TO, int N, bool TILED, bool SPLIT>
+template <typename T, typename TO, int N, int KIND, bool SPLIT>
 __global__ void __launch_bounds__(kCta, 1) k_bwd_noisy(const BwdParams p) {
   pdl_sync();
-  static_assert(!(TILED && SPLIT), "a split launch has one block per CTA");
+  static_assert(!(KIND == kTiles && SPLIT), "a split launch has one block per CTA");
+  constexpr bool TILED = KIND == kTiles, SEGS = KIND == kSegs;
   extern __shared__ __align__(16) unsigned char smem[];
-  using L = NoisyBwdSmem<T, N>;
+  using L = NoisyBwdSmem<T, N, KIND>;
   const Geo& g = p.g;
   const int tid = threadIdx.x, warp = tid >> 5;
   const int sw = swz_of_lane<N>();
@@ -47,30 +55,32 @@ __global__ void __launch_bounds__(kCta, 1) k_bwd_noisy(const BwdParams p) {
   const int c = blockIdx.y;
   const int64_t d0 = (int64_t)blockIdx.x * kCta, d = d0 + tid;
   const bool act = d < g.D;
-  const int Bs = (int)g.Bs, TS = Bs < 16 ? Bs : 16, NSEG = Bs / TS;
+  const int Bs = KIND == kOneSeg && !SPLIT ? 16 : (int)g.Bs;
+  const int TS = SEGS || (KIND == kOneSeg && !SPLIT) ? 16 : Bs, NSEG = SEGS ? Bs / 16 : 1;
   const int k_lo = chunk_lo(g, c), k_hi = chunk_lo(g, c + 1) - 1;
   // debug build: the chunk's last token and the channel group lie inside the sizes
   if (!(dguard(kSiteBwdNoisy, b, g.Bt) && dguard(kSiteBwdNoisy, (int64_t)(k_hi + 1) * Bs - 1, g.L) &&
         dguard(kSiteBwdNoisy, d0, g.D)))
     return;
 
-  enum { XN = 0, DTF = 1, DTR = 2, DYN = 3, DTC = 4, DYC = 5 };
-  enum { BF = 0, CF = 1, BR = 2, CR = 3, CC = 4 };
+  constexpr int XN = 0, DTF = 1, DTR = SEGS ? 1 : 2, DYN = SEGS ? 2 : 3, DTC = SEGS ? 0 : 4, DYC = SEGS ? 1 : 5;
+  constexpr int BF = 0, CF = 1, BR = SEGS ? 0 : 2, CR = SEGS ? 1 : 3, CC = SEGS ? 0 : 4;
   typename L::St st;
   st.carve(smem, TS);
-  st.td_src[XN] = (const T*)p.xn;
-  st.td_src[DTF] = (const T*)p.dtf;
-  st.td_src[DTR] = (const T*)p.dtr;
-  st.td_src[DYN] = (const T*)p.dyn;
-  st.td_src[DTC] = (const T*)p.dtc;
-  st.td_src[DYC] = (const T*)p.dyc;
-  st.row_src[BF] = (const T*)p.Bf;
-  st.row_src[CF] = (const T*)p.Cf;
-  st.row_src[BR] = (const T*)p.Br;
-  st.row_src[CR] = (const T*)p.Cr;
-  st.row_src[CC] = (const T*)p.Cc;
-  const bool resident = NSEG > 1 && p.seg_resident;
-  const int bufs = NSEG == 1 ? (is_f32<T>::value ? p.stage_bufs : 2) : (resident ? NSEG : 1);
+  if constexpr (!SEGS) {
+    st.td_src[XN] = (const T*)p.xn;
+    st.td_src[DTF] = (const T*)p.dtf;
+    st.td_src[DTR] = (const T*)p.dtr;
+    st.td_src[DYN] = (const T*)p.dyn;
+    st.td_src[DTC] = (const T*)p.dtc;
+    st.td_src[DYC] = (const T*)p.dyc;
+    st.row_src[BF] = (const T*)p.Bf;
+    st.row_src[CF] = (const T*)p.Cf;
+    st.row_src[BR] = (const T*)p.Br;
+    st.row_src[CR] = (const T*)p.Cr;
+    st.row_src[CC] = (const T*)p.Cc;
+  }
+  const int bufs = is_f32<T>::value ? p.stage_bufs : 2;
   float* dxr_part = p.dx_part;  // SPLIT: where the two directions leave their share of dx
   float* dxf_part = SPLIT ? p.dx_part + g.Bt * g.L * g.D : nullptr;
   float* dxbuf = reinterpret_cast<float*>(smem + L::dx_off(bufs));
@@ -111,17 +121,55 @@ __global__ void __launch_bounds__(kCta, 1) k_bwd_noisy(const BwdParams p) {
   float2 dSn[N / 2];  // seed gradient of the block to the right of the current one
   vzero2<N>(dSn);
 
+  // SEGS: the steps (pass, segment) of a block in the order they are used, one
+  // step staged ahead. Passes 0: clean, 1 / 2: reverse checkpoints / segments,
+  // 3 / 4: forward checkpoints / segments.
+  int nk = k_hi, np = 0, ns = NSEG - 1, fill = 0, cur = 0;  // next step to copy, buffers
+  auto enter = [&](int pass) {
+    for (;; ++pass) {
+      if (pass > 4) {
+        pass = 0;
+        --nk;
+      }
+      if (pass == 0 ? do_clean : pass <= 2 ? do_rev : do_fwd) break;
+    }
+    np = pass;
+    ns = pass == 2 || pass == 3 ? 0 : NSEG - 1;
+  };
+  auto copy_step = [&]() {
+    if (nk < k_lo) return false;
+    const bool fwd = np >= 3, adj = np == 2 || np == 4;
+    st.td_src[0] = (const T*)(np == 0 ? p.dtc : p.xn);
+    st.td_src[1] = (const T*)(np == 0 ? p.dyc : fwd ? p.dtf : p.dtr);
+    st.row_src[0] = (const T*)(np == 0 ? p.Cc : fwd ? p.Bf : p.Br);
+    if constexpr (SEGS) {
+      st.td_src[2] = (const T*)p.dyn;
+      st.row_src[1] = (const T*)(fwd ? p.Cf : p.Cr);
+    }
+    st.issue_first(fill, b * g.L + (int64_t)nk * Bs + ns * TS, TS, g.D, d0, adj ? 3 : 2, adj ? 2 : 1);
+    fill ^= bufs - 1;
+    if (np == 2 || np == 3) {
+      if (++ns > (np == 2 ? NSEG - 1 : NSEG - 2)) enter(np + 1);
+    } else {
+      if (--ns < (np == 1 ? 1 : 0)) enter(np + 1);
+    }
+    return true;
+  };
+  auto next_step = [&](int nrow) {  // the next step's tiles become current
+    __syncthreads();                // the buffer to fill is no longer read
+    const bool ahead = copy_step() && bufs == 2;
+    st.complete(cur, TS, ahead ? 1 : 0, nrow);
+    cur ^= bufs - 1;
+  };
+  if (SEGS) {
+    enter(0);
+    if (bufs == 2) copy_step();
+  }
+
   // everything for block k, whose tokens start at `off` in the staged tile
   auto block = [&](int k, int off) {
     const int64_t t0 = (int64_t)k * Bs;
     const int64_t row0 = b * g.L + t0;
-    // make segment s current: staged now, or already resident
-    auto stage_seg = [&](int s) {
-      if (resident)
-        st.select(s);
-      else
-        st.load(row0 + (int64_t)s * TS, TS, g.D, d0);
-    };
 
     // ---- clean stream: chunk-local adjoint over block k ----
     if (k < k_hi) {
@@ -135,7 +183,7 @@ __global__ void __launch_bounds__(kCta, 1) k_bwd_noisy(const BwdParams p) {
       }
     }
     if (do_clean) for (int s = NSEG - 1; s >= 0; --s) {
-      if (NSEG > 1) stage_seg(s);
+      if (SEGS) next_step(1);
 #pragma unroll 4
       for (int i = TS - 1; i >= 0; --i) {
         const float dt = st.at(DTC, off + i), dy = st.at(DYC, off + i);
@@ -150,11 +198,11 @@ __global__ void __launch_bounds__(kCta, 1) k_bwd_noisy(const BwdParams p) {
 
     // ---- noisy block k, reverse direction (zero state at the block end) ----
     if (do_rev) {
-      if (NSEG > 1) {
+      if (SEGS) {
         float2 h[N / 2];
         vzero2<N>(h);
         for (int s = NSEG - 1; s >= 1; --s) {
-          stage_seg(s);
+          next_step(1);
 #pragma unroll 4
           for (int i = TS - 1; i >= 0; --i) scan_state_swz<N>(h, A2r, st.at(DTR, i), st.at(XN, i), st.row(BR, i), sw);
           ck_store<N>(ck, s - 1, h);
@@ -163,7 +211,7 @@ __global__ void __launch_bounds__(kCta, 1) k_bwd_noisy(const BwdParams p) {
       float2 gr[N / 2];  // a_{t-1} gbar_{t-1}, entering token t from the left
       vzero2<N>(gr);
       for (int s = 0; s < NSEG; ++s) {
-        if (NSEG > 1) stage_seg(s);
+        if (SEGS) next_step(2);
         float2 h[N / 2];
         if (s == NSEG - 1)
           vzero2<N>(h);
@@ -191,12 +239,12 @@ __global__ void __launch_bounds__(kCta, 1) k_bwd_noisy(const BwdParams p) {
       float2 seed[N / 2];
       vzero2<N>(seed);
       if (k > 0 && act) vload2<N>(seed, p.states + ((b * g.nb + (k - 1)) * g.D + d) * N, sw);
-      if (NSEG > 1) {
+      if (SEGS) {
         float2 h[N / 2];
 #pragma unroll
         for (int j = 0; j < N / 2; ++j) h[j] = seed[j];
         for (int s = 0; s < NSEG - 1; ++s) {
-          stage_seg(s);
+          next_step(1);
 #pragma unroll 4
           for (int i = 0; i < TS; ++i) scan_state_swz<N>(h, A2f, st.at(DTF, i), st.at(XN, i), st.row(BF, i), sw);
           ck_store<N>(ck, s, h);
@@ -205,7 +253,7 @@ __global__ void __launch_bounds__(kCta, 1) k_bwd_noisy(const BwdParams p) {
       float2 gf[N / 2];  // a_{t+1} gbar_{t+1}, entering token t from the right
       vzero2<N>(gf);
       for (int s = NSEG - 1; s >= 0; --s) {
-        if (NSEG > 1) stage_seg(s);
+        if (SEGS) next_step(2);
         float2 h[N / 2];
         if (s == 0) {
 #pragma unroll
@@ -261,23 +309,19 @@ __global__ void __launch_bounds__(kCta, 1) k_bwd_noisy(const BwdParams p) {
       if (do_fwd) red_flush<N>(p, red, 2, 3, 2, 3, b, ts0, nbk * Bs);
       kt_hi = kt_lo - 1;
     }
+  } else if (SEGS) {
+    for (int k = k_hi; k >= k_lo; --k) block(k, 0);
   } else {
-    // one-segment blocks, two buffers: block k-1 is copied while block k is processed
-    if (NSEG == 1 && bufs == 2) st.issue(0, b * g.L + (int64_t)k_hi * Bs, TS, g.D, d0);
+    // two buffers: block k-1 is copied while block k is processed
+    if (bufs == 2) st.issue(0, b * g.L + (int64_t)k_hi * Bs, TS, g.D, d0);
     for (int k = k_hi; k >= k_lo; --k) {
       const int64_t row0 = b * g.L + (int64_t)k * Bs;
-      if (NSEG == 1) {
-        const int buf = bufs == 2 ? (k_hi - k) & 1 : 0;
-        const bool ahead = bufs == 2 && k > k_lo;
-        __syncthreads();  // the buffer to fill is no longer read
-        if (bufs == 1) st.issue(0, row0, TS, g.D, d0);
-        if (ahead) st.issue(buf ^ 1, row0 - Bs, TS, g.D, d0);
-        st.complete(buf, TS, ahead ? 1 : 0);
-      } else if (resident) {  // every segment of the block, once
-        __syncthreads();  // the previous block is no longer read
-        for (int s = 0; s < NSEG; ++s) st.issue(s, row0 + (int64_t)s * TS, TS, g.D, d0);
-        for (int s = 0; s < NSEG; ++s) st.complete(s, TS, 0);
-      }
+      const int buf = bufs == 2 ? (k_hi - k) & 1 : 0;
+      const bool ahead = bufs == 2 && k > k_lo;
+      __syncthreads();  // the buffer to fill is no longer read
+      if (bufs == 1) st.issue(0, row0, TS, g.D, d0);
+      if (ahead) st.issue(buf ^ 1, row0 - Bs, TS, g.D, d0);
+      st.complete(buf, TS, ahead ? 1 : 0);
       block(k, 0);
     }
   }
@@ -300,40 +344,47 @@ __global__ void __launch_bounds__(kCta, 1) k_bwd_noisy(const BwdParams p) {
 
 namespace {
 
-template <typename T, typename TO, int N, bool TILED, bool SPLIT>
+template <typename T, typename TO, int N, int KIND, bool SPLIT>
 BwdLaunch noisy_launch(int Bs, int dev) {
-  const int TS = Bs < 16 ? Bs : 16;
-  return bwd_launch<NoisyBwdSmem<T, N>, is_f32<T>::value>(k_bwd_noisy<T, TO, N, TILED, SPLIT>, Bs, full_cols(TS, N), dev);
+  return bwd_launch<NoisyBwdSmem<T, N, KIND>, is_f32<T>::value>(k_bwd_noisy<T, TO, N, KIND, SPLIT>, Bs,
+                                                               full_cols(Bs < 16 ? Bs : 16, N), dev);
 }
-template <typename T, typename TO, int N, bool TILED, bool SPLIT>
+template <typename T, typename TO, int N, int KIND, bool SPLIT>
 cudaError_t bwd_noisy_tt(const BwdParams& p_in, cudaStream_t s) {
   int dev = 0;
   cudaError_t e = cudaGetDevice(&dev);
   if (e != cudaSuccess) return e;
-  const BwdLaunch l = noisy_launch<T, TO, N, TILED, SPLIT>((int)p_in.g.Bs, dev);
+  const BwdLaunch l = noisy_launch<T, TO, N, KIND, SPLIT>((int)p_in.g.Bs, dev);
   BwdParams p = p_in;
-  p.seg_resident = l.resident;
   p.stage_bufs = l.bufs;
-  e = set_bwd_attrs(k_bwd_noisy<T, TO, N, TILED, SPLIT>, l.smem);
+  e = set_bwd_attrs(k_bwd_noisy<T, TO, N, KIND, SPLIT>, l.smem);
   if (e != cudaSuccess) return e;
   dim3 grid((unsigned)p.g.G, (unsigned)p.g.nc, (unsigned)(SPLIT ? 3 * p.g.Bt : p.g.Bt));
-  launch_pdl(k_bwd_noisy<T, TO, N, TILED, SPLIT>, grid, kCta, l.smem, s, p);
+  launch_pdl(k_bwd_noisy<T, TO, N, KIND, SPLIT>, grid, kCta, l.smem, s, p);
   return cudaGetLastError();
 }
 template <typename T, typename TO, int N>
 cudaError_t bwd_noisy_t(const BwdParams& p, cudaStream_t s) {
-  if (p.dx_part != nullptr) return bwd_noisy_tt<T, TO, N, false, true>(p, s);
-  return p.g.Bs < kBwdTS ? bwd_noisy_tt<T, TO, N, true, false>(p, s) : bwd_noisy_tt<T, TO, N, false, false>(p, s);
+  const bool split = p.dx_part != nullptr;
+  switch (bwd_kind(p.g.Bs, split)) {
+    case kTiles: return bwd_noisy_tt<T, TO, N, kTiles, false>(p, s);
+    case kSegs: return split ? bwd_noisy_tt<T, TO, N, kSegs, true>(p, s) : bwd_noisy_tt<T, TO, N, kSegs, false>(p, s);
+    default: return split ? bwd_noisy_tt<T, TO, N, kOneSeg, true>(p, s) : bwd_noisy_tt<T, TO, N, kOneSeg, false>(p, s);
+  }
 }
 
+template <typename T, typename TO, int N, int KIND>
+int noisy_resident(int Bs, int dev) {
+  return resident_ctas(k_bwd_noisy<T, TO, N, KIND, false>, noisy_launch<T, TO, N, KIND, false>(Bs, dev).smem,
+                       full_cols(Bs < 16 ? Bs : 16, N), dev);
+}
 template <typename T, typename TO, int N>
 int bwd_noisy_per_sm_t(int Bs, int dev) {
-  const int TS = Bs < 16 ? Bs : 16;
-  if (Bs < kBwdTS)
-    return resident_ctas(k_bwd_noisy<T, TO, N, true, false>, noisy_launch<T, TO, N, true, false>(Bs, dev).smem,
-                         full_cols(TS, N), dev);
-  return resident_ctas(k_bwd_noisy<T, TO, N, false, false>, noisy_launch<T, TO, N, false, false>(Bs, dev).smem,
-                       full_cols(TS, N), dev);
+  switch (bwd_kind(Bs, false)) {
+    case kTiles: return noisy_resident<T, TO, N, kTiles>(Bs, dev);
+    case kSegs: return noisy_resident<T, TO, N, kSegs>(Bs, dev);
+    default: return noisy_resident<T, TO, N, kOneSeg>(Bs, dev);
+  }
 }
 
 }  // namespace

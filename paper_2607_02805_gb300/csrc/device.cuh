@@ -204,9 +204,23 @@ struct Stage {
     for (int j = 0; j < NROW; ++j) issue_rows<T, N, REV>(r + (size_t)j * stride() * N, row_src[j], row0, nsteps);
     cp_async_commit();
   }
+  // The same for the first `ntd` token-by-channel tensors and the first `nrow`
+  // token-by-state ones only.
+  __device__ void issue_first(int buf, int64_t row0, int nsteps, int64_t D, int64_t d0, int ntd, int nrow) {
+    T* t = td(buf);
+    T* r = raw(buf);
+#pragma unroll
+    for (int j = 0; j < NTD; ++j)
+      if (j < ntd) issue_td<T, REV>(t + (size_t)j * stride() * kCta, td_src[j], row0, nsteps, D, d0);
+#pragma unroll
+    for (int j = 0; j < NROW; ++j)
+      if (j < nrow) issue_rows<T, N, REV>(r + (size_t)j * stride() * N, row_src[j], row0, nsteps);
+    cp_async_commit();
+  }
   // Waits for the copies of buffer `buf` (with `pending` newer groups still in
-  // flight), widens its B/C rows to fp32 and makes it the current buffer.
-  __device__ void complete(int buf, int nsteps, int pending) {
+  // flight), widens its (first `nrow`) B/C rows to fp32 and makes it the
+  // current buffer.
+  __device__ void complete(int buf, int nsteps, int pending, int nrow = NROW) {
     if (pending)
       cp_async_wait_one();
     else
@@ -218,6 +232,7 @@ struct Stage {
       float* f = rows(buf);
 #pragma unroll
       for (int j = 0; j < NROW; ++j) {
+        if (j >= nrow) break;
         const T* rj = r + (size_t)j * stride() * N;
         float* fj = f + (size_t)j * stride() * N;
         for (int q = threadIdx.x; q < half; q += kCta)
