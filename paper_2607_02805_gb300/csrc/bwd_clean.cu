@@ -24,7 +24,7 @@ struct CleanBwdSmem {
   }
 };
 
-// KIND: how the chunk is walked (bwd_common.cuh). Blocks of several segments
+// KIND: how the chunk is walked (params.h). Blocks of several segments
 // make two passes, the checkpoints and the segments, each staging what it
 // reads, one segment ahead.
 template <typename T, typename TO, int N, int KIND>
@@ -248,7 +248,7 @@ cudaError_t bwd_clean_tt(const BwdParams& p_in, cudaStream_t s) {
 }
 template <typename T, typename TO, int N>
 cudaError_t bwd_clean_t(const BwdParams& p, cudaStream_t s) {
-  switch (bwd_kind(p.g.Bs, false)) {
+  switch (block_kind(p.g.Bs)) {
     case kTiles: return bwd_clean_tt<T, TO, N, kTiles>(p, s);
     case kSegs: return bwd_clean_tt<T, TO, N, kSegs>(p, s);
     default: return bwd_clean_tt<T, TO, N, kOneSeg>(p, s);
@@ -262,7 +262,7 @@ int clean_resident(int Bs, int dev) {
 }
 template <typename T, typename TO, int N>
 int bwd_clean_per_sm_t(int Bs, int dev) {
-  switch (bwd_kind(Bs, false)) {
+  switch (block_kind(Bs)) {
     case kTiles: return clean_resident<T, TO, N, kTiles>(Bs, dev);
     case kSegs: return clean_resident<T, TO, N, kSegs>(Bs, dev);
     default: return clean_resident<T, TO, N, kOneSeg>(Bs, dev);

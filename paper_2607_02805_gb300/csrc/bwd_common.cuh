@@ -63,12 +63,6 @@ __device__ __forceinline__ void ck_load(float2 (&h)[N / 2], const float* ck, int
                        ck[((size_t)slot * N + 2 * j + 1) * kCta + threadIdx.x]);
 }
 
-// How a TMEM kernel walks a chunk: blocks of one segment, one at a time; tiles
-// of several shorter blocks; blocks of several 16-token segments, staged
-// segment by segment and pass by pass.
-constexpr int kOneSeg = 0, kTiles = 1, kSegs = 2;
-inline int bwd_kind(int64_t Bs, bool split) { return Bs > 16 ? kSegs : Bs < 16 && !split ? kTiles : kOneSeg; }
-
 // Tokens per backward segment; also the fixed stride of the staged tiles and
 // of the reduction buffer, so that their addresses are immediates.
 constexpr int kBwdTS = 16;

@@ -30,7 +30,7 @@ struct NoisyBwdSmem {
   static __host__ __device__ size_t bytes(int bufs, int TS, int Bs) { return slot_off(bufs, TS, Bs) + 16; }
 };
 
-// KIND: how the chunk is walked (bwd_common.cuh). Blocks of several segments
+// KIND: how the chunk is walked (params.h). Blocks of several segments
 // make five passes over each: the clean local adjoint, and per direction the
 // checkpoints and the segments themselves. Each pass stages what it reads, and
 // the next pass's or segment's copies run under the current one's work (8 x
@@ -366,7 +366,7 @@ cudaError_t bwd_noisy_tt(const BwdParams& p_in, cudaStream_t s) {
 template <typename T, typename TO, int N>
 cudaError_t bwd_noisy_t(const BwdParams& p, cudaStream_t s) {
   const bool split = p.dx_part != nullptr;
-  switch (bwd_kind(p.g.Bs, split)) {
+  switch (split && p.g.Bs < 16 ? kOneSeg : block_kind(p.g.Bs)) {
     case kTiles: return bwd_noisy_tt<T, TO, N, kTiles, false>(p, s);
     case kSegs: return split ? bwd_noisy_tt<T, TO, N, kSegs, true>(p, s) : bwd_noisy_tt<T, TO, N, kSegs, false>(p, s);
     default: return split ? bwd_noisy_tt<T, TO, N, kOneSeg, true>(p, s) : bwd_noisy_tt<T, TO, N, kOneSeg, false>(p, s);
@@ -380,7 +380,7 @@ int noisy_resident(int Bs, int dev) {
 }
 template <typename T, typename TO, int N>
 int bwd_noisy_per_sm_t(int Bs, int dev) {
-  switch (bwd_kind(Bs, false)) {
+  switch (block_kind(Bs)) {
     case kTiles: return noisy_resident<T, TO, N, kTiles>(Bs, dev);
     case kSegs: return noisy_resident<T, TO, N, kSegs>(Bs, dev);
     default: return noisy_resident<T, TO, N, kOneSeg>(Bs, dev);

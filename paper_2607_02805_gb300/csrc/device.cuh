@@ -249,6 +249,12 @@ struct Stage {
     issue(0, row0, nsteps, D, d0);
     complete(0, nsteps, 0);
   }
+  // The same for the first `ntd` and `nrow` tensors.
+  __device__ void load_first(int64_t row0, int nsteps, int64_t D, int64_t d0, int ntd, int nrow) {
+    __syncthreads();
+    issue_first(0, row0, nsteps, D, d0, ntd, nrow);
+    complete(0, nsteps, 0, nrow);
+  }
   __device__ __forceinline__ float at(int j, int step) const {
     return cvt(cur_td[(j * stride() + step) * kCta]);
   }

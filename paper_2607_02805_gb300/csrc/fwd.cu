@@ -181,12 +181,16 @@ struct ScanLayout {
   static constexpr int BF = 2, CF = BF + 1, BR = BF + 2, CR = BF + 3;
 };
 
-// TILED (blocks shorter than kScanSeg): several blocks per staged tile.
+// KIND: how the chunk is walked (params.h). The clean scans copy the next block,
+// tile or segment while the current one is scanned; in mode 0 a second buffer
+// would cost a resident CTA per SM, which measured slower than the overlap it
+// buys. There the forward pass over a segment stages the clean and forward
+// tensors, the reverse pass its own.
 // The stride of the staged tiles is fixed at kScanSeg tokens, so a token's
 // addresses are immediates (16 tokens, 8 x 2048 x 1536 x 16, mode 0: 336 ->
 // 321 us). The clean scans alone fit six CTAs per SM (65,536 x 2048 x 16,
 // mode 1: 545 us with four, 528 with five, 520 with six, 610 with seven).
-template <typename T, typename TO, int N, int MODE, bool TILED>
+template <typename T, typename TO, int N, int MODE, int KIND>
 __global__ void __launch_bounds__(kCta, MODE == 0 ? 4 : 6) k_block_scan(const FwdParams p) {
   pdl_sync();
   using Ly = ScanLayout<MODE>;
@@ -200,8 +204,9 @@ __global__ void __launch_bounds__(kCta, MODE == 0 ? 4 : 6) k_block_scan(const Fw
   if (!(dguard(kSiteBlockScan, b, g.Bt) && dguard(kSiteBlockScan, (int64_t)c * g.m * g.Bs, g.L) &&
         dguard(kSiteBlockScan, d0, g.D)))
     return;
-  const int Bs = (int)g.Bs;
-  const int SEG = Bs < kScanSeg ? Bs : kScanSeg, NSEG = (Bs + SEG - 1) / SEG;
+  constexpr bool SEGS = KIND == kSegs, TILED = KIND == kTiles;
+  const int Bs = KIND == kOneSeg ? kScanSeg : (int)g.Bs;
+  const int SEG = TILED ? Bs : kScanSeg, NSEG = SEGS ? (Bs + SEG - 1) / SEG : 1;
   // blocks shorter than kScanSeg are staged TB at a time (one tile of at most
   // kScanSeg tokens), so the staging and its barriers are paid per tile
   const int TB = TILED ? kScanSeg / Bs : 1;
@@ -210,9 +215,8 @@ __global__ void __launch_bounds__(kCta, MODE == 0 ? 4 : 6) k_block_scan(const Fw
   st.carve(smem, kScanSeg);
   // the row holding logical row x = b L + t (t reversed in time for MODE 2)
   auto prow = [&](int64_t x) { return kRev ? 2 * b * g.L + g.L - 1 - x : x; };
-  const bool dbuf = p.stage_bufs == 2 && NSEG == 1;
-  float* yfbuf = reinterpret_cast<float*>(smem + decltype(st)::buf_bytes(st.stride()) *
-                                                       (dbuf ? 2 : 1));
+  constexpr bool dbuf = !Ly::kNoisy;
+  float* yfbuf = reinterpret_cast<float*>(smem + decltype(st)::buf_bytes(kScanSeg));  // mode 0
   if (Ly::kClean) {
     st.td_src[Ly::XC] = (const T*)p.xc;
     st.td_src[Ly::DTC] = (const T*)p.dtc;
@@ -254,16 +258,30 @@ __global__ void __launch_bounds__(kCta, MODE == 0 ? 4 : 6) k_block_scan(const Fw
   if (act) vload2<N>(hc, p.hst + ((b * (g.nc + 1) + c) * g.D + d) * N, 0);
 
   auto tile_blocks = [&](int k0) { return k_hi - k0 + 1 < TB ? k_hi - k0 + 1 : TB; };
-  if (dbuf) st.issue(0, prow(b * g.L + (int64_t)k_lo * Bs), tile_blocks(k_lo) * Bs, g.D, d0);
+  // SEGS, clean scans: the chunk's segments in order, one copied ahead
+  int nk = k_lo, ns0 = 0, fill = 0, cur = 0;  // next segment to copy (block, first token), buffers
+  auto copy_seg = [&]() {
+    if (nk > k_hi) return false;
+    st.issue(fill, prow(b * g.L + (int64_t)nk * Bs + ns0), Bs - ns0 < SEG ? Bs - ns0 : SEG, g.D, d0);
+    fill ^= 1;
+    ns0 += SEG;
+    if (ns0 >= Bs) {
+      ns0 = 0;
+      ++nk;
+    }
+    return true;
+  };
+  if (dbuf && SEGS) copy_seg();
+  if (dbuf && !SEGS) st.issue(0, prow(b * g.L + (int64_t)k_lo * Bs), tile_blocks(k_lo) * Bs, g.D, d0);
   for (int k0 = k_lo; k0 <= k_hi; k0 += TB) {
     const int nbk = tile_blocks(k0), tile = (k0 - k_lo) / TB;
     const int64_t trow = b * g.L + (int64_t)k0 * Bs;
-    if (dbuf) {
+    if (dbuf && !SEGS) {
       __syncthreads();  // the other buffer is no longer read
       const int k1 = k0 + TB;
       if (k1 <= k_hi) st.issue((tile + 1) & 1, prow(trow + (int64_t)nbk * Bs), tile_blocks(k1) * Bs, g.D, d0);
       st.complete(tile & 1, nbk * Bs, k1 <= k_hi ? 1 : 0);
-    } else if (NSEG == 1) {
+    } else if (!SEGS) {
       st.load(prow(trow), nbk * Bs, g.D, d0);
     }
     for (int kk = 0; kk < nbk; ++kk) {
@@ -275,7 +293,18 @@ __global__ void __launch_bounds__(kCta, MODE == 0 ? 4 : 6) k_block_scan(const Fw
       for (int j = 0; j < N / 2; ++j) hs[j] = hc[j];  // the block's seed: state before its first token
       for (int sg = 0; sg < NSEG; ++sg) {  // segments left to right
         const int i0 = sg * SEG, ns = Bs - i0 < SEG ? Bs - i0 : SEG;
-        if (NSEG > 1) st.load(prow(row0 + i0), ns, g.D, d0);
+        if (SEGS && dbuf) {
+          __syncthreads();  // the other buffer is no longer read
+          const bool ahead = copy_seg();
+          st.complete(cur, ns, ahead ? 1 : 0);
+          cur ^= 1;
+        } else if (SEGS) {
+          st.td_src[0] = (const T*)p.xc;
+          st.td_src[1] = (const T*)p.dtc;
+          st.row_src[0] = (const T*)p.Bc;
+          st.row_src[1] = (const T*)p.Cc;
+          st.load_first(row0 + i0, ns, g.D, d0, 4, 4);  // x_c, dt_c, x_n, dt_f; B_c, C_c, B_f, C_f
+        }
         int64_t o = prow(row0 + i0) * g.D + d;  // the token's element, stepped
 #pragma unroll 2
         for (int ii = 0; ii < ns; ++ii, o += kRev ? -g.D : g.D) {
@@ -305,15 +334,23 @@ __global__ void __launch_bounds__(kCta, MODE == 0 ? 4 : 6) k_block_scan(const Fw
       if (Ly::kNoisy) {
         float2 hr[N / 2];
         vzero2<N>(hr);
-        for (int sg = NSEG - 1; sg >= 0; --sg) {  // segments right to left; the last is still staged
+        // SEGS: the reverse pass stages its tensors in the first slots
+        constexpr int XR = SEGS ? 0 : Ly::XN, DTR = SEGS ? 1 : Ly::DTR, BR = SEGS ? 0 : Ly::BR, CR = SEGS ? 1 : Ly::CR;
+        for (int sg = NSEG - 1; sg >= 0; --sg) {  // segments right to left
           const int i0 = sg * SEG, ns = Bs - i0 < SEG ? Bs - i0 : SEG;
-          if (sg < NSEG - 1) st.load(prow(row0 + i0), ns, g.D, d0);
+          if (SEGS) {
+            st.td_src[0] = (const T*)p.xn;
+            st.td_src[1] = (const T*)p.dtr;
+            st.row_src[0] = (const T*)p.Br;
+            st.row_src[1] = (const T*)p.Cr;
+            st.load_first(row0 + i0, ns, g.D, d0, 2, 2);
+          }
           int64_t o = prow(row0 + i0 + ns - 1) * g.D + d;
 #pragma unroll 2
           for (int ii = ns - 1; ii >= 0; --ii, o -= g.D) {  // noisy streams are never reversed
             const int i = i0 + ii;
-            const float x = st.at(Ly::XN, toff + ii), dt = st.at(Ly::DTR, toff + ii);
-            const float y = scan_step<N>(hr, A2r, dt, x, st.row(Ly::BR, toff + ii), st.row(Ly::CR, toff + ii));
+            const float x = st.at(XR, toff + ii), dt = st.at(DTR, toff + ii);
+            const float y = scan_step<N>(hr, A2r, dt, x, st.row(BR, toff + ii), st.row(CR, toff + ii));
             if (act)
               reinterpret_cast<TO*>(p.yn)[o] =
                   to_out<TO>(combine_dirs(yfbuf[i * kCta + threadIdx.x], with_skip(y, Dr, x)));
@@ -540,45 +577,25 @@ cudaError_t chunk_local_t(const FwdParams& p, cudaStream_t s) {
   return p.rev ? chunk_local_rt<T, N, true>(p, s) : chunk_local_rt<T, N, false>(p, s);
 }
 
-// Above this much shared memory per CTA the block scan stages synchronously:
-// at 16-token blocks a second buffer would cost a resident CTA per SM, which
-// measured slower than the overlap it buys.
-constexpr size_t kDoubleBufferLimit = 48 * 1024;
-
-template <typename T, typename TO, int N, int MODE>
-int block_scan_bufs_t(int64_t Bs) {
+template <typename T, typename TO, int N, int MODE, int KIND>
+cudaError_t block_scan_k(int nchunks, const FwdParams& p, cudaStream_t s) {
   using Ly = ScanLayout<MODE>;
-  if (Bs > kScanSeg) return 1;  // segments are staged when needed
-  const size_t extra = Ly::kNoisy ? (size_t)Bs * kCta * sizeof(float) : 0;
-  return 2 * Stage<T, N, Ly::NTD, Ly::NROW, 2>::buf_bytes(kScanSeg) + extra <= kDoubleBufferLimit ? 2 : 1;
-}
-
-template <typename T, typename TO, int N, int MODE>
-size_t block_scan_smem_t(int64_t Bs) {
-  using Ly = ScanLayout<MODE>;
-  size_t b = Stage<T, N, Ly::NTD, Ly::NROW, 2>::buf_bytes(kScanSeg) * block_scan_bufs_t<T, TO, N, MODE>(Bs);
-  if (Ly::kNoisy) b += (size_t)Bs * kCta * sizeof(float);
-  return b;
-}
-
-template <typename T, typename TO, int N, int MODE>
-cudaError_t block_scan_t(int nchunks, const FwdParams& p_in, cudaStream_t s) {
-  FwdParams p = p_in;
-  p.stage_bufs = block_scan_bufs_t<T, TO, N, MODE>(p.g.Bs);
-  const size_t smem = block_scan_smem_t<T, TO, N, MODE>(p.g.Bs);
+  const size_t buf = Stage<T, N, Ly::NTD, Ly::NROW, 2>::buf_bytes(kScanSeg);
+  const size_t smem = Ly::kNoisy ? buf + (size_t)p.g.Bs * kCta * sizeof(float) : 2 * buf;
+  cudaError_t e = cudaFuncSetAttribute(k_block_scan<T, TO, N, MODE, KIND>,
+                                       cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
+  if (e != cudaSuccess) return e;
   dim3 grid((unsigned)p.g.G, (unsigned)nchunks, (unsigned)p.g.Bt);
-  if (p.g.Bs < kScanSeg) {
-    cudaError_t e = cudaFuncSetAttribute(k_block_scan<T, TO, N, MODE, true>,
-                                         cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
-    if (e != cudaSuccess) return e;
-    launch_pdl(k_block_scan<T, TO, N, MODE, true>, grid, kCta, smem, s, p);
-  } else {
-    cudaError_t e = cudaFuncSetAttribute(k_block_scan<T, TO, N, MODE, false>,
-                                         cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
-    if (e != cudaSuccess) return e;
-    launch_pdl(k_block_scan<T, TO, N, MODE, false>, grid, kCta, smem, s, p);
-  }
+  launch_pdl(k_block_scan<T, TO, N, MODE, KIND>, grid, kCta, smem, s, p);
   return cudaGetLastError();
+}
+template <typename T, typename TO, int N, int MODE>
+cudaError_t block_scan_t(int nchunks, const FwdParams& p, cudaStream_t s) {
+  switch (block_kind(p.g.Bs)) {
+    case kTiles: return block_scan_k<T, TO, N, MODE, kTiles>(nchunks, p, s);
+    case kSegs: return block_scan_k<T, TO, N, MODE, kSegs>(nchunks, p, s);
+    default: return block_scan_k<T, TO, N, MODE, kOneSeg>(nchunks, p, s);
+  }
 }
 
 template <typename T, typename TO, int N>

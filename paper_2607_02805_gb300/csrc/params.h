@@ -36,7 +36,6 @@ struct FwdParams {
   const float* init;   // [Bt][D][N] or null: state before token 0
   const float* seed;   // active block: [Bt][D][N]
   int c_begin;         // first chunk handled by a block-scan launch
-  int stage_bufs;      // block scan: 2 = copy the next block while computing, 1 = synchronous
   int carry_last_only; // chunk carry: only the state after the last full chunk is read afterwards
   int rev;             // chunk-local scan: right to left in time (with block-scan mode 2)
   // active block with adaptive layer norm: per batch row shift, scale, gate
@@ -74,6 +73,11 @@ struct BwdParams {
   float* ck_noisy;
   float* ck_clean;
 };
+
+// How the scan and TMEM kernels walk a chunk: blocks of one 16-token segment,
+// one at a time; tiles of several shorter blocks; blocks of several segments.
+constexpr int kOneSeg = 0, kTiles = 1, kSegs = 2;
+inline int block_kind(int64_t Bs) { return Bs > 16 ? kSegs : Bs < 16 ? kTiles : kOneSeg; }
 
 // Launchers (fwd.cu / bwd.cu). dt: 0 = f32 in/out, 1 = bf16 in/out, 2 = bf16 in, f32 out.
 cudaError_t launch_chunk_local(int dt, int N, const FwdParams& p, cudaStream_t s);
