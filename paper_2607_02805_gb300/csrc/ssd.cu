@@ -248,13 +248,17 @@ __global__ void __launch_bounds__(256) k_ssd_state_pass(const SsdPassParams p) {
 }
 
 // Copies one 128-token tile of a [tokens][N] bf16 tensor into K-major
-// swizzled shared memory (N / 64 atom columns).
+// swizzled shared memory (N / 64 atom columns), by threads 0..255. A thread's
+// pieces are 8 or more rows apart in one column: both addresses are stepped.
 template <int N>
 __device__ __forceinline__ void stage_rows(unsigned char* dst, const __nv_bfloat16* src, const RowMap& tok, int row0) {
-  for (int c = threadIdx.x; c < 128 * N / 8; c += blockDim.x) {
-    const int r = c / (N / 8), ch = c % (N / 8);
-    cp_async16(dst + (ch >> 3) * kTile16 + sw128(r, ch & 7), src + tok(row0 + r) * N + ch * 8, 16);
-  }
+  constexpr int CPR = N / 8, RPP = 256 / CPR;
+  const int r = (int)threadIdx.x / CPR, ch = (int)threadIdx.x % CPR;
+  unsigned char* d = dst + (ch >> 3) * kTile16 + sw128(r, ch & 7);
+  const __nv_bfloat16* p = src + tok(row0 + r) * N + ch * 8;
+  const int64_t step = tok.step * (RPP * N);
+#pragma unroll
+  for (int q = 0; q < 128 / RPP; ++q, p += step) cp_async16(d + q * RPP * 128, p, 16);
 }
 
 // Gram product D[128 x 128] = A_rows . B_rows^T over K = N (both K-major).
@@ -303,12 +307,26 @@ struct ScanSmem {
   }
 };
 
-constexpr int kScanThreads = 256;
-constexpr int kScanIssuer = 128;  // the thread that issues a head's MMAs
+constexpr int kScanThreads = 256;                 // the eight warps that stage, build and write out
+constexpr int kScanNinth = kScanThreads + 32;     // and, in clean scans, a ninth that issues copies and MMAs
+constexpr int kScanIssuer = 128;                  // the thread that issues them in noisy ones
+template <bool NOISY>
+constexpr bool kHasNinth = !NOISY;
+template <bool NOISY>
+constexpr int kScanCta = kHasNinth<NOISY> ? kScanNinth : kScanThreads;
 constexpr int kMaxHeadsPerCta = 16;
 
+// Named barriers between the eight working warps, which arrive and go on, and
+// the issuing warp, which waits: a mixing tile (0 or 1) is in shared memory.
+__device__ __forceinline__ void tile_arrive(int j) {
+  asm volatile("bar.arrive %0, %1;\n" ::"r"(1 + j), "n"(kScanNinth) : "memory");
+}
+__device__ __forceinline__ void tile_wait(int j) {
+  asm volatile("bar.sync %0, %1;\n" ::"r"(1 + j), "n"(kScanNinth) : "memory");
+}
+
 // Issues the cp.async copies of one head's x tiles (MN-major) and its seed
-// (fp32, as stored) for a CTA of kScanThreads threads.
+// (fp32, as stored) by threads 0..255.
 template <int N>
 __device__ __forceinline__ void issue_head_loads(unsigned char* sm, const ScanSmem& L, const __nv_bfloat16* x,
                                                  const RowMap& tok, int H, int h, int ntile, const float* seed_h,
@@ -368,8 +386,15 @@ __device__ __forceinline__ void setup_dir(const T* dt, int hs, int n, float A2, 
   }
 }
 
-// One CTA of 8 warps per (batch row, block, 128-token tile i of the block)
-// and group of at most 16 heads. Warp w serves token rows 32 (w % 4) .. +31 of
+// One CTA of 8 working warps per (batch row, block, 128-token tile i of the
+// block) and group of at most 16 heads. The thread that issues MMAs is held
+// while the tensor pipe takes a head's 24 to 32 of them, about 80 cycles each.
+// In clean scans a ninth warp issues them and the copies, so that the seed's
+// MMAs run under the first tile's building and no building waits for the
+// issue: 371 -> 355 us (8 x 8192 x 26 x 128) against thread 128, whose warp has
+// the least mixing work on a diagonal tile. In noisy scans, whose tiles take
+// twice the registers, nine warps at 168 registers cost more (467 -> 540 us).
+// Warp w < 8 serves token rows 32 (w % 4) .. +31 of
 // the tile (TMEM lanes of its quarter) and column half w / 4 of each mixing
 // tile and of the output.
 // TMEM columns: Gram products at 128 q (forward products of s-tiles 0..i,
@@ -381,7 +406,7 @@ __device__ __forceinline__ void setup_dir(const T* dt, int hs, int n, float A2, 
 // the forward direction and its first token for the reverse one); only the
 // 32 x 32 blocks on the diagonal take one exp per element.
 template <int N, bool NOISY>
-__global__ void __launch_bounds__(kScanThreads, 1) k_ssd_block_scan(const SsdScanParams p,
+__global__ void __launch_bounds__(kScanCta<NOISY>, 1) k_ssd_block_scan(const SsdScanParams p,
                                                                     const __grid_constant__ CUtensorMap xmap) {
   pdl_sync();
   extern __shared__ unsigned char smraw[];
@@ -420,15 +445,20 @@ __global__ void __launch_bounds__(kScanThreads, 1) k_ssd_block_scan(const SsdSca
     seed_src = p.seed + b * p.seed_bstride + (int64_t)(p.seed_shift ? k - 1 : k) * H * kSsdP * N;
   }
   const bool has_seed = seed_src != nullptr;
+  constexpr bool NINTH = kHasNinth<NOISY>;
+  const bool worker = !NINTH || t < kScanThreads;
+  const bool issuer = t == (NINTH ? kScanThreads : kScanIssuer);
   // --- Gram products C B^T of this tile against the block's s-tiles
-  stage_rows<N>(sm + L.cf, p.Cf, tok, i * kSsdT);
-  for (int j = 0; j < nf; ++j) stage_rows<N>(sm + L.r + j * 128u * N * 2u, p.Bf, tok, j * kSsdT);
-  if (NOISY) {
-    stage_rows<N>(sm + L.m1, p.Cr, tok, i * kSsdT);
-    for (int j = i; j < m; ++j)
-      stage_rows<N>(sm + L.r + (nf + j - i) * 128u * N * 2u, p.Br, tok, j * kSsdT);
+  if (worker) {
+    stage_rows<N>(sm + L.cf, p.Cf, tok, i * kSsdT);
+    for (int j = 0; j < nf; ++j) stage_rows<N>(sm + L.r + j * 128u * N * 2u, p.Bf, tok, j * kSsdT);
+    if (NOISY) {
+      stage_rows<N>(sm + L.m1, p.Cr, tok, i * kSsdT);
+      for (int j = i; j < m; ++j)
+        stage_rows<N>(sm + L.r + (nf + j - i) * 128u * N * 2u, p.Br, tok, j * kSsdT);
+    }
+    cp_async_commit();
   }
-  cp_async_commit();
   float* s_prm = reinterpret_cast<float*>(sm + L.prm);  // [4][16]: A_f, D_f, A_r, D_r of the CTA's heads
   if (t < hg) {
     s_prm[t] = p.Af[h0 + t];
@@ -438,11 +468,12 @@ __global__ void __launch_bounds__(kScanThreads, 1) k_ssd_block_scan(const SsdSca
       s_prm[48 + t] = p.Dr[h0 + t];
     }
   }
-  {  // dt of the CTA's heads, bf16 as stored (Bs hg <= 256 * 16): every load issued before the stores
+  if (worker) {  // dt of the CTA's heads, bf16 as stored (Bs hg <= 256 * 16): every load issued before the stores
     __nv_bfloat16 vf[kMaxHeadsPerCta], vr[kMaxHeadsPerCta];
     const int ne = Bs * hg;
 #pragma unroll
     for (int q = 0; q < kMaxHeadsPerCta; ++q) {
+      if (q * kScanThreads >= ne) break;
       const int e = t + q * kScanThreads, s = e / hg, hh = e - s * hg;
       if (e < ne) {
         vf[q] = p.dtf[tok(s) * H + h0 + hh];
@@ -451,6 +482,7 @@ __global__ void __launch_bounds__(kScanThreads, 1) k_ssd_block_scan(const SsdSca
     }
 #pragma unroll
     for (int q = 0; q < kMaxHeadsPerCta; ++q) {
+      if (q * kScanThreads >= ne) break;
       const int e = t + q * kScanThreads;
       if (e < ne) {
         s_dtf[e] = vf[q];
@@ -471,7 +503,7 @@ __global__ void __launch_bounds__(kScanThreads, 1) k_ssd_block_scan(const SsdSca
   umma::fence_after_sync();
   const uint32_t tm = tslot;
   const uint32_t lane_base = tm + ((uint32_t)(32 * q4) << 16);
-  if (t == 0) {
+  if (issuer) {
     const uint32_t base = umma::smem_u32(sm);
     for (int qq = 0; qq < nf + nr; ++qq)
       mma_gram<N>(tm + 128u * qq, base + (qq < nf ? L.cf : L.m1), base + L.r + qq * 128u * N * 2u);
@@ -479,7 +511,7 @@ __global__ void __launch_bounds__(kScanThreads, 1) k_ssd_block_scan(const SsdSca
   }
   bool alive = cta_wait(&bar[1], 0, p.flag);
   umma::fence_after_sync();
-  // one head's x tiles and raw seed into buffer xbuf: by TMA (thread 0; a
+  // one head's x tiles and raw seed into buffer xbuf: by TMA (the issuing thread; a
   // 128-token x tile is one box of the [tokens][heads][64] map, the seed one
   // contiguous run) when the launcher set up the map, else by cp.async
   bool ld_pending = false;  // a TMA phase issued and not yet waited for
@@ -489,30 +521,32 @@ __global__ void __launch_bounds__(kScanThreads, 1) k_ssd_block_scan(const SsdSca
     if (p.tma) {
       ld_pending = true;
       ld_parity = (uint32_t)((hd - h0) & 1);
-      if (t == 0) {
+      if (issuer) {
         umma::fence_async_smem();  // the buffers' earlier generic accesses before the async writes
         bar_expect_tx(&bar[2], (uint32_t)ntile * 16384u + (seed_h != nullptr ? (uint32_t)(kSsdP * N * 4) : 0u));
         const int row0 = (int)(b * g.L + (int64_t)k * Bs);
         for (int j = 0; j < ntile; ++j) tma_load_3d(sm + xbuf + (uint32_t)j * 16384u, &xmap, 0, hd, row0 + 128 * j, &bar[2]);
         if (seed_h != nullptr) bulk_load(sm + L.raw, seed_h, (uint32_t)(kSsdP * N * 4), &bar[2]);
       }
-    } else {
+    } else if (worker) {
       issue_head_loads<N>(sm, L, p.x, tok, H, hd, ntile, seed_h, xbuf);
     }
   };
   // the first head's x and seed (the B tiles are no longer read)
   if (alive && h0 < h1) load_head(h0, L.x);
-  // decay vectors of head hh into buffer `buf`: warp 0 the forward direction,
-  // warp 1 the reverse one (each scans, then fills its column factors;
-  // forward referenced to the column group's last token, reverse to its first)
+  // decay vectors of head hh into buffer `buf`: one warp the forward direction,
+  // one the reverse one (each scans, then fills its column factors;
+  // forward referenced to the column group's last token, reverse to its
+  // first). In clean scans warp 5 has nothing to build in a diagonal tile.
+  constexpr int kSetupF = NOISY ? 0 : 5, kSetupR = 1;
   auto setup = [&](int hh, int buf) {
     float* v = vec0 + buf * 1536;
-    if (w == 0)
+    if (w == kSetupF)
       setup_dir<false>(s_dtf + hh, hg, Bs, __fmul_rn(s_prm[hh], kLog2e), v, v + 256, v + 512);
-    else if (NOISY && w == 1)
+    else if (NOISY && w == kSetupR)
       setup_dir<true>(s_dtr + hh, hg, Bs, __fmul_rn(s_prm[32 + hh], kLog2e), v + 768, v + 1024, v + 1280);
   };
-  if (alive && h0 < h1) setup(0, 0);
+  if (alive && h0 < h1 && worker) setup(0, 0);
   // mixing tile j of head hh into shared buffer mt: this warp's two 32-column
   // groups (0: no term, 1: factored decay, 2: diagonal block; uniform per warp)
   auto build = [&](int j, const float* v, unsigned char* mt) {
@@ -596,23 +630,24 @@ __global__ void __launch_bounds__(kScanThreads, 1) k_ssd_block_scan(const SsdSca
       }
     }
   };
-  // MMAs of mixing tile j (and, first, the seed term) by thread 0
-  auto issue = [&](int j, uint32_t xcur, bool seed_term) {
-    umma::fence_after_sync();
+  // the seed term's MMAs, C^f . seed^T into columns 448..511, and those of
+  // mixing tile j, by the issuing thread
+  auto issue_seed = [&]() {
     const uint32_t base = umma::smem_u32(sm);
-    if (seed_term) {  // C^f . seed^T into columns 448..511
-      constexpr uint32_t id = umma::idesc_bf16(128, 64, false, false);
-      const uint64_t dc = umma::sdesc(base + L.cf, 16, 1024), dh = umma::sdesc(base + L.seed, 16, 1024),
-                     dl = umma::sdesc(base + L.seed + 128u * N, 16, 1024);
+    constexpr uint32_t id = umma::idesc_bf16(128, 64, false, false);
+    const uint64_t dc = umma::sdesc(base + L.cf, 16, 1024), dh = umma::sdesc(base + L.seed, 16, 1024),
+                   dl = umma::sdesc(base + L.seed + 128u * N, 16, 1024);
 #pragma unroll
-      for (int kk = 0; kk < N / 16; ++kk) {
-        const uint32_t offc = (kk >> 2) * kTile16 + (kk & 3) * 32u;
-        const uint32_t offs = (kk >> 2) * 8192u + (kk & 3) * 32u;
-        const uint64_t a = umma::sdesc_adv(dc, offc);
-        umma::mma_bf16(tm + 448, a, umma::sdesc_adv(dh, offs), id, kk > 0);
-        umma::mma_bf16(tm + 448, a, umma::sdesc_adv(dl, offs), id, true);
-      }
+    for (int kk = 0; kk < N / 16; ++kk) {
+      const uint32_t offc = (kk >> 2) * kTile16 + (kk & 3) * 32u;
+      const uint32_t offs = (kk >> 2) * 8192u + (kk & 3) * 32u;
+      const uint64_t a = umma::sdesc_adv(dc, offc);
+      umma::mma_bf16(tm + 448, a, umma::sdesc_adv(dh, offs), id, kk > 0);
+      umma::mma_bf16(tm + 448, a, umma::sdesc_adv(dl, offs), id, true);
     }
+  };
+  auto issue = [&](int j, uint32_t xcur) {
+    const uint32_t base = umma::smem_u32(sm);
     const uint64_t dm = umma::sdesc(base + (j ? L.m1 : L.m0), 16, 1024),
                    dx = umma::sdesc(base + xcur + (uint32_t)j * 16384u, 1024, 1024);
     constexpr uint32_t id = umma::idesc_bf16(128, 64, false, true);
@@ -635,7 +670,7 @@ __global__ void __launch_bounds__(kScanThreads, 1) k_ssd_block_scan(const SsdSca
       cp_async_wait_all();
     }
     __syncthreads();  // the head's x and raw seed have landed, its decay vectors are ready
-    if (has_seed) {   // seed (fp32, staged in m1) -> bf16 high + low parts, K-major
+    if (has_seed && worker) {  // seed (fp32, staged in m1) -> bf16 high + low parts, K-major
       for (int c = t; c < kSsdP * N / 8; c += kScanThreads) {
         const int pr = c / (N / 8), ch = c % (N / 8);
         const float4 u0 = *reinterpret_cast<const float4*>(sm + L.raw + (pr * N + ch * 8) * 4);
@@ -653,29 +688,62 @@ __global__ void __launch_bounds__(kScanThreads, 1) k_ssd_block_scan(const SsdSca
         *reinterpret_cast<uint4*>(sm + L.seed + 128u * N + off) = make_uint4(wl[0], wl[1], wl[2], wl[3]);
       }
     }
-    build(0, v, sm + L.m0);
-    umma::fence_async_smem();
-    umma::fence_before_sync();
-    __syncthreads();
-    // The issuing thread is held while the tensor pipe takes the MMAs, so it
-    // is thread 128: warp 4 (rows 0..31, right column half) has the least
-    // mixing work on a diagonal tile (nothing for a clean block's, one term
-    // per column group for a noisy block's)
-    if (t == kScanIssuer) {
-      issue(0, xcur, has_seed);
-      if (ntile == 1) umma::mma_commit(&bar[0]);
-    }
-    if (ntile > 1) {  // the second tile is built while the first one's MMAs run
-      build(1, v, sm + L.m1);
+    if constexpr (NINTH) {
+      umma::fence_async_smem();
+      umma::fence_before_sync();
+      __syncthreads();  // the seed's parts are in shared memory, its raw copy (in m1) is no longer read
+      if (worker) {
+        build(0, v, sm + L.m0);
+        umma::fence_async_smem();
+        umma::fence_before_sync();
+        tile_arrive(0);
+        if (ntile > 1) {  // the second tile is built while the first one's MMAs run
+          build(1, v, sm + L.m1);
+          umma::fence_async_smem();
+          umma::fence_before_sync();
+          tile_arrive(1);
+        }
+        if (hh + 1 < hg) setup(hh + 1, (hh + 1) & 1);  // under this head's MMAs
+      } else {
+        if (issuer && has_seed) {
+          umma::fence_after_sync();
+          issue_seed();
+        }
+        __syncwarp();
+        for (int j = 0; j < ntile; ++j) {
+          tile_wait(j);
+          if (issuer) {
+            umma::fence_after_sync();
+            issue(j, xcur);
+            if (j == ntile - 1) umma::mma_commit(&bar[0]);
+          }
+          __syncwarp();
+        }
+      }
+    } else {
+      build(0, v, sm + L.m0);
       umma::fence_async_smem();
       umma::fence_before_sync();
       __syncthreads();
-      if (t == kScanIssuer) {
-        issue(1, xcur, false);
-        umma::mma_commit(&bar[0]);
+      if (issuer) {
+        umma::fence_after_sync();
+        if (has_seed) issue_seed();
+        issue(0, xcur);
+        if (ntile == 1) umma::mma_commit(&bar[0]);
       }
+      if (ntile > 1) {  // the second tile is built while the first one's MMAs run
+        build(1, v, sm + L.m1);
+        umma::fence_async_smem();
+        umma::fence_before_sync();
+        __syncthreads();
+        if (issuer) {
+          umma::fence_after_sync();
+          issue(1, xcur);
+          umma::mma_commit(&bar[0]);
+        }
+      }
+      if (hh + 1 < hg) setup(hh + 1, (hh + 1) & 1);  // under this head's MMAs
     }
-    if (hh + 1 < hg) setup(hh + 1, (hh + 1) & 1);  // under this head's MMAs
     if (!cta_wait(&bar[0], hh & 1, p.flag)) {
       alive = false;
       break;
@@ -685,7 +753,7 @@ __global__ void __launch_bounds__(kScanThreads, 1) k_ssd_block_scan(const SsdSca
     if (hh + 1 < hg) load_head(h + 1, L.x + ((hh + 1) & 1) * L.xsz);
     // --- epilogue: y = mixing term + decayed seed term + D x, bf16 out;
     // this warp's 32 channels of its token row
-    {
+    if (worker) {
       float ya[32], yo[32];
       if (has_seed)
         umma::tmem_ld32x2(lane_base + 384u + 32u * hf, ya, lane_base + 448u + 32u * hf, yo);
@@ -872,7 +940,7 @@ cudaError_t scan_t(const SsdScanParams& p_in, cudaStream_t s) {
   // streams read right to left keep the cp.async path (a box cannot reverse rows)
   p.tma = !p.rev && encode_head_map(&xmap, p.x, p.g.Bt * p.g.L, p.g.H) ? 1 : 0;
   const dim3 grid((unsigned)tiles, (unsigned)((p.g.H + p.hg - 1) / p.hg));
-  launch_pdl(k_ssd_block_scan<N, NOISY>, grid, kScanThreads, L.total, s, p, xmap);
+  launch_pdl(k_ssd_block_scan<N, NOISY>, grid, kScanCta<NOISY>, L.total, s, p, xmap);
   return cudaGetLastError();
 }
 
