@@ -88,18 +88,23 @@ __global__ void __launch_bounds__(kStateThreads, 1) k_ssd_block_state(const SsdS
   const RowMap tok(b, g.L, (int64_t)k * Bs, p.rev != 0);
   float* s_w = reinterpret_cast<float*>(sm + S.w);  // [hg][256]
   // B rows: chunk c of 8 state indices of token s goes to half c / 8
-  for (int c = t; c < Bs * N / 8; c += kStateThreads) {
-    const int s = c / (N / 8), ch = c % (N / 8);
-    cp_async16(sm + S.b + (ch >> 3) * half + sw128(s, ch & 7), p.B + tok(s) * N + ch * 8, 16);
+  {
+    constexpr int CPR = N / 8, RPP = kStateThreads / CPR;
+    const int s = t / CPR, ch = t % CPR;
+    unsigned char* d = sm + S.b + (ch >> 3) * half + sw128(s, ch & 7);
+    const __nv_bfloat16* src = p.B + tok(s) * N + ch * 8;
+    for (int r = s; r < Bs; r += RPP, d += RPP * 128, src += tok.step * (RPP * N)) cp_async16(d, src, 16);
   }
   if (N == 64)
     for (int c = t; c < Bs * 8; c += kStateThreads)
       *reinterpret_cast<uint4*>(sm + S.b + half + c * 16) = make_uint4(0, 0, 0, 0);
   auto load_x = [&](int h, int buf) {
-    for (int c = t; c < Bs * 8; c += kStateThreads) {
-      const int s = c >> 3, ch = c & 7;
-      cp_async16(sm + S.xr + buf * half + sw128(s, ch), p.x + (tok(s) * H + h) * kSsdP + ch * 8, 16);
-    }
+    constexpr int RPP = kStateThreads / 8;
+    const int s = t >> 3, ch = t & 7;
+    unsigned char* d = sm + S.xr + buf * half + sw128(s, ch);
+    const __nv_bfloat16* src = p.x + (tok(s) * H + h) * kSsdP + ch * 8;
+    const int64_t step = tok.step * ((int64_t)RPP * H * kSsdP);
+    for (int r = s; r < Bs; r += RPP, d += RPP * 128, src += step) cp_async16(d, src, 16);
     cp_async_commit();
   };
   if (h0 < h1) load_x(h0, 0);
@@ -245,6 +250,63 @@ __global__ void __launch_bounds__(256) k_ssd_state_pass(const SsdPassParams p) {
   if (!p.emit_all) p.states[b * per_b + r] = S;
   if (p.final_state != nullptr) p.final_state[b * per_b + r] = S;
   dfinite(kSiteSsdStatePass, S, idx);  // debug build: a non-finite cached state
+}
+
+// The recurrence over blocks is one fused multiply-add per block and state
+// element: the kernel is bound by the bytes it keeps in flight. A CTA of 64
+// threads owns 64 consecutive elements of one head, one per thread, and
+// streams the block states through a ring of kPassStages cp.async groups of
+// kPassRows blocks. For chains above kPassLong blocks (65,536 tokens, 26 heads x
+// 128, 256 blocks: 72 us, k_ssd_state_pass 96); shorter ones end before its
+// extra CTAs pay (21 blocks of 14 heads x 64: 359 us a step, 365 with the
+// ring), unless there are very many (32 blocks, 1.7 M elements: 75 and 69 us,
+// of 4920). In place: a block's state is
+// read into the ring before the same element is written.
+constexpr int kPassW = 64, kPassRows = 8, kPassStages = 4, kPassLong = 64;
+__global__ void __launch_bounds__(kPassW) k_ssd_state_pass_ring(const SsdPassParams p) {
+  pdl_sync();
+  __shared__ __align__(16) float tbuf[kPassStages][kPassRows][kPassW];
+  const SsdGeo& g = p.g;
+  const int64_t per_b = (int64_t)g.H * kSsdP * g.N;
+  const int64_t e0 = (int64_t)blockIdx.x * kPassW, b = e0 / per_b, r0 = e0 - b * per_b, r = r0 + threadIdx.x;
+  const int h = (int)(r0 / ((int64_t)kSsdP * g.N));
+  // debug build: the last block-state slot the CTA reads
+  if (!dguard(kSiteSsdStatePass, (b * g.nb + g.nb - 1) * per_b + r0 + kPassW - 1, g.Bt * g.nb * per_b)) return;
+  const float A2 = __fmul_rn(p.A[h], kLog2e);
+  float S = p.init != nullptr ? p.init[b * per_b + r] : 0.f;
+  const float* T = p.T + b * g.nb * per_b + r0;
+  const float* sd = p.sumdt + b * g.nb * g.H + h;
+  const int nst = (g.nb + kPassRows - 1) / kPassRows;
+  auto issue = [&](int st) {
+    if (st < nst) {
+      const int k0 = st * kPassRows, slot = st % kPassStages;
+#pragma unroll
+      for (int q = threadIdx.x; q < kPassRows * (kPassW / 4); q += kPassW) {
+        const int k = q / (kPassW / 4), j = (q % (kPassW / 4)) * 4;
+        if (k0 + k < g.nb) cp_async16(&tbuf[slot][k][j], T + (int64_t)(k0 + k) * per_b + j, 16);
+      }
+    }
+    cp_async_commit();
+  };
+  for (int st = 0; st < kPassStages - 1; ++st) issue(st);
+  for (int st = 0; st < nst; ++st) {
+    const int k0 = st * kPassRows, slot = st % kPassStages;
+    float dv[kPassRows];
+#pragma unroll
+    for (int u = 0; u < kPassRows; ++u) dv[u] = sd[(int64_t)min(k0 + u, g.nb - 1) * g.H];
+    asm volatile("cp.async.wait_group %0;\n" ::"n"(kPassStages - 2) : "memory");
+    __syncthreads();  // stage st has arrived, and stage st - 1 is no longer read
+    issue(st + kPassStages - 1);
+#pragma unroll
+    for (int u = 0; u < kPassRows; ++u) {
+      if (k0 + u >= g.nb) break;
+      S = __fmaf_rn(ex2(__fmul_rn(A2, dv[u])), S, tbuf[slot][u][threadIdx.x]);
+      if (p.emit_all) p.states[(b * g.nb + k0 + u) * per_b + r] = S;
+    }
+  }
+  if (!p.emit_all) p.states[b * per_b + r] = S;
+  if (p.final_state != nullptr) p.final_state[b * per_b + r] = S;
+  dfinite(kSiteSsdStatePass, S, b * per_b + r);  // debug build: a non-finite cached state
 }
 
 // Copies one 128-token tile of a [tokens][N] bf16 tensor into K-major
@@ -885,7 +947,10 @@ cudaError_t launch_ssd_block_state(const SsdStateParams& p, cudaStream_t s) {
 cudaError_t launch_ssd_state_pass(const SsdPassParams& p, cudaStream_t s) {
   const int64_t n = p.g.Bt * p.g.H * kSsdP * p.g.N;
   if (n == 0) return cudaSuccess;
-  launch_pdl(k_ssd_state_pass, (unsigned)((n + 255) / 256), 256, 0, s, p);
+  if (p.g.nb > kPassLong)
+    launch_pdl(k_ssd_state_pass_ring, (unsigned)(n / kPassW), kPassW, 0, s, p);  // 64 N elements per head
+  else
+    launch_pdl(k_ssd_state_pass, (unsigned)((n + 255) / 256), 256, 0, s, p);
   return cudaGetLastError();
 }
 

@@ -49,3 +49,31 @@ def test_ssd_head_groups_match_oracle(Bt, nb, Bs, H, N):
                               wl.t32["dstates"].astype("float64"))
     for k in NAMES:
         P.assert_close("d" + k, to_numpy(g[k]), ref[k], P.GRAD_TOL, 0.0 if k in f32 else P.BF16_U)
+
+
+@pytest.mark.parametrize("nb,Bt,H,N", [(64, 1, 1, 64), (65, 2, 2, 64), (70, 1, 3, 128), (97, 1, 1, 64)])
+def test_ssd_long_state_pass_matches_oracle(nb, Bt, H, N):
+    """The state recurrence on both sides of the length where it streams its
+    blocks through a ring (64), with part of a ring stage left over; states and
+    outputs against the oracle, the final-state build bit for bit."""
+    from oracle import ssd as oracle_ssd
+    P.oracle_threads()
+    L = nb * 128
+    wl = SsdWorkload(Bt, L, 128, H, N, seed=nb, with_init=True)
+    t = {k: to_device(wl.dev_bits(k) if k != "init_state" else wl.t32[k],
+                      binding.BDSCAN_F32 if k in ("A_f", "A_r", "D_f", "D_r", "init_state") else binding.BDSCAN_BF16,
+                      "cuda") for k in wl.t32}
+    dims = binding.make_ssd_dims(Bt, L, 128, H, N)
+    every = torch.full((Bt, nb, H, 64, N), float("nan"), device="cuda")
+    last = torch.full((Bt, 1, H, 64, N), float("nan"), device="cuda")
+    y = torch.empty_like(t["x_c"])
+    for emit, st, out in ((1, every, y), (0, last, None)):
+        ws = torch.empty(binding.bdscan_ssd_boundary_states_workspace_size(dims, emit), dtype=torch.uint8, device="cuda")
+        binding.ssd_boundary_states(dims, t, t["init_state"], out, st, emit, ws)
+    torch.cuda.synchronize()
+    assert binding.bdscan_ssd_wait_flag(1) == 0
+    assert torch.equal(last[:, 0], every[:, -1])
+    ref = oracle_ssd.boundary_states(128, *[wl.f64(k) for k in ("x_c", "dt_c", "B_c", "C_c", "A_f", "D_f")],
+                                     init_state=wl.t32["init_state"].astype("float64"), emit_all=True, want_y=True)
+    P.assert_close("states", to_numpy(every), ref[0], P.FWD_TOL)
+    P.assert_close("y_c", to_numpy(y), ref[1], P.FWD_TOL, P.BF16_U)
