@@ -99,16 +99,59 @@ __global__ void __launch_bounds__(kCta) k_chunk_local(const FwdParams p) {
   }
 }
 
+// The carry over a few chunks: one thread per (batch row, channel, state).
+template <int N>
+__global__ void __launch_bounds__(256) k_chunk_carry(const FwdParams p) {
+  pdl_sync();
+  const Geo& g = p.g;
+  const int64_t idx = (int64_t)blockIdx.x * 256 + threadIdx.x;
+  if (idx >= g.Bt * g.D * N) return;
+  const int n = (int)(idx % N);
+  const int64_t d = (idx / N) % g.D, b = idx / ((int64_t)N * g.D);
+  // debug build: the last state slot this thread writes (no barrier follows)
+  if (!dguard(kSiteChunkCarry, ((b * (g.nc + 1) + g.nc_full) * g.D + d) * N + n, g.Bt * (g.nc + 1) * g.D * N)) return;
+  const float A2 = __fmul_rn(p.Af[d * N + n], kLog2e);
+  float H = p.init ? p.init[(b * g.D + d) * N + n] : 0.f;
+  const int64_t hstride = g.D * N;
+  float* hs = p.hst + b * (g.nc + 1) * hstride + d * N + n;
+  const float* sd = p.sdt + b * g.nc * g.D + d;
+  constexpr int U = 8;
+  int c = 0;
+  for (; c + U <= g.nc_full; c += U) {
+    float hl[U], s[U];
+#pragma unroll
+    for (int j = 0; j < U; ++j) {
+      hl[j] = hs[(int64_t)(c + j) * hstride];
+      s[j] = sd[(int64_t)(c + j) * g.D];
+    }
+#pragma unroll
+    for (int j = 0; j < U; ++j) {
+      hs[(int64_t)(c + j) * hstride] = H;
+      H = __fmaf_rn(ex2(__fmul_rn(A2, s[j])), H, hl[j]);
+    }
+  }
+  for (; c < g.nc_full; ++c) {
+    const float hl = hs[(int64_t)c * hstride], s = sd[(int64_t)c * g.D];
+    hs[(int64_t)c * hstride] = H;
+    H = __fmaf_rn(ex2(__fmul_rn(A2, s)), H, hl);
+  }
+  hs[(int64_t)g.nc_full * hstride] = H;
+  dfinite(kSiteChunkCarry, H, idx);  // debug build: a non-finite cached state
+}
+
 // The carry over chunks is one fused multiply-add per chunk and state, so the
 // kernel is bound by how many bytes it keeps in flight. A CTA of 64 threads
 // owns 64 consecutive (channel, state) elements of one batch row, one per
 // thread, and streams the chunk rows (256 bytes of local end states plus the
 // sums of dt) through a ring of kCarryStages cp.async groups of kCarryRows
-// rows: 12 KB ahead of the chain per CTA. With one load per thread and chunk,
-// eight in flight, 2048 chunks x 32768 elements took 291 us (1.8 TB/s).
-constexpr int kCarryW = 64, kCarryRows = 16, kCarryStages = 4;
+// rows: 12 KB ahead of the chain per CTA: 2048 chunks x 32768 elements 102 us,
+// 291 (1.8 TB/s) in k_chunk_carry, which has eight loads per thread in flight.
+// Up to kCarryFew chunks that one is taken: with few rounds of loads the ring's
+// fill is not made up for (16 chunks x 196608 elements: 7.8 us, 10.0 through
+// the ring; 32 x 16384: 7.7 us either way).
+constexpr int kCarryW = 64, kCarryRows = 16, kCarryStages = 4, kCarryFew = 32;
 template <int N>
-__global__ void __launch_bounds__(kCarryW) k_chunk_carry(const FwdParams p) {
+__global__ void __launch_bounds__(kCarryW) k_chunk_carry_ring(const FwdParams p) {
   pdl_sync();
   constexpr int CH = kCarryW / N;        // channels of the CTA's elements
   constexpr int HQ = kCarryW / 4, SQ = CH / 4;  // 16-byte pieces of one row of states, of dt sums
@@ -641,8 +684,12 @@ cudaError_t launch_chunk_local(int dt, int N, const FwdParams& p, cudaStream_t s
 
 cudaError_t launch_chunk_carry(int N, const FwdParams& p, cudaStream_t s) {
   if (p.g.Bt * p.g.D * N == 0) return cudaSuccess;
+  if (p.g.nc_full <= kCarryFew) {
+    const unsigned blocks = (unsigned)((p.g.Bt * p.g.D * N + 255) / 256);
+    BDS_DISPATCH_N(N, launch_pdl(k_chunk_carry<NN>, blocks, 256, 0, s, p); return cudaGetLastError();)
+  }
   const dim3 grid((unsigned)((p.g.D * N + kCarryW - 1) / kCarryW), (unsigned)p.g.Bt);
-  BDS_DISPATCH_N(N, launch_pdl(k_chunk_carry<NN>, grid, kCarryW, 0, s, p); return cudaGetLastError();)
+  BDS_DISPATCH_N(N, launch_pdl(k_chunk_carry_ring<NN>, grid, kCarryW, 0, s, p); return cudaGetLastError();)
 }
 
 cudaError_t launch_block_scan(int dt, int N, int mode, int nchunks, const FwdParams& p, cudaStream_t s) {

@@ -26,6 +26,9 @@ from paper_2607_02805_gb300.layer import to_device, to_numpy  # noqa: E402
     (2, 16, 0, 32, 20, 16, "f32"),    # exactly one stage
     (1, 49, 3, 16, 24, 16, "bf16"),   # one row more than the stages in flight
     (1, 80, 0, 64, 36, 8, "f32"),     # the ring wraps
+    (1, 32, 1, 16, 24, 16, "bf16"),   # the last count without the ring
+    (2, 33, 0, 32, 20, 16, "f32"),    # the first with it, one row past two stages
+    (2, 47, 1, 16, 12, 8, "f32"),     # the ring with the second CTA half empty
     (3, 0, 2, 16, 8, 16, "bf16"),     # no full chunk
 ])
 def test_chunk_carry_matches_oracle(Bt, chunks, tail, Bs, D, N, dt):
