@@ -19,32 +19,26 @@
 namespace bds {
 
 // ---------------------------------------------------------------------------
-// Launches. Every kernel of the library starts with pdl_sync(). Launched with
-// launch_pdl(), a small grid's CTAs may be placed while the kernel before it on
-// the stream drains; they wait there until that kernel has completed and its
-// writes are visible, before they read or write anything. Since every kernel
-// waits in all of its CTAs, a kernel's completion implies its predecessors'.
-// (Nine launches of the 256 x 32 training step: 85 -> 72 us; 15 of the
-// 3 x 2688 x 14 SSD step: 512 -> 502 us.) A grid above two CTAs per SM, and any
-// grid behind one above eight, is launched after the kernel before it: placed
-// early, its CTAs pile up on the SMs that drain first (every grid early: the
-// 8 x 8192 x 26 SSD step 5307 -> 5526 us; the chunk carry behind 32768 CTAs of
-// the chunk scan: 1361 -> 1401 us). The size of the thread's last launch only
-// guesses at the predecessor; the order on the stream never depends on it.
+// Launches. Every kernel of the library starts with pdl_sync() and is launched
+// with launch_pdl(): its CTAs are placed once every CTA of the kernel before it
+// on the stream has ended, and wait there until that kernel's writes are
+// visible, before they read or write anything. What is saved is the time from
+// the end of one grid to the start of the next. Since every kernel waits in all
+// of its CTAs, a kernel's completion implies its predecessors'. Without it and
+// with it: the 2 x 512 x 256 x 16 training step 102 and 83 us, 1 x 8192 x 256 x
+// 4 heads of SSD training 256 and 224, the 16384 x 512 clean prefill 43 and 37;
+// with it for grids up to 304 CTAs only and for all: the 8 x 2048 x 1536
+// training step 1477 and 1453, the same step's mixer 2537 and 2476.
+//
+// No kernel releases its successor earlier (griddepcontrol.launch_dependents at
+// its start): CTAs placed while the predecessor runs pile up on the SMs with
+// room instead of spreading over the idle ones. The 8192 x 512 clean prefill
+// took 100 us so, with small grids alone placed early; 59 without overlap and
+// 52 as here.
 // ---------------------------------------------------------------------------
-__device__ __forceinline__ void pdl_sync() {
-  asm volatile("griddepcontrol.launch_dependents;\n" ::: "memory");
-  asm volatile("griddepcontrol.wait;\n" ::: "memory");
-}
-constexpr uint64_t kPdlMaxCtas = 304, kPdlMaxBefore = 1216;
-inline uint64_t& last_launch_ctas() {
-  static thread_local uint64_t n = 0;
-  return n;
-}
+__device__ __forceinline__ void pdl_sync() { asm volatile("griddepcontrol.wait;\n" ::: "memory"); }
 template <typename... K, typename... A>
 inline cudaError_t launch_pdl(void (*kernel)(K...), dim3 grid, dim3 block, size_t smem, cudaStream_t s, A... args) {
-  const uint64_t ctas = (uint64_t)grid.x * grid.y * grid.z, before = last_launch_ctas();
-  last_launch_ctas() = ctas;
   cudaLaunchAttribute attr;
   attr.id = cudaLaunchAttributeProgrammaticStreamSerialization;
   attr.val.programmaticStreamSerializationAllowed = 1;
@@ -54,7 +48,7 @@ inline cudaError_t launch_pdl(void (*kernel)(K...), dim3 grid, dim3 block, size_
   cfg.dynamicSmemBytes = smem;
   cfg.stream = s;
   cfg.attrs = &attr;
-  cfg.numAttrs = ctas <= kPdlMaxCtas && before <= kPdlMaxBefore ? 1 : 0;
+  cfg.numAttrs = 1;
   return cudaLaunchKernelEx(&cfg, kernel, static_cast<K>(args)...);
 }
 
