@@ -38,17 +38,29 @@ constexpr int kScanSeg = 16;
 // REV: the scan runs right to left in time (logical token t is row L-1-t).
 // Bound by the exponentials (one ex2 per token, channel and state) together
 // with the packed FP32 operations around them: 262,144 x 2048 x 16 takes
-// 1245 us, of which the ex2 alone need 853. The staged spans have a
+// 1182 us, of which the ex2 alone need 853. The staged spans have a
 // compile-time stride, so a token's addresses are immediates (1273 us with a
 // run-time stride and half the unroll).
-template <typename T, int N, bool REV>
+// A thread scans NS of the N states of its channel: N / NS CTAs share a channel
+// group, and each stages the group's tokens for itself. All of them in one
+// thread is the least work. With few CTAs the chunk's serial walk is what takes
+// the time, and it is shorter over fewer states: four of them up to one CTA per
+// SM, eight up to two (128 tokens per chunk, N = 16; 16 / 8 / 4 states each:
+// 4 CTAs 20.4 / 17.2 / 13.2 us, 128 CTAs 21.5 / 19.4 / 17.6, 304 CTAs
+// 23.9 / 22.8 / 26.9, 608 CTAs 32.4 / 38.2 / 45.2; N = 8, 8 / 4 states: 15.0 /
+// 14.0, 15.1 / 14.8, 17.3 / 17.2, 21.5 / 25.6). Each state is the same sequence
+// of operations either way.
+constexpr int kLocalQuarter = 152, kLocalHalf = 304;
+template <typename T, int N, int NS, bool REV>
 __global__ void __launch_bounds__(kCta) k_chunk_local(const FwdParams p) {
   pdl_sync();
   extern __shared__ __align__(16) unsigned char smem[];
   const Geo& g = p.g;
   const int64_t b = blockIdx.z;
   const int c = blockIdx.y;
-  const int64_t d0 = (int64_t)blockIdx.x * kCta, d = d0 + threadIdx.x;
+  constexpr int Q = N / NS;
+  const int n0 = (int)(blockIdx.x % Q) * NS;
+  const int64_t d0 = (int64_t)(blockIdx.x / Q) * kCta, d = d0 + threadIdx.x;
   const bool act = d < g.D;
   {  // debug build: the chunk's tokens, channels and state slot lie inside the sizes
     const int64_t tc = (int64_t)g.m * g.Bs, dl = (d0 + kCta < g.D ? d0 + kCta : g.D) - 1;
@@ -64,13 +76,13 @@ __global__ void __launch_bounds__(kCta) k_chunk_local(const FwdParams p) {
   st.td_src[1] = (const T*)p.dtc;
   st.row_src[0] = (const T*)p.Bc;
 
-  float2 A2[N / 2], h[N / 2];
-  vzero2<N>(A2);
-  vzero2<N>(h);
+  float2 A2[NS / 2], h[NS / 2];
+  vzero2<NS>(A2);
+  vzero2<NS>(h);
   if (act) {
-    vload2<N>(A2, p.Af + d * N, 0);
+    vload2<NS>(A2, p.Af + d * N + n0, 0);
 #pragma unroll
-    for (int j = 0; j < N / 2; ++j) A2[j] = mul2(A2[j], f2(kLog2e));
+    for (int j = 0; j < NS / 2; ++j) A2[j] = mul2(A2[j], f2(kLog2e));
   }
   float sdt = 0.f;
   const int64_t tc = (int64_t)g.m * g.Bs;
@@ -89,13 +101,13 @@ __global__ void __launch_bounds__(kCta) k_chunk_local(const FwdParams p) {
 #pragma unroll 8
     for (int i = 0; i < ns; ++i) {
       const float dt = st.at(1, i);
-      scan_state<N>(h, A2, dt, st.at(0, i), st.row(0, i));
+      scan_state<NS>(h, A2, dt, st.at(0, i), st.row(0, i) + n0);
       sdt = __fadd_rn(sdt, dt);
     }
   }
   if (act) {
-    vstore2<N>(p.hst + ((b * (g.nc + 1) + c) * g.D + d) * N, h, 0);
-    p.sdt[(b * g.nc + c) * g.D + d] = sdt;
+    vstore2<NS>(p.hst + ((b * (g.nc + 1) + c) * g.D + d) * N + n0, h, 0);
+    if (n0 == 0) p.sdt[(b * g.nc + c) * g.D + d] = sdt;
   }
 }
 
@@ -605,15 +617,22 @@ __global__ void __launch_bounds__(256) k_combine(const float* yf, const float* y
 // ---------------------------------------------------------------------------
 namespace {
 
-template <typename T, int N, bool REV>
-cudaError_t chunk_local_rt(const FwdParams& p, cudaStream_t s) {
+template <typename T, int N, int NS, bool REV>
+cudaError_t chunk_local_k(const FwdParams& p, cudaStream_t s) {
   const size_t smem = Stage<T, N, 2, 1, 2>::bytes(kLocalSpan);
   cudaError_t e =
-      cudaFuncSetAttribute(k_chunk_local<T, N, REV>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
+      cudaFuncSetAttribute(k_chunk_local<T, N, NS, REV>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
   if (e != cudaSuccess) return e;
-  dim3 grid((unsigned)p.g.G, (unsigned)p.g.nc_full, (unsigned)p.g.Bt);
-  launch_pdl(k_chunk_local<T, N, REV>, grid, kCta, smem, s, p);
+  dim3 grid((unsigned)(p.g.G * (N / NS)), (unsigned)p.g.nc_full, (unsigned)p.g.Bt);
+  launch_pdl(k_chunk_local<T, N, NS, REV>, grid, kCta, smem, s, p);
   return cudaGetLastError();
+}
+template <typename T, int N, bool REV>
+cudaError_t chunk_local_rt(const FwdParams& p, cudaStream_t s) {
+  const int64_t ctas = (int64_t)p.g.G * p.g.nc_full * p.g.Bt;
+  if (ctas <= kLocalQuarter) return chunk_local_k<T, N, 4, REV>(p, s);
+  if (N == 16 && ctas <= kLocalHalf) return chunk_local_k<T, N, 8, REV>(p, s);
+  return chunk_local_k<T, N, N, REV>(p, s);
 }
 template <typename T, int N>
 cudaError_t chunk_local_t(const FwdParams& p, cudaStream_t s) {
