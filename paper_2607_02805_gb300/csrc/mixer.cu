@@ -711,7 +711,7 @@ cudaError_t prep(const Geo& g, const MixIn<T>& a, float* x_c, float* dt_c, float
   cudaError_t e = set_smem_cached((const void*)k_mix_prep<T>, (int)prep_smem<T>(), -1);
   if (e != cudaSuccess) return e;
   launch_pdl(k_mix_prep<T>, dim3(runs(Ls), tiles, (unsigned)g.Bt), dim3(tx, ty), prep_smem<T>(), s, a, x_c, dt_c, x_n, dt_f,
-                                                                                           dt_r, Ls);
+             dt_r, Ls);
   return api_launched(cudaGetLastError(), s);
 }
 
@@ -784,12 +784,12 @@ cudaError_t mix_backward_t(const Geo& g, int N, const bdscan_clean* cl, const vo
   if (e != cudaSuccess) return e;
   const int64_t n = g.Bt * g.L * g.D, nn = g.Bt * g.L * N;
   float* dy[2] = {(float*)(ws + w.dy[0]), (float*)(ws + w.dy[1])};
-  launch_pdl(k_mix_gate_bwd<T, TO>, vec_blocks<T>(n), 256, 0, s, n, (const float*)(ws + w.y[0]), (const T*)z_c, (const T*)dout_c,
-                                                     dy[0], (TO*)dz_c);
+  launch_pdl(k_mix_gate_bwd<T, TO>, vec_blocks<T>(n), 256, 0, s, n, (const float*)(ws + w.y[0]), (const T*)z_c,
+             (const T*)dout_c, dy[0], (TO*)dz_c);
   e = api_launched(cudaGetLastError(), s);
   if (e != cudaSuccess) return e;
-  launch_pdl(k_mix_gate_bwd<T, TO>, vec_blocks<T>(n), 256, 0, s, n, (const float*)(ws + w.y[1]), (const T*)z_n, (const T*)dout_n,
-                                                     dy[1], (TO*)dz_n);
+  launch_pdl(k_mix_gate_bwd<T, TO>, vec_blocks<T>(n), 256, 0, s, n, (const float*)(ws + w.y[1]), (const T*)z_n,
+             (const T*)dout_n, dy[1], (TO*)dz_n);
   e = api_launched(cudaGetLastError(), s);
   if (e != cudaSuccess) return e;
   float* G[5];
@@ -842,9 +842,9 @@ cudaError_t mix_backward_t(const Geo& g, int N, const bdscan_clean* cl, const vo
   const int64_t want = ctas(Ls);
   const int slices = (int)(want < kParSplit ? want : kParSplit);
   if ((e = set_smem_cached((const void*)k_mix_bwd<T, TO>, (int)mix_bwd_smem<T>(), -1)) != cudaSuccess) return e;
-  launch_pdl(k_mix_bwd<T, TO>, dim3((unsigned)slices, (unsigned)tiles), dim3(32, kBwdGroups), mix_bwd_smem<T>(), s, 
-      a, G[0], G[1], G[2], G[3], G[4], (TO*)gc->dx, (TO*)gc->ddt, (TO*)gn->dx, (TO*)gn->ddt_f, (TO*)gn->ddt_r, Ls,
-      (int)((g.L + Ls - 1) / Ls), part);
+  launch_pdl(k_mix_bwd<T, TO>, dim3((unsigned)slices, (unsigned)tiles), dim3(32, kBwdGroups), mix_bwd_smem<T>(), s,
+             a, G[0], G[1], G[2], G[3], G[4], (TO*)gc->dx, (TO*)gc->ddt, (TO*)gn->dx, (TO*)gn->ddt_f, (TO*)gn->ddt_r, Ls,
+             (int)((g.L + Ls - 1) / Ls), part);
   e = api_launched(cudaGetLastError(), s);
   if (e != cudaSuccess) return e;
   CvtSet cv;
@@ -854,8 +854,8 @@ cudaError_t mix_backward_t(const Geo& g, int N, const bdscan_clean* cl, const vo
     cv.dst[i] = gbc_out[i];
   }
   if ((e = cvt_all<float, TO>(cv, 6, nn, s)) != cudaSuccess) return e;
-  launch_pdl(k_mix_par_red, blocks_of(g.D * (kW + 3)), 256, 0, s, g.D, slices, part, gm->dconv_w, gm->dconv_b, gm->ddt_bias_f,
-                                                          gm->ddt_bias_r);
+  launch_pdl(k_mix_par_red, blocks_of(g.D * (kW + 3)), 256, 0, s, g.D, slices, part, gm->dconv_w, gm->dconv_b,
+             gm->ddt_bias_f, gm->ddt_bias_r);
   return api_launched(cudaGetLastError(), s);
 }
 

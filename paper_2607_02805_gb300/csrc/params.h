@@ -63,7 +63,7 @@ struct BwdParams {
   float* part_tok;  // [6][Bt][L][G][N] per channel-group sums of dB_c, dC_c, dB_f, dC_f, dB_r, dC_r
   float* part_A;    // [3][Bt*nc][D][N] dA partial sums: noisy fwd, noisy rev, clean
   float* part_D;    // [2][Bt*nc][D]    dD partial sums: noisy, clean
-  int stage_bufs;    // set per launch: staging buffers of one-segment blocks
+  int stage_bufs;    // set per launch: staging buffers (fp32 instances; bf16 ones have two)
   // noisy kernel with a CTA per part of a block (split_parts below): fp32
   // partials of dx_n, [2][Bt][L][D] (reverse, forward direction), joined by
   // the token reduction; null otherwise

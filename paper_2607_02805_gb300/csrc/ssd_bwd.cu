@@ -1268,8 +1268,8 @@ cudaError_t launch_ssd_bwd_dbc(const SsdGeo& g, int ngrp, int ngrp_state, const 
                                __nv_bfloat16* dBr, __nv_bfloat16* dCr, cudaStream_t s) {
   const int64_t n = g.Bt * g.L * (g.N / 4);
   if (n == 0) return cudaSuccess;
-  launch_pdl(k_ssd_bwd_dbc, (unsigned)((n + 255) / 256), 256, 0, s, g, ngrp, ngrp_state, dBp_c, dBs, dCp_c, dBp_f, dCp_f, dBp_r, dCp_r, dBc,
-                                                              dCc, dBf, dCf, dBr, dCr);
+  launch_pdl(k_ssd_bwd_dbc, (unsigned)((n + 255) / 256), 256, 0, s, g, ngrp, ngrp_state, dBp_c, dBs,
+             dCp_c, dBp_f, dCp_f, dBp_r, dCp_r, dBc, dCc, dBf, dCf, dBr, dCr);
   return cudaGetLastError();
 }
 
