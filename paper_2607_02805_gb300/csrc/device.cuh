@@ -30,12 +30,15 @@ namespace bds {
 // with it for grids up to 304 CTAs only and for all: the 8 x 2048 x 1536
 // training step 1477 and 1453, the same step's mixer 2537 and 2476.
 //
-// No kernel releases its successor earlier (griddepcontrol.launch_dependents at
-// its start): CTAs placed while the predecessor runs pile up on the SMs with
-// room instead of spreading over the idle ones. The 8192 x 512 clean prefill
-// took 100 us so, with small grids alone placed early; 59 without overlap and
-// 52 as here.
+// Kernels do not release their successor earlier (pdl_release() at the start):
+// CTAs placed while the predecessor runs pile up on the SMs with room instead
+// of spreading over the idle ones. The 8192 x 512 clean prefill took 100 us so,
+// with small grids alone placed early; 59 without overlap and 52 as here. The
+// exception is the SSD active block: its CTAs take most of an SM each, so in the
+// loop of denoising steps the next step's go to the idle SMs (16 steps of 26
+// heads: 167 -> 163 us).
 // ---------------------------------------------------------------------------
+__device__ __forceinline__ void pdl_release() { asm volatile("griddepcontrol.launch_dependents;\n" ::: "memory"); }
 __device__ __forceinline__ void pdl_sync() { asm volatile("griddepcontrol.wait;\n" ::: "memory"); }
 template <typename... K, typename... A>
 inline cudaError_t launch_pdl(void (*kernel)(K...), dim3 grid, dim3 block, size_t smem, cudaStream_t s, A... args) {

@@ -470,6 +470,7 @@ __device__ __forceinline__ void setup_dir(const T* dt, int hs, int n, float A2, 
 template <int N, bool NOISY>
 __global__ void __launch_bounds__(kScanCta<NOISY>, 1) k_ssd_block_scan(const SsdScanParams p,
                                                                     const __grid_constant__ CUtensorMap xmap) {
+  if (p.release) pdl_release();
   pdl_sync();
   extern __shared__ unsigned char smraw[];
   unsigned char* sm = align1024(smraw);

@@ -58,6 +58,7 @@ struct SsdScanParams {
   __nv_bfloat16* y;   // [Bt][L][H][P]
   int hg;
   int* flag;
+  int release;        // 1: the next grid on the stream may be placed beside this one
   int rev;            // 1: the stream is read right to left (as in SsdStateParams)
   float* y32;         // non-null: write the output in fp32 here instead of y
   const float* y32_add;  // non-null: add this fp32 array to the output before rounding to y

@@ -302,6 +302,7 @@ int bdscan_ssd_active_block(const bdscan_ssd_dims* dims, const float* seed, cons
   np.seed = seed;
   np.seed_bstride = (int64_t)g.H * 64 * g.N;
   np.seed_shift = 0;
+  np.release = 1;
   const cudaError_t e = bds::api_launched(bds::launch_ssd_block_scan(true, np, s), s);
   if (e != cudaSuccess) return cuda_fail(e, fn);
   return bds::api_ok();
