@@ -413,6 +413,7 @@ struct SsdBwdWs {
 void ssd_bwd_groups(const bds::SsdGeo& g, int64_t units, int maxg, int* hg, int* ngrp) {
   constexpr int64_t kSms = 152;
   *hg = *ngrp = 1;
+  if (g.H <= 0) return;  // zero heads is a valid size: the counts below start at one group
   int64_t best = -1;
   for (int n = (g.H + maxg - 1) / maxg; n <= g.H; ++n) {
     const int per = (g.H + n - 1) / n, groups = (g.H + per - 1) / per;
