@@ -988,36 +988,100 @@ void api_begin() { g_launches = 0; }
 
 cudaError_t api_launched(cudaError_t e, cudaStream_t s) { return launched(e, s); }
 
-// Kernel attributes are set once per (kernel, device, size): repeated calls
-// (an active-block loop) then skip the runtime calls on their host path.
+// What the library knows of a kernel on a device. The attributes belong to the
+// kernel, not to a call: another host thread may be about to launch the same
+// kernel with more shared memory (another block size, another staging plan), so
+// they are looked at and changed under one lock and the shared-memory limit
+// only grows. A kernel that finds no room in the table is asked for each time.
+namespace {
+struct KernelEntry {
+  const void* fn;
+  int dev, regs, limit, carveout;
+  size_t static_smem;
+};
+constexpr unsigned kKernelSlots = 1024;  // a few hundred instances per device at most
+std::mutex g_kernel_mu;
+KernelEntry g_kernels[kKernelSlots];
+
+// The entry of `fn` on the current device `dev` (`spare` where the table is
+// full); g_kernel_mu is held.
+KernelEntry* kernel_entry(const void* fn, int dev, KernelEntry* spare, cudaError_t* err) {
+  *err = cudaSuccess;
+  unsigned at = (unsigned)(((uintptr_t)fn >> 4) + 131u * (unsigned)dev) % kKernelSlots;
+  KernelEntry* e = spare;
+  for (unsigned i = 0; i < kKernelSlots; ++i, at = (at + 1) % kKernelSlots) {
+    if (g_kernels[at].fn == fn && g_kernels[at].dev == dev) return &g_kernels[at];
+    if (g_kernels[at].fn == nullptr) {
+      e = &g_kernels[at];
+      break;
+    }
+  }
+  cudaFuncAttributes fa;
+  if ((*err = cudaFuncGetAttributes(&fa, fn)) != cudaSuccess) return spare;
+  *e = KernelEntry{fn, dev, fa.numRegs, fa.maxDynamicSharedSizeBytes, -1, fa.sharedSizeBytes};
+  return e;
+}
+}  // namespace
+
+// Lets the kernel be launched with `bytes` of dynamic shared memory. Repeated
+// calls (an active-block loop) skip the runtime calls on their host path.
 cudaError_t set_smem_cached(const void* fn, int bytes, int carveout) {
   int dev = 0;
-  cudaError_t e = cudaGetDevice(&dev);
-  if (e != cudaSuccess) return e;
-  struct Entry {
-    const void* fn;
-    int dev, bytes, carveout;
-  };
-  static std::mutex mu;
-  static Entry tab[256];
-  static int n = 0;
-  {
-    std::lock_guard<std::mutex> lk(mu);
-    for (int i = 0; i < n; ++i)
-      if (tab[i].fn == fn && tab[i].dev == dev && tab[i].bytes >= bytes && tab[i].carveout == carveout)
-        return cudaSuccess;
+  cudaError_t err = cudaGetDevice(&dev);
+  if (err != cudaSuccess) return err;
+  std::lock_guard<std::mutex> lk(g_kernel_mu);
+  KernelEntry spare;
+  KernelEntry* e = kernel_entry(fn, dev, &spare, &err);
+  if (err != cudaSuccess) return err;
+  if (bytes > e->limit) {
+    if ((err = cudaFuncSetAttribute(fn, cudaFuncAttributeMaxDynamicSharedMemorySize, bytes)) != cudaSuccess) return err;
+    e->limit = bytes;
   }
-  if ((e = cudaFuncSetAttribute(fn, cudaFuncAttributeMaxDynamicSharedMemorySize, bytes)) != cudaSuccess) return e;
-  if (carveout >= 0 && (e = cudaFuncSetAttribute(fn, cudaFuncAttributePreferredSharedMemoryCarveout, carveout)) !=
-                           cudaSuccess)
-    return e;
+  if (carveout >= 0 && carveout != e->carveout) {
+    err = cudaFuncSetAttribute(fn, cudaFuncAttributePreferredSharedMemoryCarveout, carveout);
+    if (err != cudaSuccess) return err;
+    e->carveout = carveout;
+  }
+  return cudaSuccess;
+}
+
+// Registers per thread and static shared memory of a kernel on device `dev`,
+// the current one. Sets nothing.
+cudaError_t kernel_use(const void* fn, int dev, int* regs, size_t* static_smem) {
+  cudaError_t err;
+  std::lock_guard<std::mutex> lk(g_kernel_mu);
+  KernelEntry spare;
+  const KernelEntry* e = kernel_entry(fn, dev, &spare, &err);
+  if (err != cudaSuccess) return err;
+  *regs = e->regs;
+  *static_smem = e->static_smem;
+  return cudaSuccess;
+}
+
+// Per-SM limits of a device, looked up once per device.
+cudaError_t sm_limits(int dev, SmLimits* out) {
+  static std::mutex mu;
+  static SmLimits tab[256];
   std::lock_guard<std::mutex> lk(mu);
-  for (int i = 0; i < n; ++i)
-    if (tab[i].fn == fn && tab[i].dev == dev && tab[i].carveout == carveout) {
-      if (bytes > tab[i].bytes) tab[i].bytes = bytes;
-      return cudaSuccess;
-    }
-  if (n < 256) tab[n++] = Entry{fn, dev, bytes, carveout};
+  const bool keep = dev >= 0 && dev < 256;
+  if (keep && tab[dev].threads > 0) {
+    *out = tab[dev];
+    return cudaSuccess;
+  }
+  SmLimits l;
+  const struct {
+    int* to;
+    cudaDeviceAttr attr;
+  } q[] = {{&l.smem, cudaDevAttrMaxSharedMemoryPerMultiprocessor},
+           {&l.regs, cudaDevAttrMaxRegistersPerMultiprocessor},
+           {&l.threads, cudaDevAttrMaxThreadsPerMultiProcessor},
+           {&l.reserve, cudaDevAttrReservedSharedMemoryPerBlock}};
+  for (const auto& a : q) {
+    const cudaError_t e = cudaDeviceGetAttribute(a.to, a.attr, dev);
+    if (e != cudaSuccess) return e;
+  }
+  if (keep) tab[dev] = l;
+  *out = l;
   return cudaSuccess;
 }
 

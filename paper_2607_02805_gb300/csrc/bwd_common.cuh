@@ -325,15 +325,12 @@ inline size_t pad_for_tmem(size_t smem, uint32_t cols) {
   return smem > need ? smem : need;
 }
 
-// Both attributes are set before every launch and before the occupancy query:
-// the padded shared memory exceeds the 48 KB default, and without the largest
-// carveout the driver may configure an SM for one such CTA instead of the two
-// its TMEM can hold.
+// Both attributes are set before a launch: the padded shared memory exceeds the
+// 48 KB default, and without the largest carveout the driver may configure an
+// SM for one such CTA instead of the two its TMEM can hold.
 template <typename K>
 cudaError_t set_bwd_attrs(K kernel, size_t smem) {
-  cudaError_t e = cudaFuncSetAttribute(kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
-  if (e != cudaSuccess) return e;
-  return cudaFuncSetAttribute(kernel, cudaFuncAttributePreferredSharedMemoryCarveout, (int)cudaSharedmemCarveoutMaxShared);
+  return set_smem_cached((const void*)kernel, (int)smem, (int)cudaSharedmemCarveoutMaxShared);
 }
 
 // Resident CTAs per SM of a backward kernel (0 on failure), from the per-SM
@@ -341,24 +338,22 @@ cudaError_t set_bwd_attrs(K kernel, size_t smem) {
 // whole warps, registers allocated per thread in multiples of 8), shared
 // memory with the per-CTA reserve, and threads. The runtime's occupancy
 // calculator reports one CTA for the noisy kernel where the hardware admits
-// two, so it is not used.
+// two, so it is not used. A query: the plans that are compared by it leave the
+// kernel's attributes as they are.
 template <typename K>
 int resident_ctas(K kernel, size_t smem, uint32_t tcols, int dev) {
-  cudaFuncAttributes fa;
-  int sm_smem = 0, sm_regs = 0, sm_threads = 0, reserve = 0;
-  if (set_bwd_attrs(kernel, smem) != cudaSuccess || cudaFuncGetAttributes(&fa, kernel) != cudaSuccess ||
-      cudaDeviceGetAttribute(&sm_smem, cudaDevAttrMaxSharedMemoryPerMultiprocessor, dev) != cudaSuccess ||
-      cudaDeviceGetAttribute(&sm_regs, cudaDevAttrMaxRegistersPerMultiprocessor, dev) != cudaSuccess ||
-      cudaDeviceGetAttribute(&sm_threads, cudaDevAttrMaxThreadsPerMultiProcessor, dev) != cudaSuccess ||
-      cudaDeviceGetAttribute(&reserve, cudaDevAttrReservedSharedMemoryPerBlock, dev) != cudaSuccess) {
+  SmLimits l;
+  int regs = 0;
+  size_t static_smem = 0;
+  if (kernel_use((const void*)kernel, dev, &regs, &static_smem) != cudaSuccess || sm_limits(dev, &l) != cudaSuccess) {
     cudaGetLastError();
     return 0;
   }
   const int by_tmem = (int)(512 / tcols);
-  const int warp_regs = ((fa.numRegs + 7) / 8 * 8) * 32;
-  const int by_regs = warp_regs > 0 ? (sm_regs / 4 / warp_regs) * 4 / kWarps : 0;
-  const int by_smem = (int)((size_t)sm_smem / (smem + fa.sharedSizeBytes + (size_t)reserve));
-  const int by_threads = sm_threads / kCta;
+  const int warp_regs = ((regs + 7) / 8 * 8) * 32;
+  const int by_regs = warp_regs > 0 ? (l.regs / 4 / warp_regs) * 4 / kWarps : 0;
+  const int by_smem = (int)((size_t)l.smem / (smem + static_smem + (size_t)l.reserve));
+  const int by_threads = l.threads / kCta;
   int n = by_tmem;
   n = by_regs < n ? by_regs : n;
   n = by_smem < n ? by_smem : n;

@@ -118,6 +118,11 @@ int api_ok();
 void api_begin();
 cudaError_t api_launched(cudaError_t e, cudaStream_t s);
 cudaError_t set_smem_cached(const void* fn, int bytes, int carveout);  // carveout < 0: leave it
+cudaError_t kernel_use(const void* fn, int dev, int* regs, size_t* static_smem);
+struct SmLimits {
+  int smem, regs, threads, reserve;  // per SM, and the shared memory reserved per CTA
+};
+cudaError_t sm_limits(int dev, SmLimits* out);
 int sm_count_cached();  // 0 if unknown
 int api_check_forward_dims(const void* dims, Geo* g, int* dt, int* N, const char* fn);
 // The block scans of the all-block forward, after the chunk carry.
