@@ -620,8 +620,7 @@ namespace {
 template <typename T, int N, int NS, bool REV>
 cudaError_t chunk_local_k(const FwdParams& p, cudaStream_t s) {
   const size_t smem = Stage<T, N, 2, 1, 2>::bytes(kLocalSpan);
-  cudaError_t e =
-      cudaFuncSetAttribute(k_chunk_local<T, N, NS, REV>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
+  cudaError_t e = set_smem_cached((const void*)k_chunk_local<T, N, NS, REV>, (int)smem, -1);
   if (e != cudaSuccess) return e;
   dim3 grid((unsigned)(p.g.G * (N / NS)), (unsigned)p.g.nc_full, (unsigned)p.g.Bt);
   launch_pdl(k_chunk_local<T, N, NS, REV>, grid, kCta, smem, s, p);
@@ -644,8 +643,7 @@ cudaError_t block_scan_k(int nchunks, const FwdParams& p, cudaStream_t s) {
   using Ly = ScanLayout<MODE>;
   const size_t buf = Stage<T, N, Ly::NTD, Ly::NROW, 2>::buf_bytes(kScanSeg);
   const size_t smem = Ly::kNoisy ? buf + (size_t)p.g.Bs * kCta * sizeof(float) : 2 * buf;
-  cudaError_t e = cudaFuncSetAttribute(k_block_scan<T, TO, N, MODE, KIND>,
-                                       cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
+  cudaError_t e = set_smem_cached((const void*)k_block_scan<T, TO, N, MODE, KIND>, (int)smem, -1);
   if (e != cudaSuccess) return e;
   dim3 grid((unsigned)p.g.G, (unsigned)nchunks, (unsigned)p.g.Bt);
   launch_pdl(k_block_scan<T, TO, N, MODE, KIND>, grid, kCta, smem, s, p);
@@ -675,8 +673,7 @@ cudaError_t active_block_t(const FwdParams& p, cudaStream_t s) {
   using Ly = ActiveLayout<T, N>;
   const size_t smem = ADA ? Ly::bytes_ada((int)p.g.Bs) : Ly::bytes((int)p.g.Bs);
   if (smem > 48 * 1024) {
-    cudaError_t e =
-        cudaFuncSetAttribute(k_active_block<T, TO, N, ADA>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
+    cudaError_t e = set_smem_cached((const void*)k_active_block<T, TO, N, ADA>, (int)smem, -1);
     if (e != cudaSuccess) return e;
   }
   dim3 grid((unsigned)((p.g.D + kActW - 1) / kActW * p.g.nb), (unsigned)p.g.Bt);

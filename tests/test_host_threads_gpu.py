@@ -21,6 +21,18 @@ from paper_2607_02805_gb300 import binding  # noqa: E402
 from paper_2607_02805_gb300.layer import Layer  # noqa: E402
 
 
+def _train(Bt, L, Bs, D, N, dt, seed):
+    """A training step and its outputs."""
+    lay = Layer(Workload(Bt, L, Bs, D, N, dtype=dt, seed=seed))
+    lay.alloc_backward()
+
+    def step(stream):
+        lay.forward(stream)
+        lay.backward(stream, use_dstates=False)
+
+    return step, [lay.y_c, lay.y_n, lay.states] + list(lay.g.values())
+
+
 def _backward(Bt, L, Bs, D, N, dt, seed):
     """The backward alone, with its arguments made once: the threads then spend
     their time inside the library, where the interpreter's lock is released."""
@@ -41,6 +53,18 @@ def _backward(Bt, L, Bs, D, N, dt, seed):
 
     step.keep = structs
     return step, list(g.values())
+
+
+def _forward(Bt, L, Bs, D, N, dt, seed):
+    lay = Layer(Workload(Bt, L, Bs, D, N, dtype=dt, seed=seed, with_grads=False))
+    return lay.forward, [lay.y_c, lay.y_n, lay.states]
+
+
+def _active(Bt, Bs, D, N, dt, seed):
+    wl = Workload(Bt, Bs, Bs, D, N, dtype=dt, seed=seed, with_grads=False, parts=("noisy",))
+    lay = Layer(wl)
+    state = torch.linspace(-1, 1, Bt * D * N, device="cuda").reshape(Bt, D, N).contiguous()
+    return (lambda stream: binding.active_block(lay.dims, state, lay.t, lay.y_n, stream)), [lay.y_n]
 
 
 def _in_threads(jobs, calls):
@@ -82,3 +106,17 @@ def test_backwards_of_equal_sizes(L, Bs, D, N, dt):
     """fp32 calls choose between two staging plans with different amounts of
     shared memory; looking at the other plan may not show."""
     _in_threads([_backward(1, L, Bs, D, N, dt, seed) for seed in (1, 2, 3, 4)], 10000)
+
+
+def test_training_steps_of_block_sizes_that_share_an_instance():
+    _in_threads([_train(1, L, Bs, 64, 16, "f32", 4) for L, Bs in ((256, 32), (256, 64), (384, 128))], 1000)
+
+
+def test_forwards_of_block_sizes_that_share_an_instance():
+    sms = torch.cuda.get_device_properties(0).multi_processor_count
+    rows = 2 * sms  # the fused scan of both streams
+    _in_threads([_forward(rows, Bs, Bs, 64, 16, "bf16", 5) for Bs in (32, 64, 128)], 1500)
+
+
+def test_active_blocks_of_sizes_that_share_an_instance():
+    _in_threads([_active(1, Bs, 64, 16, "f32", 6) for Bs in (96, 160, 256)], 4000)
