@@ -1,8 +1,8 @@
 // noalloc.cu -- cache build (bdscan_boundary_states) for callers that may not
 // allocate device memory: the scratch of the chunked clean scan lives in a
 // static device array of this file instead of a caller workspace. The
-// kernels and their launch order are those of bdscan_boundary_states, so
-// the results are the same bits.
+// launches are those of bdscan_boundary_states, so the results are the same
+// bits.
 #include <cstdio>
 #include <cstring>
 #include <mutex>
@@ -109,26 +109,6 @@ extern "C" int bdscan_boundary_states_noalloc(const bdscan_dims* dims, const bds
   p.init = init_state;
   p.hst = (float*)scratch;
   p.sdt = (float*)((char*)scratch + al256((size_t)g.Bt * (g.nc + 1) * g.D * N * 4));
-  // every launch is counted (and timed by the profiling hook) as in
-  // bdscan_boundary_states
-  if (g.nc_full > 0) e = bds::api_launched(bds::launch_chunk_local(dt, N, p, s), s);
-  if (e == cudaSuccess) e = bds::api_launched(bds::launch_chunk_carry(N, p, s), s);
-  if (e == cudaSuccess) {
-    if (emit_all || y_c != nullptr) {
-      p.emit_all = emit_all ? 1 : 0;
-      p.states = emit_all ? states : nullptr;
-      p.final_state = emit_all ? nullptr : states;
-      e = bds::api_launched(bds::launch_block_scan(dt, N, 1, g.nc, p, s), s);
-    } else if (g.nc_full == g.nc) {
-      const size_t row = (size_t)g.D * N * 4;
-      e = cudaMemcpy2DAsync(states, row, p.hst + (size_t)g.nc * g.D * N, (size_t)(g.nc + 1) * row, row,
-                            (size_t)g.Bt, cudaMemcpyDeviceToDevice, s);
-    } else {
-      p.emit_all = 0;
-      p.final_state = states;
-      p.c_begin = g.nc - 1;
-      e = bds::api_launched(bds::launch_block_scan(dt, N, 1, 1, p, s), s);
-    }
-  }
+  e = bds::api_run_boundary(dt, N, p, states, emit_all, s);
   return e == cudaSuccess ? bds::api_ok() : cuda_error(e);
 }
