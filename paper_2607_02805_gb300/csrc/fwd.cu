@@ -472,8 +472,9 @@ __global__ void __launch_bounds__(2 * kActW, 1) k_active_block(const FwdParams p
   const int lane = threadIdx.x & 31, dir = threadIdx.x >> 5;  // dir 0: forward, 1: reverse
   const int64_t d = d0 + lane;
   const bool act = d < g.D;
-  // debug build: the batch row and the channel group lie inside the sizes
-  if (!(dguard(kSiteActiveBlock, b, g.Bt) && dguard(kSiteActiveBlock, d0, g.D))) return;
+  // debug build: the batch row, its block and the channel group lie inside the sizes
+  if (!(dguard(kSiteActiveBlock, b, g.Bt) && dguard(kSiteActiveBlock, k, g.nb) && dguard(kSiteActiveBlock, d0, g.D)))
+    return;
   T* td = reinterpret_cast<T*>(smem);
   float* rows = reinterpret_cast<float*>(smem + Ly::td_bytes(Bs) + Ly::raw_bytes(Bs));
   T* raw = is_f32<T>::value ? reinterpret_cast<T*>(rows) : reinterpret_cast<T*>(smem + Ly::td_bytes(Bs));
