@@ -44,8 +44,8 @@ constexpr int kScanSeg = 16;
 // A thread scans NS of the N states of its channel: N / NS CTAs share a channel
 // group, and each stages the group's tokens for itself. All of them in one
 // thread is the least work. With few CTAs the chunk's serial walk is what takes
-// the time, and it is shorter over fewer states: four of them up to one CTA per
-// SM, eight up to two (128 tokens per chunk, N = 16; 16 / 8 / 4 states each:
+// the time, and it is shorter over fewer states: four of them up to one CTA on
+// each of the part's 152 SMs, eight up to two (128 tokens per chunk, N = 16; 16 / 8 / 4 states each:
 // 4 CTAs 20.4 / 17.2 / 13.2 us, 128 CTAs 21.5 / 19.4 / 17.6, 304 CTAs
 // 23.9 / 22.8 / 26.9, 608 CTAs 32.4 / 38.2 / 45.2; N = 8, 8 / 4 states: 15.0 /
 // 14.0, 15.1 / 14.8, 17.3 / 17.2, 21.5 / 25.6). Each state is the same sequence

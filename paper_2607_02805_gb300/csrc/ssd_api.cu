@@ -409,7 +409,14 @@ struct SsdBwdWs {
 // keep fewer groups, whose partials the combine reads. A function of the
 // dimensions only, so the workspace size does not depend on the device.
 // 63 tiles of 14 heads: two groups in one wave instead of fourteen in six
-// (tile kernels 93 + 89 + 71 -> 66 + 63 + 40 us, combine 57 -> 16 us).
+// (tile kernels 93 + 89 + 71 -> 66 + 63 + 40 us, combine 57 -> 16 us); 512 tiles
+// of 26 heads: two groups. At a wave or two the model is off: it takes all tiles
+// for equal, but the second tile of a block reaches twice the s-tiles of the
+// first. At 128 tiles of 26 heads it picks two groups of 13 (the SMs are busy
+// 69 % of a seeded launch); the three tile launches and the combine take 919 +
+// 35 us so, 838 + 46 with three groups, 803 + 56 with four and 836 + 88 with
+// seven. At 128 tiles of 14 heads (N 64): 481 + 16 with its two groups, 457 +
+// 29, 439 + 35 and 495 + 51 with three, four and seven.
 void ssd_bwd_groups(const bds::SsdGeo& g, int64_t units, int maxg, int* hg, int* ngrp) {
   constexpr int64_t kSms = 152;
   *hg = *ngrp = 1;
